@@ -149,12 +149,10 @@ int he_ctx_set_multsum_variant(he_ctx *ctx, int variant);
 /* Pins the context's NTT passes (N = 2^14 .. 2^16) to one variant, without
  * tuning (-1 returns to the tuner, which times them at the next transform).
  * Variants compute identical words; this is for tests and measurement.
- * 2, 3, 5: one 8-stage tile per CTA, 2, 3 or 4 CTAs per SM (forward and
- * inverse); 4: forward passes on persistent CTAs whose tiles arrive through
- * bulk asynchronous copies (a producer warp, two buffers), inverse as 3;
- * 6 (N = 2^16; otherwise as 3): the forward transform of a limb in one pass
- * by a cluster of 8 CTAs exchanging through distributed shared memory (one
- * read and one write of every word), inverse as 3.
+ * 2, 3, 5: one 8-stage tile per CTA, compiled for 2, 3 or 4 CTAs per SM
+ * (forward and inverse); 4 and 6 are accepted and run as 3 (a persistent
+ * form fed by bulk copies and a one-pass form on 8-CTA clusters were slower
+ * at every size: 0.965 and 0.983 ms for 1024 rows of N = 2^16 against 0.619).
  * Errors: HE_ERR_ARG for other values. */
 int he_ctx_set_ntt_variant(he_ctx *ctx, int variant);
 

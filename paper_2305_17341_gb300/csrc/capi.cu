@@ -184,6 +184,7 @@ int he_ctx_create(const he_params *prm, uint64_t seed, he_ctx **out) {
     c.primes = q;
     c.primes.insert(c.primes.end(), p.begin(), p.end());
     cudaGetDevice(&c.device);
+    cudaDeviceGetAttribute(&c.nsm, cudaDevAttrMultiProcessorCount, c.device);
     if (cudaStreamCreateWithFlags(&c.stream, cudaStreamNonBlocking) != cudaSuccess) {
         delete h;
         return fail(HE_ERR_CUDA, "stream creation failed");
@@ -224,7 +225,7 @@ int he_ctx_destroy(he_ctx *ctx) {
     for (auto &kv : c.ptcache) cudaFree(kv.second);
     for (auto &kv : c.dcd)
         for (auto &f : kv.second.factors) cudaFree(f.dev);
-    void *ptrs[] = {c.d_mod, c.d_psi, c.d_psip, c.d_ipsi, c.d_ipsip, c.d_psi2, c.d_ipsi2, c.d_ninv, c.d_dn_pinv,
+    void *ptrs[] = {c.d_mod, c.d_modf, c.d_ninvf, c.d_dn_Pinvf, c.d_psi, c.d_psip, c.d_ipsi, c.d_ipsip, c.d_psi2, c.d_ipsi2, c.d_ninv, c.d_dn_pinv,
                     c.d_dn_pmod,
                     c.d_dn_Pinv, c.d_Pmod, c.d_dn_E, c.d_zeta, c.d_slot_t, c.d_sk, c.d_skM,
                     c.d_pkM};
@@ -234,6 +235,7 @@ int he_ctx_destroy(he_ctx *ctx) {
         if (l.d_up_inv) cudaFree(l.d_up_inv);
         if (l.d_up_mod) cudaFree(l.d_up_mod);
         if (l.d_rs_inv) cudaFree(l.d_rs_inv);
+        if (l.d_rs_invf) cudaFree(l.d_rs_invf);
         if (l.d_rs_qlmod) cudaFree(l.d_rs_qlmod);
     }
     c.pool.release_all();
@@ -279,13 +281,13 @@ int he_ctx_set_ntt_variant(he_ctx *ctx, int variant) {
     if (variant != -1 && (variant < 2 || variant > 6)) return fail(HE_ERR_ARG, "NTT variant -1 or 2..6");
     Ctx &c = ctx->c;
     cudaStreamSynchronize(c.stream);
+    c.ntt_pinned = variant >= 0;
     if (variant < 0) {
         c.ntt_tuned = false;   // the tuner picks again at the next transform
         c.ntt_minb = c.ntt_minb_inv = 2;
     } else {
         c.ntt_tuned = true;
-        c.ntt_minb = variant == 6 && c.logN != 16 ? 3 : variant;   // the cluster pass is for N = 2^16
-        c.ntt_minb_inv = variant == 4 || variant == 6 ? 3 : variant;   // forward-only variants
+        c.ntt_minb = c.ntt_minb_inv = variant == 4 || variant == 6 ? 3 : variant;   // 4 and 6 run as 3
     }
     return HE_OK;
 }

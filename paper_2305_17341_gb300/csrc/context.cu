@@ -127,6 +127,28 @@ static int bitrev(int x, int bits) {
     return r;
 }
 
+ModF h_modf(u64 q) {
+    ModF m = {};
+    // the range whose error bounds fq_mul derives
+    m.on = q >= (1ull << 36) && q < (3ull << 39);
+    if (!m.on) return m;
+    m.nQ = (u64)0 - (q << 22);
+    m.cst = kFqBits * (q << 22);
+    const u64 n = (u64)0 - q;
+    // low word as a signed factor: carry its sign into the high word
+    m.nq = (((n >> 32) + ((n >> 31) & 1)) << 32) | (u32)n;
+    m.qi = (float)(4294967296.0 / (double)q);
+    return m;
+}
+
+ulonglong2 h_fq(u64 w, u64 q) {
+    const i64 c = w > q / 2 ? (i64)(w - q) : (i64)w;
+    const float f = (float)((double)c / (double)q / 256.0);
+    u32 b;
+    std::memcpy(&b, &f, 4);
+    return make_ulonglong2((u64)c, b);
+}
+
 static ModQ make_mod(u64 q) {
     ModQ m;
     m.q = q;
@@ -307,6 +329,9 @@ const LevelConsts &Ctx::lc(int level) {
             rm[i] = ql % primes[i];
         }
         LC.d_rs_inv = upload(ri);
+        std::vector<ulonglong2> rf(level);
+        for (int i = 0; i < level; i++) rf[i] = h_fq(ri[i].w, primes[i]);
+        LC.d_rs_invf = upload(rf);
         LC.d_rs_qlmod = upload(rm);
     }
     return LC;
@@ -341,14 +366,43 @@ void build_tables(Ctx *c) {
     c->d_psip = upload(psip);
     c->d_ipsi = upload(ipsi);
     c->d_ipsip = upload(ipsip);
+    std::vector<ModF> modf(c->nprimes);
+    for (int k = 0; k < c->nprimes; k++) modf[k] = h_modf(c->primes[k]);
+    c->d_modf = upload(modf);
     {
-        std::vector<u64> t2(2 * psi.size()), it2(2 * psi.size());
-        for (size_t i = 0; i < psi.size(); i++) {
-            t2[2 * i] = psi[i], t2[2 * i + 1] = psip[i];
-            it2[2 * i] = ipsi[i], it2[2 * i + 1] = ipsip[i];
+        // the order of PassTw (ntt.cu): 256 column entries, then the N row
+        // entries, per prime
+        const int logM1 = logN / 2, M2 = 1 << (logN - logM1), T = M2 / 16;
+        std::vector<int> src(N + 256, 0);
+        for (int i = 0; i < (1 << logM1) && i < 256; i++) src[i] = i;
+        if (logN >= 14 && logN <= 16)
+            for (int seq = 0; seq < N / M2; seq++) {
+                const int G = N / M2 + seq;
+                int *o = src.data() + 256 + (size_t)seq * M2;
+                for (int s = 8; s >= 1; s >>= 1)
+                    for (int j = 0; j < 8 / s; j++) o[8 / s + j] = (8 / s) * G + j;
+                for (int sp = T / 2; sp >= 1; sp >>= 1)
+                    for (int j = 0; j < 8 / sp; j++)
+                        for (int t = 0; t < T; t++)
+                            o[16 + (8 / sp - 1 - (T == 8 ? 1 : 0) + j) * T + t] = (M2 / (2 * sp)) * G + t * (8 / sp) + j;
+            }
+        const size_t per = (size_t)N + 256;
+        std::vector<ulonglong2> t2(per * c->nprimes), it2(per * c->nprimes), nf(2 * (size_t)c->nprimes);
+        std::vector<ulonglong2> a(N), b(N);
+        for (int k = 0; k < c->nprimes; k++) {
+            const u64 q = c->primes[k];
+            const size_t o = (size_t)k * N;
+            for (int i = 0; i < N; i++) {
+                a[i] = modf[k].on ? h_fq(psi[o + i], q) : make_ulonglong2(psi[o + i], psip[o + i]);
+                b[i] = modf[k].on ? h_fq(ipsi[o + i], q) : make_ulonglong2(ipsi[o + i], ipsip[o + i]);
+            }
+            for (size_t i = 0; i < per; i++) t2[k * per + i] = a[src[i]], it2[k * per + i] = b[src[i]];
+            nf[2 * k] = h_fq(ninv[2 * k], q);
+            nf[2 * k + 1] = h_fq(h_mulmod(ninv[2 * k], ipsi[o + 1], q), q);
         }
         c->d_psi2 = upload(t2);
         c->d_ipsi2 = upload(it2);
+        c->d_ninvf = upload(nf);
     }
     c->d_ninv = upload(ninv);
     c->hmod.resize(c->nprimes);
@@ -380,6 +434,9 @@ void build_tables(Ctx *c) {
     c->d_dn_pinv = upload(pinv);
     c->d_dn_pmod = upload(pmod);
     c->d_dn_Pinv = upload(Pinv);
+    std::vector<ulonglong2> Pinvf(L + 1);
+    for (int r = 0; r <= L; r++) Pinvf[r] = h_fq(Pinv[r].w, c->primes[r]);
+    c->d_dn_Pinvf = upload(Pinvf);
     c->d_Pmod = upload(Pmod);
     // h = (P-1)/2 reduced mod every prime: 2h = P - 1 exactly (P odd)
     MdExact &mk = c->md_exact;

@@ -46,7 +46,7 @@ void moddown(Ctx *c, const u64 *u, int items, int level, u64 *out, long out_s, c
     if (c->logN >= 14 && c->logN <= 16) {
         // the NTT's last pass writes out = (u_Q - conv) P^-1 directly
         SubScale ep;
-        ep.u = u, ep.us = (long)rows * N, ep.out = out, ep.os = out_s, ep.w = c->d_dn_Pinv;
+        ep.u = u, ep.us = (long)rows * N, ep.out = out, ep.os = out_s, ep.w = c->d_dn_Pinv, ep.wf = c->d_dn_Pinvf;
         ep.rows_per_item = level + 1;
         ep.add = add, ep.as = add_s;
         ntt_fwd_subscale(c, conv.p, (long)items * (level + 1), c->map_q(level), c->stream, ep);
@@ -113,7 +113,7 @@ void rescale(Ctx *c, const u64 *in, int B, int level, u64 *out) {
     if (c->logN >= 14 && c->logN <= 16) {
         // the NTT's last pass writes out = (in - t) q_l^-1 directly
         SubScale ep;
-        ep.u = in, ep.us = (long)(level + 1) * N, ep.out = out, ep.os = (long)level * N, ep.w = c->lc(level).d_rs_inv;
+        ep.u = in, ep.us = (long)(level + 1) * N, ep.out = out, ep.os = (long)level * N, ep.w = c->lc(level).d_rs_inv, ep.wf = c->lc(level).d_rs_invf;
         ep.rows_per_item = level;
         ntt_fwd_subscale(c, t.p, 2L * B * level, c->map_q(level - 1), c->stream, ep);
     } else {

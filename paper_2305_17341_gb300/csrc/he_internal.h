@@ -28,6 +28,12 @@ struct RowMap {
         int kk = (int)((k + shift) % n);
         return kk <= lq ? base_q + kk : base_p + (kk - lq - 1);
     }
+    // the same for the rows of one launch (fewer than 2^31), without a 64-bit
+    // division
+    __device__ __forceinline__ int at32(unsigned k) const {
+        const unsigned kk = (k + (unsigned)shift) % (unsigned)n;
+        return (int)kk <= lq ? base_q + (int)kk : base_p + ((int)kk - lq - 1);
+    }
     __host__ __device__ RowMap shifted(long r0) const {
         RowMap m = *this;
         m.shift = (int)((shift + r0) % n);
@@ -43,15 +49,15 @@ struct RowMap {
 // Rows a forward NTT leaves untouched: in Decompose output laid out as
 // [item][digit][rows_per_digit][N], the digit's own rows r in
 // [d alpha, min(d alpha + alpha, nq)) are already in the NTT domain.
-// rows_per_digit == 0 disables the skip; row0 is the absolute index of the
-// launch's first row.
+// rows_per_digit == 0 disables the skip; row0 is the position of the launch's
+// first row in its item (any multiple of rows_per_digit ndig may be dropped).
 struct RowSkip {
     int rows_per_digit = 0, ndig = 0, alpha = 0, nq = 0;
-    long row0 = 0;
-    __host__ __device__ bool skip(long row) const {
+    unsigned row0 = 0;
+    __host__ __device__ bool skip(unsigned row) const {
         if (!rows_per_digit) return false;
-        long a = row0 + row;
-        int r = (int)(a % rows_per_digit), d = (int)((a / rows_per_digit) % ndig), i0 = d * alpha;
+        const unsigned a = row0 + row, dd = a / (unsigned)rows_per_digit;
+        const int r = (int)(a - dd * (unsigned)rows_per_digit), d = (int)(dd % (unsigned)ndig), i0 = d * alpha;
         return r >= i0 && r < i0 + alpha && r < nq;
     }
 };
@@ -119,6 +125,7 @@ struct LevelConsts {
     ShoupPair *d_up_mod = nullptr;   // [ndig][alpha][l+1+alpha]
     // Rescale by q_l: q_l^-1 mod q_i, q_l mod q_i (i < l)
     ShoupPair *d_rs_inv = nullptr;   // [l]
+    ulonglong2 *d_rs_invf = nullptr; // [l] the same for the float-quotient product
     u64 *d_rs_qlmod = nullptr;       // [l]
 };
 
@@ -145,15 +152,24 @@ struct Ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int device = 0;
+    int nsm = 1;             // SMs of the device
 
     ModQ *d_mod = nullptr;         // [nprimes]
+    ModF *d_modf = nullptr;        // [nprimes]
     u64 *d_psi = nullptr, *d_psip = nullptr, *d_ipsi = nullptr, *d_ipsip = nullptr;  // [nprimes][N]
-    u64 *d_psi2 = nullptr, *d_ipsi2 = nullptr;   // [nprimes][N][2]: (w, w') pairs, one 16-byte load each
+    // [nprimes][N + 256] twiddles of the register-blocked NTT in its order of
+    // use, one 16-byte load each: (w, w') Shoup pairs, or (centred w, bits of
+    // wq) where d_modf[k].on
+    ulonglong2 *d_psi2 = nullptr, *d_ipsi2 = nullptr;
     u64 *d_ninv = nullptr;         // [nprimes][2]
+    // [nprimes][2] where d_modf[k].on: N^-1, and N^-1 times the twiddle of the
+    // inverse transform's last stage
+    ulonglong2 *d_ninvf = nullptr;
     // ModDown constants (level independent)
     ShoupPair *d_dn_pinv = nullptr;  // [alpha]   (P/p_j)^-1 mod p_j
     ShoupPair *d_dn_pmod = nullptr;  // [alpha][L+1] (P/p_j) mod q_r
     ShoupPair *d_dn_Pinv = nullptr;  // [L+1]     P^-1 mod q_r
+    ulonglong2 *d_dn_Pinvf = nullptr;  // [L+1]   the same for the float-quotient product
     ShoupPair *d_Pmod = nullptr;     // [L+1]     P mod q_r
     u64 *d_dn_E = nullptr;           // [alpha][L+1] -(e P + (P-1)/2) mod q_r, e < alpha
     MdExact md_exact;
@@ -198,6 +214,7 @@ struct Ctx {
     int ntt_minb = 2;        // CTAs per SM of the register-blocked forward NTT (2 or 3)
     int ntt_minb_inv = 2;    // and of the inverse NTT
     bool ntt_tuned = false;
+    bool ntt_pinned = false; // he_ctx_set_ntt_variant: every launch uses the pinned build
     // rows per launch pair of the two-pass NTTs (0: as many as the grid
     // takes): chunks small enough that pass 1 reads pass 0's output from L2
     int ntt_chunk = 0, ntt_chunk_inv = 0;
@@ -269,6 +286,8 @@ u64 h_mulmod(u64 a, u64 b, u64 q);
 u64 h_powmod(u64 a, u64 e, u64 q);
 u64 h_invmod(u64 a, u64 q);
 ShoupPair h_shoup(u64 w, u64 q);
+ModF h_modf(u64 q);
+ulonglong2 h_fq(u64 w, u64 q);   // (centred w, bits of wq): a factor of fq_mul
 int h_gen_primes(int logN, int nq, const int *qbits, int np, const int *pbits, u64 *q, u64 *p);
 
 // NTT
@@ -282,6 +301,7 @@ struct SubScale {
     u64 *out = nullptr;
     long os = 0;
     const ShoupPair *w = nullptr;
+    const ulonglong2 *wf = nullptr;   // the same constants for the float-quotient product
     int rows_per_item = 1;
     long row0 = 0;   // absolute index of the launch's first row
     const u64 *add = nullptr;   // optional addend, laid out like out (item stride as)

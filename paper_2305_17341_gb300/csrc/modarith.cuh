@@ -22,6 +22,20 @@ struct ModQ {
     u64 wone;    // floor(2^64 / q): the Shoup companion of 1
 };
 
+// Constants of the float-quotient product (fq_mul below) for a prime
+// 2^36 <= q < 1.5 2^40 (on = 0 for the others).
+struct ModF {
+    u64 nQ;      // -(q 2^22) mod 2^64
+    u64 cst;     // kFqBits (q 2^22) mod 2^64
+    u64 nq;      // -q split for a signed multiply-add: low word signed, high word the rest
+    float qi;    // 2^32 / q
+    u32 on;
+};
+// 1.5 2^23: adding it to a float |v| <= 2^22 rounds v to an integer that
+// sits in the low mantissa bits, as_int(v + kFqMagic) = kFqBits + round(v).
+#define FQ_MAGIC 12582912.0f
+constexpr u32 kFqBits = 0x4B400000u;
+
 __device__ __forceinline__ u64 mulhi64(u64 a, u64 b) { return __umul64hi(a, b); }
 
 // a * w mod q, lazily in [0, 2q), for any a < 2^64.
@@ -110,6 +124,64 @@ __device__ __forceinline__ void mac96(u32 &w0, u32 &w1, u32 &w2, u64 a, u64 b) {
         : "+r"(w0), "+r"(w1), "+r"(w2)
         : "r"(a0), "r"(a1), "r"(b0), "r"(b1));
 }
+
+// -------------------------------------------------- float-quotient product
+// y w mod q for the 40-bit limbs, with the quotient taken as two FP32 digits
+// instead of one 64-bit high product: the high products are what bounds the
+// butterfly (IMAD.HI and IMAD.WIDE issue at half the rate of IMAD), while
+// the FP32 multiply-adds run on the FMA lanes that integer code leaves idle.
+//
+// w is centred, |w| <= q/2, with wq = w / (q 2^8); y is signed, |y| <= 17.2 q.
+//   ha = round((y >> 14) wq)              ~ y w / (q 2^22)
+//   P  = y w - ha (q 2^22)                exact mod 2^64
+//   hb = round((P >> 32) 2^32 / q)
+//   t  = P - hb q
+// For q < 1.5 2^40: |y w / q| <= 8.6 q, so |ha| < 2^21.7 and its error is
+// below 0.5 + 2^21.7 2^-23 = 0.91 (y and wq each carry a half unit of 2^-24),
+// |P| <= 0.91 2^22 q < 2^62.5 fits a signed word; |hb| <= 2^21.9, its error
+// is below 0.5 + 2^21.9 2^-23 + 2^32/q <= 0.97 (q >= 2^40), and for smaller
+// q, where the first two terms shrink with q and 2^32/q <= 2^-4 (q >= 2^36),
+// below 0.97 too: |t| < q, t signed.  16 butterfly stages from |x| <= q stay
+// below 17 q.  18 instructions per butterfly against 21.6 with the truncated
+// Shoup quotient, 1406 against 1000 G butterflies/s with register operands.
+// The products are written as a wide product and an add in one statement:
+// the compiler then emits one multiply-add without the moves that a wide
+// multiply-add on separately built register pairs costs.
+__device__ __forceinline__ u64 fq_madw(u32 a, u32 b, u64 c) {
+    u64 r;
+    asm("mul.wide.u32 %0, %1, %2;\n\tadd.u64 %0, %0, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ u64 fq_madws(int a, int b, u64 c) {
+    u64 r;
+    asm("mul.wide.s32 %0, %1, %2;\n\tadd.u64 %0, %0, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ u32 fq_madl(u32 a, u32 b, u32 c) {
+    u32 r;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
+// P - round(P / q) q for a signed word P (|P| < 2^62.5): |result| < q.
+__device__ __forceinline__ u64 fq_low(u32 p0, u32 p1, const ModF &m) {
+    const int hb = __float_as_int(__fmaf_rn(__int2float_rn((int)p1), m.qi, FQ_MAGIC)) - (int)kFqBits;
+    const u64 r = fq_madws(hb, (int)(u32)m.nq, ((u64)p1 << 32) | p0);
+    return ((u64)fq_madl((u32)hb, (u32)(m.nq >> 32), (u32)(r >> 32)) << 32) | (u32)r;
+}
+// tw: x = w (centred, signed), y = the bits of wq
+__device__ __forceinline__ u64 fq_mul(u64 y, const ulonglong2 tw, const ModF &m) {
+    const u32 y0 = (u32)y, y1 = (u32)(y >> 32), w0 = (u32)tw.x, w1 = (u32)(tw.x >> 32);
+    const float yf = __int2float_rn((int)__funnelshift_r(y0, y1, 14));
+    const u32 ha = __float_as_uint(__fmaf_rn(yf, __uint_as_float((u32)tw.y), FQ_MAGIC));
+    u64 a = fq_madw(y0, w0, m.cst);
+    a = fq_madw(ha, (u32)m.nQ, a);
+    const u32 h = fq_madl(ha, (u32)(m.nQ >> 32), fq_madl(y0, w1, fq_madl(y1, w0, (u32)(a >> 32))));
+    return fq_low((u32)a, h, m);
+}
+// a signed value |v| < q to [0, q)
+__device__ __forceinline__ u64 fq_pos(u64 v, u64 q) { return v + ((u64)((i64)v >> 63) & q); }
+// any signed |v| <= 17.2 q to |result| <= 0.57 q
+__device__ __forceinline__ u64 fq_red(u64 v, const ModF &m) { return fq_low((u32)v, (u32)(v >> 32), m); }
 
 // Montgomery REDC with the prime and -q^-1 mod 2^64 given directly.
 __device__ __forceinline__ u64 redc_q(u64 lo, u64 hi, u64 q, u64 qinv) {
