@@ -225,18 +225,17 @@ int he_ctx_destroy(he_ctx *ctx) {
     for (auto &kv : c.ptcache) cudaFree(kv.second);
     for (auto &kv : c.dcd)
         for (auto &f : kv.second.factors) cudaFree(f.dev);
-    void *ptrs[] = {c.d_mod, c.d_modf, c.d_ninvf, c.d_dn_Pinvf, c.d_psi, c.d_psip, c.d_ipsi, c.d_ipsip, c.d_psi2, c.d_ipsi2, c.d_ninv, c.d_dn_pinv,
+    void *ptrs[] = {c.d_mod, c.d_modf, c.d_ninvf, c.d_dn_Pinvf, c.d_dn_fq, c.d_psi, c.d_psip, c.d_ipsi, c.d_ipsip, c.d_psi2, c.d_ipsi2, c.d_ninv, c.d_dn_pinv,
                     c.d_dn_pmod,
                     c.d_dn_Pinv, c.d_Pmod, c.d_dn_E, c.d_zeta, c.d_slot_t, c.d_sk, c.d_skM,
                     c.d_pkM};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (auto &l : c.lvl) {
-        if (l.d_up_inv) cudaFree(l.d_up_inv);
-        if (l.d_up_mod) cudaFree(l.d_up_mod);
-        if (l.d_rs_inv) cudaFree(l.d_rs_inv);
-        if (l.d_rs_invf) cudaFree(l.d_rs_invf);
-        if (l.d_rs_qlmod) cudaFree(l.d_rs_qlmod);
+        void *lp[] = {l.d_up_inv, l.d_up_mod, l.d_up_fq, l.d_rs_inv, l.d_rs_invf, l.d_rs_qlmod, l.d_mr_inv, l.d_mr_invf,
+                      l.d_mr_E};
+        for (void *p : lp)
+            if (p) cudaFree(p);
     }
     c.pool.release_all();
     if (c.h_err) cudaFreeHost(c.h_err);

@@ -149,6 +149,20 @@ ulonglong2 h_fq(u64 w, u64 q) {
     return make_ulonglong2((u64)c, b);
 }
 
+FqPair h_fq_pair(u64 w, u64 q) {
+    FqPair p;
+    ulonglong2 *o[2] = {&p.lo, &p.hi};
+    for (int i = 0; i < 2; i++) {
+        const u64 v = i ? h_mulmod(w % q, ((u64)1 << 32) % q, q) : w % q;
+        const i64 c = v > q / 2 ? (i64)(v - q) : (i64)v;
+        const float f = (float)((double)c / (double)q / 4194304.0);
+        u32 b;
+        std::memcpy(&b, &f, 4);
+        *o[i] = make_ulonglong2((u64)c, b);
+    }
+    return p;
+}
+
 static ModQ make_mod(u64 q) {
     ModQ m;
     m.q = q;
@@ -301,6 +315,7 @@ const LevelConsts &Ctx::lc(int level) {
     LC.ndig = ndig(level);
     int rows = level + 1 + alpha;
     std::vector<ShoupPair> inv((size_t)LC.ndig * alpha), mod((size_t)LC.ndig * alpha * rows);
+    std::vector<FqPair> fq(mod.size());
     for (int d = 0; d < LC.ndig; d++) {
         int i0 = d * alpha, ns = std::min(alpha, level + 1 - i0);
         for (int s = 0; s < ns; s++) {
@@ -314,12 +329,16 @@ const LevelConsts &Ctx::lc(int level) {
                 u64 v = 1;
                 for (int t = 0; t < ns; t++)
                     if (t != s) v = h_mulmod(v, primes[i0 + t] % pr, pr);
-                mod[((size_t)d * alpha + s) * rows + r] = h_shoup(v, pr);
+                const size_t o = ((size_t)d * alpha + s) * rows + r;
+                mod[o] = h_shoup(v, pr);
+                fq[o] = h_fq_pair(v, pr);
+                if (qi < kNarrow) fq[o].lo = h_fq(v, pr);
             }
         }
     }
     LC.d_up_inv = upload(inv);
     LC.d_up_mod = upload(mod);
+    LC.d_up_fq = upload(fq);
     if (level > 0) {
         std::vector<ShoupPair> ri(level);
         std::vector<u64> rm(level);
@@ -332,6 +351,25 @@ const LevelConsts &Ctx::lc(int level) {
         std::vector<ulonglong2> rf(level);
         for (int i = 0; i < level; i++) rf[i] = h_fq(ri[i].w, primes[i]);
         LC.d_rs_invf = upload(rf);
+        std::vector<ShoupPair> mi(level);
+        std::vector<ulonglong2> mf(level);
+        std::vector<u64> mE(2 * (size_t)alpha * level);
+        for (int i = 0; i < level; i++) {
+            const u64 qi = primes[i];
+            u64 P = 1;
+            for (int t = 0; t < alpha; t++) P = h_mulmod(P, primes[L + 1 + t] % qi, qi);
+            mi[i] = h_shoup(h_invmod(h_mulmod(P, ql % qi, qi), qi), qi);
+            mf[i] = h_fq(mi[i].w, qi);
+            const u64 h = h_mulmod((P + qi - 1) % qi, h_invmod(2, qi), qi), qP = h_mulmod(ql % qi, P, qi);
+            for (int neg = 0; neg < 2; neg++)
+                for (int e = 0; e < alpha; e++) {
+                    const u64 t = (h_mulmod((u64)e, P, qi) + h + (neg ? qP : 0)) % qi;
+                    mE[((size_t)neg * alpha + e) * level + i] = t ? qi - t : 0;
+                }
+        }
+        LC.d_mr_inv = upload(mi);
+        LC.d_mr_invf = upload(mf);
+        LC.d_mr_E = upload(mE);
         LC.d_rs_qlmod = upload(rm);
     }
     return LC;
@@ -438,6 +476,12 @@ void build_tables(Ctx *c) {
     for (int r = 0; r <= L; r++) Pinvf[r] = h_fq(Pinv[r].w, c->primes[r]);
     c->d_dn_Pinvf = upload(Pinvf);
     c->d_Pmod = upload(Pmod);
+    std::vector<FqPair> dfq((size_t)(a + 1) * (L + 1));
+    for (int j = 0; j <= a; j++)
+        for (int r = 0; r <= L; r++)
+            dfq[(size_t)j * (L + 1) + r] =
+                h_fq_pair(j < a ? pmod[(size_t)j * (L + 1) + r].w : Pmod[r].w, c->primes[r]);
+    c->d_dn_fq = upload(dfq);
     // h = (P-1)/2 reduced mod every prime: 2h = P - 1 exactly (P odd)
     MdExact &mk = c->md_exact;
     mk = MdExact();

@@ -15,8 +15,7 @@ namespace he {
 void modup(Ctx *c, const u64 *poly, long item_s, int B, int level, u64 *digits) {
     const int N = c->N, nq = level + 1;
     Buf coef(&c->pool, (size_t)B * nq * N);
-    launch_copy_rows(coef.p, (long)nq * N, poly, item_s, B, (long)nq * N, c->stream);
-    ntt_inv(c, coef.p, (long)B * nq, c->map_q(level), c->stream);
+    ntt_inv(c, coef.p, (long)B * nq, c->map_q(level), c->stream, NttSrc{poly, item_s, nq});
     const long rows = (long)B * c->ndig(level) * c->qp_rows(level);
     if (c->logN >= 14 && c->logN <= 16) {
         // the digit's own rows are the input's NTT-domain rows: copy them and
@@ -40,8 +39,7 @@ void modup(Ctx *c, const u64 *poly, long item_s, int B, int level, u64 *digits) 
 void moddown(Ctx *c, const u64 *u, int items, int level, u64 *out, long out_s, const u64 *add, long add_s) {
     const int N = c->N, rows = c->qp_rows(level), a = c->alpha;
     Buf pc(&c->pool, (size_t)items * a * N), conv(&c->pool, (size_t)items * (level + 1) * N);
-    launch_copy_rows(pc.p, (long)a * N, u + (long)(level + 1) * N, (long)rows * N, items, (long)a * N, c->stream);
-    ntt_inv(c, pc.p, (long)items * a, c->map_p(), c->stream);
+    ntt_inv(c, pc.p, (long)items * a, c->map_p(), c->stream, NttSrc{u + (long)(level + 1) * N, (long)rows * N, a});
     launch_moddown_bconv(c, pc.p, conv.p, items, level, c->stream);
     if (c->logN >= 14 && c->logN <= 16) {
         // the NTT's last pass writes out = (u_Q - conv) P^-1 directly
@@ -106,9 +104,8 @@ void rescale(Ctx *c, const u64 *in, int B, int level, u64 *out) {
     const int N = c->N;
     if (level < 1) throw HeError(HE_ERR_LEVEL, "rescale at level 0");
     Buf last(&c->pool, (size_t)2 * B * N), t(&c->pool, (size_t)2 * B * level * N);
-    launch_copy_rows(last.p, N, in + (long)level * N, (long)(level + 1) * N, 2 * B, N, c->stream);
     RowMap one = RowMap::single(level);
-    ntt_inv(c, last.p, 2L * B, one, c->stream);
+    ntt_inv(c, last.p, 2L * B, one, c->stream, NttSrc{in + (long)level * N, (long)(level + 1) * N, 1});
     launch_rescale_prep(c, last.p, t.p, 2 * B, level, c->stream);
     if (c->logN >= 14 && c->logN <= 16) {
         // the NTT's last pass writes out = (in - t) q_l^-1 directly
@@ -120,6 +117,27 @@ void rescale(Ctx *c, const u64 *in, int B, int level, u64 *out) {
         ntt_fwd(c, t.p, 2L * B * level, c->map_q(level - 1), c->stream);
         launch_rescale_final(c, out, in, t.p, 2 * B, level, (long)(level + 1) * N, (long)level * N, c->stream);
     }
+}
+
+// ModDown then Rescale of items over Q_l P ([2 B][rows][N]) -> [B][2][l][N]:
+// the words of moddown and rescale in a row, with one forward NTT of l rows per
+// polynomial for the two (k_moddown_bconv, RS).
+void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out) {
+    const int N = c->N, rows = c->qp_rows(level), a1 = c->alpha + 1;
+    if (level < 1) throw HeError(HE_ERR_LEVEL, "rescale at level 0");
+    if (c->logN < 14 || c->logN > 16) {
+        Buf t(&c->pool, (size_t)B * 2 * (level + 1) * N);
+        moddown(c, u, 2 * B, level, t.p, (long)(level + 1) * N);
+        rescale(c, t.p, B, level, out);
+        return;
+    }
+    Buf pc(&c->pool, (size_t)2 * B * a1 * N), z(&c->pool, (size_t)2 * B * level * N);
+    ntt_inv(c, pc.p, 2L * B * a1, c->map_lp(level), c->stream, NttSrc{u + (long)level * N, (long)rows * N, a1});
+    launch_moddown_rescale_bconv(c, pc.p, z.p, 2 * B, level, c->stream);
+    SubScale ep;
+    ep.u = u, ep.us = (long)rows * N, ep.out = out, ep.os = (long)level * N;
+    ep.w = c->lc(level).d_mr_inv, ep.wf = c->lc(level).d_mr_invf, ep.rows_per_item = level;
+    ntt_fwd_subscale(c, z.p, 2L * B * level, c->map_q(level - 1), c->stream, ep);
 }
 
 // Level drop: keep limbs 0..to of both polys.
@@ -293,9 +311,8 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
             launch_add(c, acc.p, acc.p, term, 2L * B * rows, qp, c->stream);
         }
     }
-    moddown(c, acc.p, 2 * B, level, ctmp.p, (long)nq * N);
+    moddown_rescale(c, acc.p, B, level, out);
     c->n_md += B;
-    rescale(c, ctmp.p, B, level, out);
 }
 
 // ct <- ct + Rot(ct, -n^2 2^j) for j = 0 .. log2(S/n^2)-1 (period n^2).
@@ -398,7 +415,7 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
     Buf AkP(&c->pool, ident ? 1 : P * ct2), BkP(&c->pool, ident ? 1 : P * ct2);
     // relin_once: the summed d2 of the n tensors (d0, d1 are summed in acc)
     Buf acc2(&c->pool, relin_once ? (size_t)P * (l2 + 1) * N : 1);
-    Buf R1(&c->pool, nA * qp1), R2(&c->pool, nA * qp1), S(&c->pool, nA * qp1), Akp(&c->pool, nA * ct1);
+    Buf R1(&c->pool, nA * qp1), R2(&c->pool, nA * qp1), S(&c->pool, nA * qp1);
     RowMap q2 = c->map_q(l2);
 
     // The babies of a source are all its hoisted rotations at once (one
@@ -469,9 +486,8 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
                 const u64 *Rs[2] = {R1.p, R2.p};
                 launch_pmul_acc(c, S.p, pts, Rs, 2, nA, l1, (long)qp1, c->stream);
             }
-            moddown(c, Sk, 2 * nA, l1, Akp.p, (long)(l1 + 1) * N);
+            moddown_rescale(c, Sk, nA, l1, Ak.p);
             c->n_md += nA;
-            rescale(c, Akp.p, nA, l1, Ak.p);
         }
         // ---- B^(k) = R^k B^(0), dropped to l2
         int gb2 = k / n1t, bb = k % n1t;

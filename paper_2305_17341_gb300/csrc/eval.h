@@ -31,6 +31,7 @@ void rot_qp_multi(Ctx *c, const u64 *ct, int B, int level, const u64 *digits, co
 void rotate_digits(Ctx *c, const u64 *ct, int B, int level, const u64 *digits, uint32_t g, u64 *out);
 void rotate(Ctx *c, const u64 *ct, int B, int level, uint32_t g, u64 *out);
 void rescale(Ctx *c, const u64 *in, int B, int level, u64 *out);
+void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out);
 void drop(Ctx *c, const u64 *in, int B, int level, int to, u64 *out);
 // b may sit at a higher level b_level (its first level + 1 limbs are used in place)
 void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out, bool accumulate = false,

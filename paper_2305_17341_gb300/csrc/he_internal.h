@@ -107,6 +107,9 @@ struct ShoupPair {
     u64 w, wp;
 };
 
+// Sources below this bound are converted as one narrow word (FqDot::narrow).
+constexpr u64 kNarrow = 1ull << 41;
+
 // Constants of the exact overflow count of the rounding ModDown, alpha <= 4
 // special primes below 2^62 (kernel parameter).
 struct MdExact {
@@ -123,10 +126,16 @@ struct LevelConsts {
     // ModUp: per digit d, per source i (alpha max), qhat_inv (pair); per target row r, qhat_mod[d][i][r]
     ShoupPair *d_up_inv = nullptr;   // [ndig][alpha]
     ShoupPair *d_up_mod = nullptr;   // [ndig][alpha][l+1+alpha]
+    FqPair *d_up_fq = nullptr;       // the same for float-quotient rows
     // Rescale by q_l: q_l^-1 mod q_i, q_l mod q_i (i < l)
     ShoupPair *d_rs_inv = nullptr;   // [l]
     ulonglong2 *d_rs_invf = nullptr; // [l] the same for the float-quotient product
     u64 *d_rs_qlmod = nullptr;       // [l]
+    // ModDown fused with the rescale by q_l (i < l): (P q_l)^-1 mod q_i, and
+    // -(e P + (P-1)/2) - neg q_l P mod q_i for e < alpha, neg < 2
+    ShoupPair *d_mr_inv = nullptr;     // [l]
+    ulonglong2 *d_mr_invf = nullptr;   // [l]
+    u64 *d_mr_E = nullptr;             // [2][alpha][l]
 };
 
 // One factor of a Diagonal Convergence Decomposition (Sec. 4.2): the
@@ -171,6 +180,7 @@ struct Ctx {
     ShoupPair *d_dn_Pinv = nullptr;  // [L+1]     P^-1 mod q_r
     ulonglong2 *d_dn_Pinvf = nullptr;  // [L+1]   the same for the float-quotient product
     ShoupPair *d_Pmod = nullptr;     // [L+1]     P mod q_r
+    FqPair *d_dn_fq = nullptr;       // [alpha+1][L+1] (P/p_j) mod q_r, then P mod q_r, for float-quotient rows
     u64 *d_dn_E = nullptr;           // [alpha][L+1] -(e P + (P-1)/2) mod q_r, e < alpha
     MdExact md_exact;
     std::vector<LevelConsts> lvl;
@@ -249,6 +259,12 @@ struct Ctx {
         m.n = level + 1 + alpha, m.lq = level, m.base_p = L + 1;
         return m;
     }
+    // q_level, then the special primes
+    RowMap map_lp(int level) const {
+        RowMap m;
+        m.n = alpha + 1, m.lq = 0, m.base_q = level, m.base_p = L + 1;
+        return m;
+    }
     RowMap map_p() const {
         RowMap m;
         m.n = alpha, m.lq = -1, m.base_p = L + 1;
@@ -288,6 +304,7 @@ u64 h_invmod(u64 a, u64 q);
 ShoupPair h_shoup(u64 w, u64 q);
 ModF h_modf(u64 q);
 ulonglong2 h_fq(u64 w, u64 q);   // (centred w, bits of wq): a factor of fq_mul
+FqPair h_fq_pair(u64 w, u64 q);  // a factor of FqDot::wide
 int h_gen_primes(int logN, int nq, const int *qbits, int np, const int *pbits, u64 *q, u64 *p);
 
 // NTT
@@ -308,7 +325,15 @@ struct SubScale {
     long as = 0;
 };
 void ntt_fwd_subscale(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStream_t st, const SubScale &ep);
-void ntt_inv(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStream_t st);
+// src (may be null): the input, items of rows_per_item contiguous rows at a
+// stride of `stride` words; the output goes to data ([rows][N]).
+struct NttSrc {
+    const u64 *src = nullptr;
+    long stride = 0;
+    int rows_per_item = 1;
+    unsigned row0 = 0;
+};
+void ntt_inv(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStream_t st, const NttSrc &src = NttSrc());
 
 // ---- kernels.cu launchers (all asynchronous on st) ----
 void launch_sample_uniform(Ctx *c, u64 *out, int rows, const RowMap &rm, const int *limb_id, uint32_t obj,
@@ -348,6 +373,10 @@ void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, in
 void launch_modup_bconv(Ctx *c, const u64 *coef, u64 *out, int B, int level, cudaStream_t st,
                         const u64 *own_ntt = nullptr, long own_s = 0);
 void launch_moddown_bconv(Ctx *c, const u64 *pcoef, u64 *out, int items, int level, cudaStream_t st);
+// The conversion of ModDown followed by Rescale: pcoef [items][1+alpha][N] holds
+// row q_l then the p rows in coefficient form; out [items][l][N] is what
+// (u_i - NTT(out_i)) (P q_l)^-1 takes.
+void launch_moddown_rescale_bconv(Ctx *c, const u64 *pcoef, u64 *out, int items, int level, cudaStream_t st);
 void launch_moddown_final(Ctx *c, u64 *out, const u64 *u, const u64 *conv, const u64 *addend, int items,
                           int level, long u_item_stride, long out_item_stride, long add_item_stride,
                           cudaStream_t st);

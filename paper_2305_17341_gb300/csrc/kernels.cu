@@ -356,11 +356,9 @@ void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, in
 // blockIdx.y is the digit: a CTA stages that digit's conversion constants
 // and row primes in shared memory once and walks (item, coefficient pair)
 // with a grid stride.  Each thread converts two adjacent coefficients with
-// 16-byte loads and stores.  When the digit's primes and the row's prime are
-// below 2^42 the products y_i (w_i 2^64 mod r) accumulate in 96 bits with
-// carry-chained 32-bit multiply-adds and one Montgomery reduction ends the
-// row; otherwise the A lazy Shoup products (each in [0, 2r)) are summed and
-// reduced once.
+// 16-byte loads and stores.  Rows of 40-bit primes sum their products with one
+// float quotient (FqDot); the others sum A lazy Shoup products (each in
+// [0, 2r)) and reduce once.  Bound by the integer multiplies (FMA-heavy pipe).
 static int sm_count(int dev) {
     static int n[64];
     dev &= 63;
@@ -392,36 +390,36 @@ __device__ __forceinline__ void store_words(u64 *p, const Words<C> &r) {
 
 // A: special primes per digit; C: adjacent coefficients per thread (2 on
 // launches that fill the GPU, 1 on small ones, where more threads hide more
-// latency).
+// latency).  up_fq null: every row takes the Shoup products.
 template <int A, int C>
 __global__ void __launch_bounds__(256) k_modup_bconv(const u64 *coef, u64 *out, int B, int level, int ndig, int N,
-                                                     RowMap qp, const ModQ *mods, const ShoupPair *up_inv,
-                                                     const ShoupPair *up_mod, const u64 *own_ntt, long own_s) {
+                                                     RowMap qp, const ModQ *mods, const ModF *modf,
+                                                     const ShoupPair *up_inv, const ShoupPair *up_mod,
+                                                     const FqPair *up_fq, const u64 *own_ntt, long own_s) {
     __shared__ ShoupPair s_mod[A * 64];   // [s][r], rows <= 64
-    __shared__ u64 s_mont[A * 64];        // w 2^64 mod r of the same constants
-    __shared__ u64 s_q[64], s_w1[64], s_qinv[64];
+    __shared__ FqPair s_fq[A * 64];
+    __shared__ ModF s_f[64];
+    __shared__ u64 s_q[64], s_w1[64];
     const int d = blockIdx.y;
     const int rows = level + 1 + A;
     const int i0 = d * A;
     const int ns = min(A, level + 1 - i0);
     for (int r = threadIdx.x; r < rows; r += blockDim.x) {
-        const ModQ m = mods[r <= qp.lq ? r : qp.base_p + (r - qp.lq - 1)];   // qp is unshifted
-        s_q[r] = m.q, s_w1[r] = m.wone, s_qinv[r] = m.qinv;
+        const int p = r <= qp.lq ? r : qp.base_p + (r - qp.lq - 1);   // qp is unshifted
+        s_q[r] = mods[p].q, s_w1[r] = mods[p].wone, s_f[r] = modf[p];
+        if (!up_fq) s_f[r].on = 0;
     }
-    __syncthreads();
     for (int e = threadIdx.x; e < ns * rows; e += blockDim.x) {
         const int sd = e / rows, r = e - sd * rows;
-        const ShoupPair w = up_mod[((long)d * A + sd) * rows + r];
-        s_mod[e] = w;
-        // w 2^64 - w' r is in [0, r) and congruent to -w' r modulo 2^64
-        s_mont[e] = (u64)0 - w.wp * s_q[r];
+        s_mod[e] = up_mod[((long)d * A + sd) * rows + r];
+        if (up_fq) s_fq[e] = up_fq[((long)d * A + sd) * rows + r];
     }
     ShoupPair inv[A];
     u64 qs[A];
-    bool narrow = true;   // every source prime below 2^42 (uniform over the CTA)
+    bool narrow[A];   // uniform over the CTA
 #pragma unroll
     for (int sd = 0; sd < A; sd++)
-        if (sd < ns) inv[sd] = up_inv[d * A + sd], qs[sd] = mods[i0 + sd].q, narrow = narrow && qs[sd] < (1ull << 42);
+        if (sd < ns) inv[sd] = up_inv[d * A + sd], qs[sd] = mods[i0 + sd].q, narrow[sd] = qs[sd] < kNarrow;
     __syncthreads();
     const int per = N / C;
     const long units = (long)B * per;
@@ -445,21 +443,24 @@ __global__ void __launch_bounds__(256) k_modup_bconv(const u64 *coef, u64 *out, 
             Words<C> o;
             if (r >= i0 && r < i0 + ns) {   // uniform over the CTA
                 o = load_words<C>(own_ntt ? own_ntt + (long)b * own_s + (long)r * N + x : cb + (long)r * N);
-            } else if (narrow && s_q[r] < (1ull << 42)) {   // uniform over the CTA
-                // products below 2^84: A of them stay below 2^86 < r 2^64
-                u32 w0[C], w1[C], w2[C];
+            } else if (s_f[r].on) {   // uniform over the CTA
+                const ModF m = s_f[r];
+                FqDot t[C];
 #pragma unroll
-                for (int c = 0; c < C; c++) w0[c] = w1[c] = w2[c] = 0;
+                for (int c = 0; c < C; c++) t[c] = FqDot(0, m);
 #pragma unroll
                 for (int sd = 0; sd < A; sd++) {
                     if (sd < ns) {
-                        const u64 wm = s_mont[sd * rows + r];
+                        const FqPair w = s_fq[sd * rows + r];
 #pragma unroll
-                        for (int c = 0; c < C; c++) mac96(w0[c], w1[c], w2[c], y[c][sd], wm);
+                        for (int c = 0; c < C; c++) {
+                            if (narrow[sd]) t[c].narrow(y[c][sd], w.lo);
+                            else t[c].wide(y[c][sd], w);
+                        }
                     }
                 }
 #pragma unroll
-                for (int c = 0; c < C; c++) o.w[c] = redc_q(((u64)w1[c] << 32) | w0[c], w2[c], s_q[r], s_qinv[r]);
+                for (int c = 0; c < C; c++) o.w[c] = t[c].get(s_q[r], m);
             } else {
                 const u64 q = s_q[r];
                 u64 acc[C];
@@ -484,7 +485,8 @@ __global__ void __launch_bounds__(256) k_modup_bconv(const u64 *coef, u64 *out, 
 
 template <int A>
 static void modup_launch_a(Ctx *c, const u64 *coef, u64 *out, int B, int level, int nd, const ShoupPair *up_inv,
-                           const ShoupPair *up_mod, const u64 *own_ntt, long own_s, cudaStream_t st) {
+                           const ShoupPair *up_mod, const FqPair *up_fq, const u64 *own_ntt, long own_s,
+                           cudaStream_t st) {
     const int nsm = sm_count(c->device);
     // two coefficients per thread once the launch fills the GPU with 8 CTAs
     // of 256 threads per SM, one below that
@@ -495,18 +497,19 @@ static void modup_launch_a(Ctx *c, const u64 *coef, u64 *out, int B, int level, 
     const dim3 grid((unsigned)gx, (unsigned)nd);
     const RowMap qp = c->map_qp(level);
     if (wide)
-        k_modup_bconv<A, 2><<<grid, 256, 0, st>>>(coef, out, B, level, nd, c->N, qp, c->d_mod, up_inv, up_mod, own_ntt, own_s);
+        k_modup_bconv<A, 2><<<grid, 256, 0, st>>>(coef, out, B, level, nd, c->N, qp, c->d_mod, c->d_modf, up_inv, up_mod, up_fq, own_ntt, own_s);
     else
-        k_modup_bconv<A, 1><<<grid, 256, 0, st>>>(coef, out, B, level, nd, c->N, qp, c->d_mod, up_inv, up_mod, own_ntt, own_s);
+        k_modup_bconv<A, 1><<<grid, 256, 0, st>>>(coef, out, B, level, nd, c->N, qp, c->d_mod, c->d_modf, up_inv, up_mod, up_fq, own_ntt, own_s);
 }
 
 static void modup_launch(Ctx *c, const u64 *coef, u64 *out, int B, int level, int nd, const ShoupPair *up_inv,
-                         const ShoupPair *up_mod, const u64 *own_ntt, long own_s, cudaStream_t st) {
+                         const ShoupPair *up_mod, const FqPair *up_fq, const u64 *own_ntt, long own_s,
+                         cudaStream_t st) {
     switch (c->alpha) {
-    case 1: modup_launch_a<1>(c, coef, out, B, level, nd, up_inv, up_mod, own_ntt, own_s, st); break;
-    case 2: modup_launch_a<2>(c, coef, out, B, level, nd, up_inv, up_mod, own_ntt, own_s, st); break;
-    case 3: modup_launch_a<3>(c, coef, out, B, level, nd, up_inv, up_mod, own_ntt, own_s, st); break;
-    default: modup_launch_a<4>(c, coef, out, B, level, nd, up_inv, up_mod, own_ntt, own_s, st); break;
+    case 1: modup_launch_a<1>(c, coef, out, B, level, nd, up_inv, up_mod, up_fq, own_ntt, own_s, st); break;
+    case 2: modup_launch_a<2>(c, coef, out, B, level, nd, up_inv, up_mod, up_fq, own_ntt, own_s, st); break;
+    case 3: modup_launch_a<3>(c, coef, out, B, level, nd, up_inv, up_mod, up_fq, own_ntt, own_s, st); break;
+    default: modup_launch_a<4>(c, coef, out, B, level, nd, up_inv, up_mod, up_fq, own_ntt, own_s, st); break;
     }
 }
 
@@ -516,7 +519,7 @@ void launch_modup_bconv(Ctx *c, const u64 *coef, u64 *out, int B, int level, cud
     c->n_launch++;
     cudaEvent_t e0;
     c->trace_begin(3, e0);
-    modup_launch(c, coef, out, B, level, L.ndig, L.d_up_inv, L.d_up_mod, own_ntt, own_s, st);
+    modup_launch(c, coef, out, B, level, L.ndig, L.d_up_inv, L.d_up_mod, L.d_up_fq, own_ntt, own_s, st);
     // the input limbs once, every digit's extended limbs once
     c->trace_end(3, e0, 8.0 * B * c->N * ((level + 1) + (double)L.ndig * c->qp_rows(level)));
 }
@@ -525,7 +528,7 @@ void launch_modup_bconv(Ctx *c, const u64 *coef, u64 *out, int B, int level, cud
 void launch_modup_bconv_with(Ctx *c, const u64 *coef, u64 *out, int B, int level, const ShoupPair *up_inv,
                              const ShoupPair *up_mod, cudaStream_t st) {
     c->n_launch++;
-    modup_launch(c, coef, out, B, level, c->ndig(level), up_inv, up_mod, nullptr, 0, st);
+    modup_launch(c, coef, out, B, level, c->ndig(level), up_inv, up_mod, nullptr, nullptr, 0, st);
 }
 
 // ----------------------------------------------------- constants per limb
@@ -626,83 +629,136 @@ __device__ __forceinline__ int md_overflow(const u64 (&y)[A], const MdExact &k) 
 
 // C adjacent coefficients per thread (2: 16-byte loads and stores, on
 // launches that fill the GPU; 1 on small ones), a grid stride over (item,
-// coefficient group); per row the lazy Shoup products and E are summed and
-// reduced once.
-template <int A, int C>
+// coefficient group); per row the products are summed with one float quotient
+// (40-bit rows) or as lazy Shoup products reduced once.
+//
+// RS: the ModDown of a ciphertext that is rescaled by q_l next.  With
+// conv_r = ((x + h) mod P) - h as above, ModDown is d_r = (u_r - conv_r) P^-1, and
+// the rescale takes t = d_l centred (coefficient form, from row l of u):
+// (d_i - t) q_l^-1 = (u_i - (conv_i + t P)) (P q_l)^-1, so one forward NTT of
+// z_i = conv_i + t P does for both: out [items][l][N] holds z.  pcoef:
+// [items][1 + A][N], row q_l first.  E: [neg][e][r], -q_l P folded in where the
+// centred t is negative.
+template <int A, int C, bool RS>
 __global__ void __launch_bounds__(256) k_moddown_bconv(const u64 *pcoef, u64 *out, int items, int level, int N,
                                                        const __grid_constant__ MdExact k, const ModQ *mods,
-                                                       const ShoupPair *pmod, const u64 *E, int L) {
-    __shared__ ShoupPair s_c[A * 64];
-    __shared__ u64 s_E[A * 64], s_q[64], s_w1[64];
-    const int nr = level + 1;
-    for (int r = threadIdx.x; r < nr; r += blockDim.x) s_q[r] = mods[r].q, s_w1[r] = mods[r].wone;
-    for (int e = threadIdx.x; e < A * nr; e += blockDim.x) {
-        const int j = e / nr, r = e - j * nr;
-        s_c[e] = pmod[j * (L + 1) + r];
-        s_E[e] = E[j * (L + 1) + r];
+                                                       const ModF *modf, const ShoupPair *pmod, const FqPair *pfq,
+                                                       const ShoupPair *Pmod, const ShoupPair *Pinv, const u64 *E,
+                                                       int Es, const u64 *El, int L) {
+    constexpr int S = RS ? A + 1 : A;   // sources: y_j, then t
+    __shared__ ShoupPair s_c[S * 64];
+    __shared__ FqPair s_fq[S * 64];
+    __shared__ ModF s_f[64];
+    __shared__ u64 s_E[(RS ? 2 : 1) * A * 64], s_El[A], s_q[64], s_w1[64];
+    const int nr = RS ? level : level + 1, nt = level + 1;   // rows written; rows with constants
+    for (int r = threadIdx.x; r < nt; r += blockDim.x) s_q[r] = mods[r].q, s_w1[r] = mods[r].wone, s_f[r] = modf[r];
+    for (int e = threadIdx.x; e < S * nt; e += blockDim.x) {
+        const int j = e / nt, r = e - j * nt;
+        s_c[e] = j < A ? pmod[j * (L + 1) + r] : Pmod[r];
+        s_fq[e] = pfq[j * (L + 1) + r];
     }
+    for (int e = threadIdx.x; e < (RS ? 2 : 1) * A * nr; e += blockDim.x) {
+        const int j = e / nr, r = e - j * nr;
+        s_E[e] = E[j * Es + r];
+    }
+    if (RS && threadIdx.x < A) s_El[threadIdx.x] = El[threadIdx.x * (L + 1) + level];
+    const ShoupPair pil = RS ? Pinv[level] : ShoupPair{0, 0};
     __syncthreads();
     const int per = N / C;
     const long units = (long)items * per;
+    // sum_j y_j w_jr + e for the first n sources
+    auto dot = [&](const u64 *y, int n, int r, u64 e) -> u64 {
+        if (s_f[r].on) {   // uniform over the CTA
+            const ModF m = s_f[r];
+            FqDot t(e, m);
+#pragma unroll
+            for (int j = 0; j < S; j++)
+                if (j < n) t.wide(y[j], s_fq[j * nt + r]);
+            return t.get(s_q[r], m);
+        }
+        const u64 q = s_q[r];
+        u64 acc = e;   // < (2 S + 1) q <= 11 q < 2^64
+#pragma unroll
+        for (int j = 0; j < S; j++)
+            if (j < n) acc += shoup_lazy(y[j], s_c[j * nt + r].w, s_c[j * nt + r].wp, q);
+        return reduce_any(acc, q, s_w1[r]);
+    };
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < units; idx += (long)gridDim.x * blockDim.x) {
         const int it = (int)(idx / per);
         const int x = C * (int)(idx - (long)it * per);
-        u64 y[C][A];
+        const u64 *pi = pcoef + (long)it * S * N + x;
+        u64 y[C][S];
 #pragma unroll
         for (int j = 0; j < A; j++) {
-            const Words<C> v = load_words<C>(pcoef + ((long)it * A + j) * N + x);
+            const Words<C> v = load_words<C>(pi + (long)(RS ? j + 1 : j) * N);
             const u64 p = k.p[j];
 #pragma unroll
             for (int c = 0; c < C; c++) y[c][j] = shoup(addmod(v.w[c], k.hp[j], p), k.pinv[j].w, k.pinv[j].wp, p);
         }
         int e[C];
 #pragma unroll
-        for (int c = 0; c < C; c++) e[c] = md_overflow<A>(y[c], k);
+        for (int c = 0; c < C; c++) {
+            u64 ya[A];
+#pragma unroll
+            for (int j = 0; j < A; j++) ya[j] = y[c][j];
+            e[c] = md_overflow<A>(ya, k);
+        }
+        if constexpr (RS) {
+            const Words<C> v = load_words<C>(pi);
+            const u64 ql = s_q[level];
+#pragma unroll
+            for (int c = 0; c < C; c++) {
+                const u64 cl = dot(y[c], A, level, s_El[e[c]]);
+                const u64 t = shoup(submod(v.w[c], cl, ql), pil.w, pil.wp, ql);
+                y[c][A] = t;
+                if (t > (ql >> 1)) e[c] += A;
+            }
+        }
         u64 *op = out + (long)it * nr * N + x;
         for (int r = 0; r < nr; r++) {
-            const u64 q = s_q[r];
-            u64 acc[C];
-#pragma unroll
-            for (int c = 0; c < C; c++) acc[c] = s_E[e[c] * nr + r];
-#pragma unroll
-            for (int j = 0; j < A; j++) {
-                const ShoupPair w = s_c[j * nr + r];
-#pragma unroll
-                for (int c = 0; c < C; c++) acc[c] += shoup_lazy(y[c][j], w.w, w.wp, q);
-            }
-            // < (2 A + 1) q <= 9q < 2^64
             Words<C> o;
 #pragma unroll
-            for (int c = 0; c < C; c++) o.w[c] = reduce_any(acc[c], q, s_w1[r]);
+            for (int c = 0; c < C; c++) o.w[c] = dot(y[c], S, r, s_E[e[c] * nr + r]);
             store_words<C>(op + (long)r * N, o);
         }
     }
 }
 
-template <int A>
+template <int A, bool RS>
 static void moddown_launch_a(Ctx *c, const u64 *pcoef, u64 *out, int items, int level, cudaStream_t st) {
     const int nsm = sm_count(c->device);
     const bool wide = (long)items * (c->N / 2) >= (long)nsm * 8 * 256;
     const long units = (long)items * (c->N / (wide ? 2 : 1));
     const unsigned grid = (unsigned)std::min<long>((long)nsm * 8, nblk(units, 256));
     const MdExact &k = c->md_exact;
+    const u64 *E = RS ? c->lc(level).d_mr_E : c->d_dn_E;
+    const int Es = RS ? level : c->L + 1;
     if (wide)
-        k_moddown_bconv<A, 2><<<grid, 256, 0, st>>>(pcoef, out, items, level, c->N, k, c->d_mod, c->d_dn_pmod, c->d_dn_E, c->L);
+        k_moddown_bconv<A, 2, RS><<<grid, 256, 0, st>>>(pcoef, out, items, level, c->N, k, c->d_mod, c->d_modf, c->d_dn_pmod, c->d_dn_fq, c->d_Pmod, c->d_dn_Pinv, E, Es, c->d_dn_E, c->L);
     else
-        k_moddown_bconv<A, 1><<<grid, 256, 0, st>>>(pcoef, out, items, level, c->N, k, c->d_mod, c->d_dn_pmod, c->d_dn_E, c->L);
+        k_moddown_bconv<A, 1, RS><<<grid, 256, 0, st>>>(pcoef, out, items, level, c->N, k, c->d_mod, c->d_modf, c->d_dn_pmod, c->d_dn_fq, c->d_Pmod, c->d_dn_Pinv, E, Es, c->d_dn_E, c->L);
 }
 
-void launch_moddown_bconv(Ctx *c, const u64 *pcoef, u64 *out, int items, int level, cudaStream_t st) {
+template <bool RS>
+static void moddown_launch(Ctx *c, const u64 *pcoef, u64 *out, int items, int level, cudaStream_t st) {
     c->n_launch++;
     cudaEvent_t e0;
     c->trace_begin(4, e0);
     switch (c->alpha) {
-    case 1: moddown_launch_a<1>(c, pcoef, out, items, level, st); break;
-    case 2: moddown_launch_a<2>(c, pcoef, out, items, level, st); break;
-    case 3: moddown_launch_a<3>(c, pcoef, out, items, level, st); break;
-    default: moddown_launch_a<4>(c, pcoef, out, items, level, st); break;
+    case 1: moddown_launch_a<1, RS>(c, pcoef, out, items, level, st); break;
+    case 2: moddown_launch_a<2, RS>(c, pcoef, out, items, level, st); break;
+    case 3: moddown_launch_a<3, RS>(c, pcoef, out, items, level, st); break;
+    default: moddown_launch_a<4, RS>(c, pcoef, out, items, level, st); break;
     }
     c->trace_end(4, e0, 8.0 * items * c->N * (c->alpha + level + 1));
+}
+
+void launch_moddown_bconv(Ctx *c, const u64 *pcoef, u64 *out, int items, int level, cudaStream_t st) {
+    moddown_launch<false>(c, pcoef, out, items, level, st);
+}
+
+void launch_moddown_rescale_bconv(Ctx *c, const u64 *pcoef, u64 *out, int items, int level, cudaStream_t st) {
+    moddown_launch<true>(c, pcoef, out, items, level, st);
 }
 
 // out_r = (u_r - conv_r) P^-1 mod q_r (+ addend_r), NTT domain, r <= level.
@@ -1743,27 +1799,34 @@ void launch_lift_P(Ctx *c, u64 *out_qp, const u64 *in_q, int items, int level, l
 // t_i = [c_l]_{q_l} mod q_i for i < l (coefficient form): the centred residue
 // of the last limb (reading of App. A Rescaling: round(c / q_l)).
 // last: [items][N]; out: [items][l][N]
-__global__ void k_rescale_prep(const u64 *last, u64 *out, int items, int level, int N, const ModQ *mods,
-                               const u64 *qlmod) {
-    long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long)items * N) return;
-    int x = (int)(idx % N);
-    int it = (int)(idx / N);
-    u64 ql = mods[level].q;
-    u64 v = last[idx];
-    bool neg = v > (ql >> 1);
+__global__ void k_rescale_prep(const u64 *last, u64 *out, int items, int level, int logN, const ModQ *mods,
+                               const ModF *modf, const u64 *qlmod) {
+    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long)items << logN) return;
+    const int N = 1 << logN, x = (int)(idx & (N - 1)), it = (int)(idx >> logN);
+    const u64 ql = mods[level].q;
+    const u64 v = last[idx];
+    const bool neg = v > (ql >> 1);
+    const u64 t = neg ? v - ql : v;   // signed
+    u64 *op = out + (long)it * level * N + x;
     for (int i = 0; i < level; i++) {
-        u64 q = mods[i].q;
-        u64 r = v % q;
-        if (neg) r = submod(r, qlmod[i], q);  // v - q_l
-        out[((long)it * level + i) * N + x] = r;
+        const u64 q = mods[i].q;
+        const ModF m = modf[i];
+        u64 r;
+        if (m.on && ql < 8 * q) {   // |t| <= 4 q
+            r = fq_pos(fq_red(t, m), q);
+        } else {
+            r = reduce_any(v, q, mods[i].wone);
+            if (neg) r = submod(r, qlmod[i], q);  // v - q_l
+        }
+        op[(long)i * N] = r;
     }
 }
 void launch_rescale_prep(Ctx *c, const u64 *lastcoef, u64 *out, int items, int level, cudaStream_t st) {
     const LevelConsts &L = c->lc(level);
     long n = (long)items * c->N;
     c->n_launch++;
-    k_rescale_prep<<<nblk(n, 256), 256, 0, st>>>(lastcoef, out, items, level, c->N, c->d_mod, L.d_rs_qlmod);
+    k_rescale_prep<<<nblk(n, 256), 256, 0, st>>>(lastcoef, out, items, level, c->logN, c->d_mod, c->d_modf, L.d_rs_qlmod);
 }
 
 // out_i = (c_i - t_i) q_l^-1 mod q_i (NTT domain), i < l.

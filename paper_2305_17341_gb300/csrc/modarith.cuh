@@ -178,8 +178,48 @@ __device__ __forceinline__ u64 fq_mul(u64 y, const ulonglong2 tw, const ModF &m)
     const u32 h = fq_madl(ha, (u32)(m.nQ >> 32), fq_madl(y0, w1, fq_madl(y1, w0, (u32)(a >> 32))));
     return fq_low((u32)a, h, m);
 }
+// Factor of a 64-bit unsigned source: y w = (low word of y) lo + (high word)
+// hi with lo = w, hi = w 2^32 mod q, both centred; .y the bits of w / (q 2^22).
+// For sources below 2^41 `lo` is instead a factor of fq_mul (see FqDot::narrow).
+struct FqPair {
+    ulonglong2 lo, hi;
+};
+// Sum of products y_i w_i + e modulo a prime with ModF constants, with one
+// quotient for the sum (its two digits, as in fq_mul): 3 or 4 wide or low
+// multiply-adds per word of y against 14 multiply slots for a Shoup product.
+// At most 4 narrow sources, or 5 wide ones, and e < q.
+struct FqDot {
+    u64 a;
+    float s;
+    FqDot() = default;
+    __device__ __forceinline__ FqDot(u64 e, const ModF &m) : a(e + m.cst), s(0.0f) {}
+    __device__ __forceinline__ void word(u32 y, const ulonglong2 w) {
+        s = __fmaf_rn(__uint2float_rn(y), __uint_as_float((u32)w.y), s);
+        a = fq_madw(y, (u32)w.x, a);
+        a = ((u64)fq_madl(y, (u32)(w.x >> 32), (u32)(a >> 32)) << 32) | (u32)a;
+    }
+    __device__ __forceinline__ void wide(u64 y, const FqPair &w) {
+        word((u32)y, w.lo);
+        word((u32)(y >> 32), w.hi);
+    }
+    __device__ __forceinline__ void narrow(u64 y, const ulonglong2 w) {
+        const u32 y0 = (u32)y, y1 = (u32)(y >> 32), w0 = (u32)w.x, w1 = (u32)(w.x >> 32);
+        s = __fmaf_rn(__int2float_rn((int)__funnelshift_r(y0, y1, 14)), __uint_as_float((u32)w.y), s);
+        a = fq_madw(y0, w0, a);
+        a = ((u64)fq_madl(y0, w1, fq_madl(y1, w0, (u32)(a >> 32))) << 32) | (u32)a;
+    }
+    // the residue in [0, q): the sum is below 2^42 q (narrow; wide 2^35 q), so
+    // |ha| <= 2^20 is exact to 0.75, |P| <= 0.75 2^22 q + q and |t| < q
+    __device__ __forceinline__ u64 get(u64 q, const ModF &m) const;
+};
+
 // a signed value |v| < q to [0, q)
 __device__ __forceinline__ u64 fq_pos(u64 v, u64 q) { return v + ((u64)((i64)v >> 63) & q); }
+__device__ __forceinline__ u64 FqDot::get(u64 q, const ModF &m) const {
+    const u32 ha = __float_as_uint(s + FQ_MAGIC);
+    const u64 r = fq_madw(ha, (u32)m.nQ, a);
+    return fq_pos(fq_low((u32)r, fq_madl(ha, (u32)(m.nQ >> 32), (u32)(r >> 32)), m), q);
+}
 // any signed |v| <= 17.2 q to |result| <= 0.57 q
 __device__ __forceinline__ u64 fq_red(u64 v, const ModF &m) { return fq_low((u32)v, (u32)(v >> 32), m); }
 

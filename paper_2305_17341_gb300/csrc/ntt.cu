@@ -572,7 +572,7 @@ __device__ __forceinline__ void inv_tile(u64 (&x)[16], u64 *sm, const PassTw<LM,
 }
 
 template <int LM, int LS, bool ROWS, bool STG, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_ntt_inv_fast(u64 *data, RowMap rm, long nr, int items,
+__global__ void __launch_bounds__(256, MINB) k_ntt_inv_fast(u64 *data, RowMap rm, long nr, int items, NttSrc src,
                                                             const ModQ *mods, const ModF *modf,
                                                             const ulonglong2 *tw2, const u64 *ninv,
                                                             const ulonglong2 *ninvf, int logN) {
@@ -593,8 +593,13 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_inv_fast(u64 *data, RowMap rm
         STG ? stg + (ROWS ? (w % (G_::W / items)) * M : 0) : ROWS ? tab + 256 + pm.seq * M : tab, t};
     u64 x[16];
     if (ROWS) {
+        const u64 *in = p;
+        if (src.src) {
+            const u32 r = src.row0 + (u32)pm.row, it = r / (u32)src.rows_per_item;
+            in = src.src + it * src.stride + (long)(r - it * src.rows_per_item) * N + pm.seq * M;
+        }
 #pragma unroll
-        for (int k = 0; k < 16; k++) sm[G_::sidx(t + T * k, w)] = p[t + T * k];
+        for (int k = 0; k < 16; k++) sm[G_::sidx(t + T * k, w)] = in[t + T * k];
         if (STG) staged_wait();
         __syncthreads();
 #pragma unroll
@@ -674,12 +679,13 @@ static void fwd_pass(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st
 }
 
 template <int LM, int LS, bool ROWS, bool STG>
-static void inv_pass_launch(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st, int items, dim3 grid) {
+static void inv_pass_launch(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st, int items, dim3 grid,
+                            const NttSrc &src) {
     typedef PassGeom<LM, ROWS> G_;
     const size_t smem = G_::SM * 8 + (STG ? (ROWS ? G_::W / items : 1) * G_::M * 16 : 0);
     const int minb = pass_build(ctx, ctx->ntt_minb_inv, grid);
 #define INV_LAUNCH(MINB)                                                                                     \
-    pass_launch<k_ntt_inv_fast<LM, LS, ROWS, STG, MINB>>(ctx, grid, smem, st, d, m, nr, items,                 \
+    pass_launch<k_ntt_inv_fast<LM, LS, ROWS, STG, MINB>>(ctx, grid, smem, st, d, m, nr, items, src,            \
                 (const ModQ *)ctx->d_mod, (const ModF *)ctx->d_modf, (const ulonglong2 *)ctx->d_ipsi2,       \
                 (const u64 *)ctx->d_ninv, (const ulonglong2 *)ctx->d_ninvf, ctx->logN)
     if (minb == 3) INV_LAUNCH(3);
@@ -689,14 +695,14 @@ static void inv_pass_launch(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStre
 }
 
 template <int LM, int LS, bool ROWS>
-static void inv_pass(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st) {
+static void inv_pass(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st, const NttSrc &src = NttSrc()) {
     const int items = ROWS ? pass_items(m.n, nr) : 1;
     const dim3 grid = PassMap<LM, ROWS>::grid(ctx->N, m.n, nr, items);
     if constexpr (ROWS) {
-        if (pass_staged(ctx, items, grid)) inv_pass_launch<LM, LS, true, true>(ctx, d, nr, m, st, items, grid);
-        else inv_pass_launch<LM, LS, true, false>(ctx, d, nr, m, st, items, grid);
+        if (pass_staged(ctx, items, grid)) inv_pass_launch<LM, LS, true, true>(ctx, d, nr, m, st, items, grid, src);
+        else inv_pass_launch<LM, LS, true, false>(ctx, d, nr, m, st, items, grid, src);
     } else {
-        inv_pass_launch<LM, LS, false, true>(ctx, d, nr, m, st, items, grid);
+        inv_pass_launch<LM, LS, false, true>(ctx, d, nr, m, st, items, grid, src);
     }
 }
 
@@ -822,9 +828,9 @@ static void fwd_both(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st
     if (ctx->logN >= 15) fwd_pass<8, 0, true>(ctx, d, nr, m, st, sk, ep);
     else fwd_pass<7, 0, true>(ctx, d, nr, m, st, sk, ep);
 }
-static void inv_both(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st) {
-    if (ctx->logN >= 15) inv_pass<8, 0, true>(ctx, d, nr, m, st);
-    else inv_pass<7, 0, true>(ctx, d, nr, m, st);
+static void inv_both(Ctx *ctx, u64 *d, long nr, const RowMap &m, cudaStream_t st, const NttSrc &src = NttSrc()) {
+    if (ctx->logN >= 15) inv_pass<8, 0, true>(ctx, d, nr, m, st, src);
+    else inv_pass<7, 0, true>(ctx, d, nr, m, st, src);
     if (ctx->logN == 16) inv_pass<8, 8, false>(ctx, d, nr, m, st);
     else if (ctx->logN == 15) inv_pass<7, 8, false>(ctx, d, nr, m, st);
     else inv_pass<7, 7, false>(ctx, d, nr, m, st);
@@ -972,8 +978,14 @@ void ntt_fwd_subscale(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStre
     }
 }
 
-void ntt_inv(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStream_t st) {
+void ntt_inv(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStream_t st, const NttSrc &src) {
     if (rows <= 0) return;
+    if (src.src && (ctx->logN < 14 || ctx->logN > 16)) {   // the shared-memory passes work in place
+        launch_copy_rows(data, (long)src.rows_per_item * ctx->N, src.src, src.stride, (int)(rows / src.rows_per_item),
+                         (long)src.rows_per_item * ctx->N, st);
+        ntt_inv(ctx, data, rows, rm, st);
+        return;
+    }
     if (ctx->autotune && !ctx->ntt_tuned && ctx->logN >= 14 && ctx->logN <= 16) tune_ntt(ctx, st);
     int logN = ctx->logN, logN1, C, R;
     split(logN, logN1, C, R);
@@ -987,7 +999,13 @@ void ntt_inv(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStream_t st) 
         cudaEvent_t e0;
         ctx->trace_begin(2, e0);
         if (logN >= 14 && logN <= 16) {
-            inv_both(ctx, d, nr, m, st);
+            // a chunk starts at row r0: the item it lies in, and its row there
+            NttSrc s = src;
+            if (s.src) {
+                const long it = r0 / s.rows_per_item;
+                s.src += it * s.stride, s.row0 = (unsigned)(r0 - it * s.rows_per_item);
+            }
+            inv_both(ctx, d, nr, m, st, s);
             ctx->trace_end(2, e0, 2.0 * nr * ctx->N * 8.0);
             continue;
         }
