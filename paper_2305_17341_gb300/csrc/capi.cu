@@ -225,7 +225,7 @@ int he_ctx_destroy(he_ctx *ctx) {
     for (auto &kv : c.ptcache) cudaFree(kv.second);
     for (auto &kv : c.dcd)
         for (auto &f : kv.second.factors) cudaFree(f.dev);
-    void *ptrs[] = {c.d_mod, c.d_modf, c.d_ninvf, c.d_dn_Pinvf, c.d_dn_fq, c.d_psi, c.d_psip, c.d_ipsi, c.d_ipsip, c.d_psi2, c.d_ipsi2, c.d_ninv, c.d_dn_pinv,
+    void *ptrs[] = {c.d_mod, c.d_modf, c.d_ninvf, c.d_dn_Pinvf, c.d_dn_fq, c.d_sd_f, c.d_sd_s, c.d_psi, c.d_psip, c.d_ipsi, c.d_ipsip, c.d_psi2, c.d_ipsi2, c.d_ninv, c.d_dn_pinv,
                     c.d_dn_pmod,
                     c.d_dn_Pinv, c.d_Pmod, c.d_dn_E, c.d_zeta, c.d_slot_t, c.d_sk, c.d_skM,
                     c.d_pkM};
@@ -233,7 +233,7 @@ int he_ctx_destroy(he_ctx *ctx) {
         if (p) cudaFree(p);
     for (auto &l : c.lvl) {
         void *lp[] = {l.d_up_inv, l.d_up_mod, l.d_up_fq, l.d_rs_inv, l.d_rs_invf, l.d_rs_qlmod, l.d_mr_inv, l.d_mr_invf,
-                      l.d_mr_E};
+                      l.d_mr_E, l.d_su_f, l.d_su_s};
         for (void *p : lp)
             if (p) cudaFree(p);
     }

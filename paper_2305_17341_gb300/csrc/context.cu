@@ -339,6 +339,20 @@ const LevelConsts &Ctx::lc(int level) {
     LC.d_up_inv = upload(inv);
     LC.d_up_mod = upload(mod);
     LC.d_up_fq = upload(fq);
+    const int nq = level + 1;
+    std::vector<ulonglong2> suf((size_t)LC.ndig * alpha * 2 * nq);
+    std::vector<ShoupPair> sus(suf.size());
+    for (int d = 0; d < LC.ndig; d++)
+        for (int s = 0; s < std::min(alpha, nq - d * alpha); s++)
+            for (int r = 0; r < nq; r++)
+                for (int h = 0; h < 2; h++) {
+                    const u64 q = primes[r], w = mod[((size_t)d * alpha + s) * rows + r].w;
+                    const u64 v = h ? h_mulmod(w, ((u64)1 << 32) % q, q) : w;
+                    const size_t o = (((size_t)d * alpha + s) * 2 + h) * nq + r;
+                    suf[o] = h_fq(v, q), sus[o] = h_shoup(v, q);
+                }
+    LC.d_su_f = upload(suf);
+    LC.d_su_s = upload(sus);
     if (level > 0) {
         std::vector<ShoupPair> ri(level);
         std::vector<u64> rm(level);
@@ -512,6 +526,27 @@ void build_tables(Ctx *c) {
     for (int m = 0; m + 1 < a; m++) {
         for (int i = 0; i < 4; i++) mk.kP[m][i] = P4[i];
         limb_mul(mk.kP[m], 4, (u64)(m + 1));
+    }
+    {
+        std::vector<ulonglong2> sf((size_t)(2 * a + 2) * (L + 1));
+        std::vector<ShoupPair> ss(sf.size());
+        for (int r = 0; r <= L; r++) {
+            const u64 qr = c->primes[r], P = Pmod[r].w;
+            const u64 h = h_mulmod((P + qr - 1) % qr, h_invmod(2, qr), qr);
+            for (int w = 0; w < 2 * a + 2; w++) {
+                u64 v;
+                if (w < 2 * a) {
+                    v = pmod[(size_t)(w % a) * (L + 1) + r].w;
+                    if (w >= a) v = h_mulmod(v, ((u64)1 << 32) % qr, qr);
+                } else {
+                    v = w == 2 * a ? P : h;   // -e P, and -h per term
+                    v = v ? qr - v : 0;
+                }
+                sf[(size_t)w * (L + 1) + r] = h_fq(v, qr), ss[(size_t)w * (L + 1) + r] = h_shoup(v, qr);
+            }
+        }
+        c->d_sd_f = upload(sf);
+        c->d_sd_s = upload(ss);
     }
     std::vector<u64> E((size_t)a * (L + 1));
     for (int r = 0; r <= L; r++) {

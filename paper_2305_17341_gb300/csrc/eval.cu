@@ -3,6 +3,7 @@
 // ciphertexts laid out contiguously as [B][2][level+1][N] (NTT domain).
 #include <algorithm>
 #include <cmath>
+#include <memory>
 #include <sstream>
 
 #include "eval.h"
@@ -144,15 +145,6 @@ void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out) {
 void drop(Ctx *c, const u64 *in, int B, int level, int to, u64 *out) {
     const int N = c->N;
     launch_copy_rows(out, (long)(to + 1) * N, in, (long)(level + 1) * N, 2 * B, (long)(to + 1) * N, c->stream);
-}
-
-// out[p] = in[idx[p]] dropped from level to `to` (both polynomials).
-static void drop_gather(Ctx *c, const u64 *in, const int *idx, int P, int level, int to, u64 *out) {
-    const int N = c->N;
-    for (int p = 0; p < P; p++)
-        launch_copy_rows(out + (size_t)p * 2 * (to + 1) * N, (long)(to + 1) * N,
-                         in + (size_t)idx[p] * 2 * (level + 1) * N, (long)(level + 1) * N, 2, (long)(to + 1) * N,
-                         c->stream);
 }
 
 // out (holding (d0, d1)) += KeySwitch(d2, rlk): the relinearisation of Mult.
@@ -384,14 +376,13 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
     if (level < depth) throw HeError(HE_ERR_LEVEL, "matrix product needs more levels");
     if ((dcd_z && (dcd_z >= n || dcd_z % n1z)) || (dcd_t && (dcd_t >= n || dcd_t % n1t)))
         throw HeError(HE_ERR_ARG, "a decomposition needs n' < n with n1 dividing n'");
+    if (!c->rlk) throw HeError(HE_ERR_KEY_MISSING, "relinearisation key missing");
     const int N = c->N;
     const long n2m = (long)n * n;
     const int l1 = level - (depth - 2), l2 = l1 - 1;
     const size_t ct1 = (size_t)2 * (l1 + 1) * N, ct2 = (size_t)2 * (l2 + 1) * N;
     const int rows1 = c->qp_rows(l1);
     const size_t qp1 = (size_t)2 * rows1 * N, dig1 = (size_t)c->ndig(l1) * rows1 * N;
-    bool ident = nA == P && nB == P;
-    for (int p = 0; p < P && ident; p++) ident = ia[p] == p && ib[p] == p;
     for (int p = 0; p < P; p++)
         if (ia[p] < 0 || ia[p] >= nA || ib[p] < 0 || ib[p] >= nB) throw HeError(HE_ERR_ARG, "bad operand index");
     Buf A0(&c->pool, nA * ct1), B0(&c->pool, nB * ct1);
@@ -408,43 +399,55 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
     modup(c, Apg.p + (long)(l1 + 1) * N, (long)ct1, nA, l1, dAp.p);
     cudaMemcpyAsync(Bg.p, B0.p, nB * ct1 * 8, cudaMemcpyDeviceToDevice, c->stream);
     modup(c, Bg.p + (long)(l1 + 1) * N, (long)ct1, nB, l1, dB.p);
-    int gA = 0, gB = 0;
+    int gA = 0;
 
-    Buf acc(&c->pool, P * ct2), Ak(&c->pool, nA * ct2);
-    // the operands of every product, gathered when operands are shared
-    Buf AkP(&c->pool, ident ? 1 : P * ct2), BkP(&c->pool, ident ? 1 : P * ct2);
-    // relin_once: the summed d2 of the n tensors (d0, d1 are summed in acc)
-    Buf acc2(&c->pool, relin_once ? (size_t)P * (l2 + 1) * N : 1);
-    Buf R1(&c->pool, nA * qp1), R2(&c->pool, nA * qp1), S(&c->pool, nA * qp1);
-    RowMap q2 = c->map_q(l2);
-
-    // The babies of a source are all its hoisted rotations at once (one
-    // read of the source's digits per kMultSumMaxKeys keys):
-    //   C^k: rotations by b of A_g and A'_g kept in Q_l P, b = 1..n1z-1;
-    //   R^k: rotations by n b of B_g (ModDown'd), b = 1..n1t-1.
+    // Terms k run by run: kn consecutive k of one A giant and one B giant, all
+    // their ModDowns, rescales, tensors and key switches in one set of launches
+    // (SA, BB: slot b of a giant's baby b, slot 0 the giant itself).  A run holds
+    // kn P items; the bound keeps its temporaries in proportion to the batch's
+    // (64 items of N = 2^16 fill the GPU many times over).
     const int nbA = n1z - 1, nbB = n1t - 1;
-    Buf SA(&c->pool, (size_t)std::max(1, nbA) * nA * qp1);
-    Buf UB(&c->pool, (size_t)std::max(1, nbB) * nB * qp1), BB(&c->pool, (size_t)std::max(1, nbB) * nB * ct1);
-    // the babies of giant g, masked and summed in one pass:
-    // SA_b = m_k (.) rot_qp(A_g; b) + m'_k (.) rot_qp(A'_g; b), k = n1z g + b
-    auto babies_A = [&]() {
+    const int kmax = (int)std::max<long>(1, std::min<long>(n, (64L << 16) / ((long)std::max(P, std::max(nA, nB)) * N)));
+    const bool summed = c->logN >= 14 && c->logN <= 16;   // the register-blocked NTT's row layouts
+    Buf SA(&c->pool, (size_t)n1z * nA * qp1), BB(&c->pool, (size_t)n1t * nB * ct1);
+    Buf Ak(&c->pool, (size_t)std::min(kmax, n1z) * nA * ct2);
+    Buf acc(&c->pool, P * ct2), D2(&c->pool, (size_t)P * (l2 + 1) * N);
+    Buf d2(&c->pool, relin_once ? 1 : (size_t)std::min(kmax, n1z) * P * (l2 + 1) * N);
+    std::unique_ptr<RelinSum> sum;
+    if (!relin_once && summed) sum.reset(new RelinSum(c, P, l2));
+    // the giant's own sources, lifted to Q_l P, masked and summed (slot 0)
+    auto giant_A = [&]() {
+        const int k = n1z * gA;
+        if (k) {
+            Buf R1(&c->pool, nA * qp1), R2(&c->pool, nA * qp1);
+            launch_lift_P(c, R1.p, Ag.p, 2 * nA, l1, (long)(l1 + 1) * N, (long)rows1 * N, c->stream);
+            launch_lift_P(c, R2.p, Apg.p, 2 * nA, l1, (long)(l1 + 1) * N, (long)rows1 * N, c->stream);
+            const u64 *pts[2] = {get_pt(c, 3, n, 0, 0, 1.0, k, l1), get_pt(c, 4, n, 0, 0, 1.0, k, l1)};
+            const u64 *Rs[2] = {R1.p, R2.p};
+            launch_pmul_acc(c, SA.p, pts, Rs, 2, nA, l1, (long)qp1, c->stream);
+        }
+        if (nbA <= 0) return;
+        // the babies, masked and summed in one pass:
+        // SA_b = m_k (.) rot_qp(A_g; b) + m'_k (.) rot_qp(A'_g; b), k = n1z g + b
         std::vector<uint32_t> gs;
         std::vector<u64 *> o;
-        std::vector<const u64 *> m1, m2;
+        std::vector<const u64 *> m1, m2, keys;
         for (int b = 1; b <= nbA; b++) {
-            const int k = n1z * gA + b;
             gs.push_back(galois_of_step(c, b % n2m));
-            o.push_back(SA.p + (size_t)(b - 1) * nA * qp1);
-            m1.push_back(get_pt(c, 3, n, 0, 0, 1.0, k, l1));
-            m2.push_back(get_pt(c, 4, n, 0, 0, 1.0, k, l1));
+            o.push_back(SA.p + (size_t)b * nA * qp1);
+            m1.push_back(get_pt(c, 3, n, 0, 0, 1.0, k + b, l1));
+            m2.push_back(get_pt(c, 4, n, 0, 0, 1.0, k + b, l1));
+            keys.push_back(need_key(c, gs.back()));
         }
-        std::vector<const u64 *> keys(nbA);
-        for (int i = 0; i < nbA; i++) keys[i] = need_key(c, gs[i]);
         launch_multsum_ck(c, o.data(), dA.p, dAp.p, keys.data(), gs.data(), m1.data(), m2.data(), nbA, nA, l1,
                           Ag.p, Apg.p, (long)ct1, c->stream);
         c->n_ms += 2LL * nA * nbA;
     };
-    auto babies_B = [&]() {
+    // B_g in slot 0, its hoisted rotations by n b (ModDown'd) in the others
+    auto giant_B = [&]() {
+        cudaMemcpyAsync(BB.p, Bg.p, nB * ct1 * 8, cudaMemcpyDeviceToDevice, c->stream);
+        if (nbB <= 0) return;
+        Buf UB(&c->pool, (size_t)nbB * nB * qp1);
         std::vector<uint32_t> gs;
         std::vector<u64 *> o;
         for (int b = 1; b <= nbB; b++) {
@@ -452,17 +455,15 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
             o.push_back(UB.p + (size_t)(b - 1) * nB * qp1);
         }
         rot_qp_multi(c, Bg.p, nB, l1, dB.p, gs.data(), nbB, o.data());
-        if (nbB > 0) {
-            moddown(c, UB.p, 2 * nB * nbB, l1, BB.p, (long)(l1 + 1) * N);
-            c->n_md += (long long)nB * nbB;
-        }
+        moddown(c, UB.p, 2 * nB * nbB, l1, BB.p + nB * ct1, (long)(l1 + 1) * N);
+        c->n_md += (long long)nB * nbB;
     };
-    if (nbA > 0) babies_A();
-    if (nbB > 0) babies_B();
-    for (int k = 0; k < n; k++) {
-        // ---- A^(k) = C^k A^(0) at level l2
-        int g = k / n1z, b = k % n1z;
-        while (gA < g) {
+    giant_A();
+    giant_B();
+    for (int k = 0, kn; k < n; k += kn) {
+        const int b = k % n1z, bb = k % n1t;
+        kn = std::min(std::min(kmax, n - k), std::min(n1z - b, n1t - bb));
+        if (k && b == 0) {
             rotate_digits(c, Ag.p, nA, l1, dA.p, galois_of_step(c, n1z % n2m), tmpA.p);
             std::swap(Ag, tmpA);
             modup(c, Ag.p + (long)(l1 + 1) * N, (long)ct1, nA, l1, dA.p);
@@ -470,56 +471,32 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
             std::swap(Apg, tmpA);
             modup(c, Apg.p + (long)(l1 + 1) * N, (long)ct1, nA, l1, dAp.p);
             gA++;
-            if (nbA > 0) babies_A();
+            giant_A();
         }
-        if (k == 0) {
-            drop(c, A0.p, nA, l1, l2, Ak.p);
-        } else {
-            const u64 *Sk = S.p;
-            if (b > 0) {
-                Sk = SA.p + (size_t)(b - 1) * nA * qp1;
-            } else {
-                // the giant's own sources, lifted to Q_l P, masked and summed
-                launch_lift_P(c, R1.p, Ag.p, 2 * nA, l1, (long)(l1 + 1) * N, (long)rows1 * N, c->stream);
-                launch_lift_P(c, R2.p, Apg.p, 2 * nA, l1, (long)(l1 + 1) * N, (long)rows1 * N, c->stream);
-                const u64 *pts[2] = {get_pt(c, 3, n, 0, 0, 1.0, k, l1), get_pt(c, 4, n, 0, 0, 1.0, k, l1)};
-                const u64 *Rs[2] = {R1.p, R2.p};
-                launch_pmul_acc(c, S.p, pts, Rs, 2, nA, l1, (long)qp1, c->stream);
-            }
-            moddown_rescale(c, Sk, nA, l1, Ak.p);
-            c->n_md += nA;
-        }
-        // ---- B^(k) = R^k B^(0), dropped to l2
-        int gb2 = k / n1t, bb = k % n1t;
-        while (gB < gb2) {
+        if (k && bb == 0) {
             rotate_digits(c, Bg.p, nB, l1, dB.p, galois_of_step(c, ((long)n * n1t) % n2m), tmpB.p);
             std::swap(Bg, tmpB);
             modup(c, Bg.p + (long)(l1 + 1) * N, (long)ct1, nB, l1, dB.p);
-            gB++;
-            if (nbB > 0) babies_B();
+            giant_B();
         }
-        // B^(k) stays at level l1: the tensor reads its first l2 + 1 limbs
-        const u64 *bsrc = bb == 0 ? Bg.p : BB.p + (size_t)(bb - 1) * nB * ct1;
-        // ---- product, relinearised, accumulated at level l2
-        const u64 *xa = Ak.p, *xb = bsrc;
-        int b_level = l1;
-        if (!ident) {
-            for (int p = 0; p < P; p++) {
-                cudaMemcpyAsync(AkP.p + (size_t)p * ct2, Ak.p + (size_t)ia[p] * ct2, ct2 * 8,
-                                cudaMemcpyDeviceToDevice, c->stream);
-            }
-            drop_gather(c, bsrc, ib, P, l1, l2, BkP.p);
-            xa = AkP.p, xb = BkP.p, b_level = l2;
+        // ---- A^(k) = C^k A^(0) at level l2
+        const int k0 = k == 0 ? 1 : 0;   // A^(0) is A0 itself
+        if (k0) drop(c, A0.p, nA, l1, l2, Ak.p);
+        if (kn > k0) {
+            moddown_rescale(c, SA.p + (size_t)(b + k0) * nA * qp1, (kn - k0) * nA, l1, Ak.p + (size_t)k0 * nA * ct2);
+            c->n_md += (long long)(kn - k0) * nA;
         }
-        if (relin_once) {
-            const long cs = 2L * (l2 + 1) * N;
-            launch_tensor(c, acc.p, acc2.p, xa, xb, P, l2 + 1, cs, 2L * (b_level + 1) * N, q2, c->stream, k > 0,
-                          (long)(b_level + 1) * N);
-        } else {
-            mult_relin(c, xa, xb, P, l2, acc.p, k > 0, b_level);
-        }
+        // ---- products with B^(k) = R^k B^(0) (at level l1: the tensor reads its
+        // first l2 + 1 limbs), relinearised and accumulated at level l2
+        launch_tensor_run(c, acc.p, D2.p, relin_once ? nullptr : d2.p, Ak.p, BB.p + (size_t)bb * nB * ct1, kn, P, nA, nB, ia,
+                          ib, l2 + 1, (long)ct1, (long)(l1 + 1) * N, k > 0);
+        if (relin_once) continue;
+        if (summed) relin_sum_run(c, *sum, d2.p, kn);
+        else
+            for (int t = 0; t < kn; t++) relin_into(c, d2.p + (size_t)t * P * (l2 + 1) * N, P, l2, acc.p);
     }
-    if (relin_once) relin_into(c, acc2.p, P, l2, acc.p);
+    if (relin_once) relin_into(c, D2.p, P, l2, acc.p);
+    else if (summed) relin_sum_finish(c, *sum, D2.p, acc.p);
     rescale(c, acc.p, P, l2, out);
 }
 

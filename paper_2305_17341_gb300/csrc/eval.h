@@ -36,6 +36,16 @@ void drop(Ctx *c, const u64 *in, int B, int level, int to, u64 *out);
 // b may sit at a higher level b_level (its first level + 1 limbs are used in place)
 void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out, bool accumulate = false,
                 int b_level = -1);
+// Sum of relinearised terms (relin.cu): the integers of the runs so far.
+struct RelinSum {
+    int P, level, terms = 0;
+    Buf SY, YP;
+    RelinSum(Ctx *c, int P, int level);
+};
+void relin_sum_run(Ctx *c, RelinSum &S, u64 *d2, int K);
+void relin_sum_finish(Ctx *c, RelinSum &S, const u64 *D2, u64 *out);
+void launch_tensor_run(Ctx *c, u64 *d01, u64 *D2, u64 *d2, const u64 *a, const u64 *b, int K, int P, int nA, int nB,
+                       const int *ia, const int *ib, int limbs, long bs, long bp, bool accumulate);
 void add(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out);
 const u64 *get_pt(Ctx *c, int kind, int n, long t, long rot, double value, int k, int level,
                   const DcdFactor *fac = nullptr);

@@ -136,6 +136,10 @@ struct LevelConsts {
     ShoupPair *d_mr_inv = nullptr;     // [l]
     ulonglong2 *d_mr_invf = nullptr;   // [l]
     u64 *d_mr_E = nullptr;             // [2][alpha][l]
+    // summed key switch (relin.cu): weights of the low and high words of a
+    // digit's y on the Q rows, [ndig][alpha][low, high][l+1]
+    ulonglong2 *d_su_f = nullptr;
+    ShoupPair *d_su_s = nullptr;
 };
 
 // One factor of a Diagonal Convergence Decomposition (Sec. 4.2): the
@@ -182,6 +186,10 @@ struct Ctx {
     ShoupPair *d_Pmod = nullptr;     // [L+1]     P mod q_r
     FqPair *d_dn_fq = nullptr;       // [alpha+1][L+1] (P/p_j) mod q_r, then P mod q_r, for float-quotient rows
     u64 *d_dn_E = nullptr;           // [alpha][L+1] -(e P + (P-1)/2) mod q_r, e < alpha
+    // summed ModDown (relin.cu), [2 alpha + 2][L+1]: weights of the low and of
+    // the high words of y_j, of e and of the number of terms
+    ulonglong2 *d_sd_f = nullptr;
+    ShoupPair *d_sd_s = nullptr;
     MdExact md_exact;
     std::vector<LevelConsts> lvl;
 
@@ -361,9 +369,6 @@ void launch_automorph(Ctx *c, u64 *out, const u64 *in, long rows, const RowMap &
 // the tensor to what d01 and d2 already hold (acc01 / acc2 select the two
 // outputs separately when given).  b_poly_stride: words from b's first
 // polynomial to its second (0: limbs * N).
-void launch_tensor(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, long a_item_stride,
-                   long b_item_stride, const RowMap &rm, cudaStream_t st, bool accumulate = false,
-                   long b_poly_stride = 0);
 void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, long as, long bs,
                        const RowMap &rm, cudaStream_t st, bool acc01, bool acc2, long b_poly_stride = 0);
 // key switching pieces
@@ -392,6 +397,7 @@ void launch_multsum_multi(Ctx *c, u64 *const *outs, const u64 *digits, const u64
 void launch_multsum_ck(Ctx *c, u64 *const *outs, const u64 *dig1, const u64 *dig2, const u64 *const *keys,
                        const uint32_t *gs, const u64 *const *m1, const u64 *const *m2, int G, int B, int level,
                        const u64 *c01, const u64 *c02, long c0s, cudaStream_t st);
+void launch_multsum_q(Ctx *c, u64 *out, const u64 *digits, const u64 *key, int B, int level, cudaStream_t st);
 void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, cudaStream_t st);
 void launch_pmul_acc(Ctx *c, u64 *out, const u64 *const *pts, const u64 *const *R, int nterms, int B,
                      int level, long R_item_stride, cudaStream_t st);

@@ -11,6 +11,7 @@
 
 #include "bulkcopy.cuh"
 #include "he_internal.h"
+#include "kernels.cuh"
 
 namespace he {
 
@@ -332,13 +333,6 @@ __global__ void k_tensor(u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, i
     o[per] = v1;
     o2[0] = v2;
 }
-void launch_tensor(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, long as, long bs,
-                   const RowMap &rm, cudaStream_t st, bool accumulate, long bps) {
-    long n = (long)B * limbs * c->N;
-    c->n_launch++;
-    k_tensor<<<nblk(n, 256), 256, 0, st>>>(d01, d2, a, b, B, limbs, c->N, as, bs, bps ? bps : (long)limbs * c->N,
-                                           rm, c->d_mod, accumulate ? 3 : 0);
-}
 void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, long as, long bs,
                        const RowMap &rm, cudaStream_t st, bool acc01, bool acc2, long bps) {
     long n = (long)B * limbs * c->N;
@@ -589,43 +583,6 @@ void launch_centre_i64_q0(Ctx *c, const u64 *a, i64 *out, cudaStream_t st) {
 // every coefficient, so it is folded in here, before the forward NTT):
 // conv_r = sum_j y_j (P/p_j mod q_r) + E_{e,r} with E_{e,r} = -(e P + h) mod q_r.
 // pcoef: [items][A][N]; out: [items][l+1][N].
-
-// e = floor(S / P) for S = sum_j y[j] (P/p_j): S < A P < 2^(64 A).
-template <int A>
-__device__ __forceinline__ int md_overflow(const u64 (&y)[A], const MdExact &k) {
-    if constexpr (A == 1) {
-        return 0;
-    } else {
-        u64 s[A];
-#pragma unroll
-        for (int i = 0; i < A; i++) s[i] = 0;
-#pragma unroll
-        for (int j = 0; j < A; j++) {
-            u64 carry = 0;
-#pragma unroll
-            for (int i = 0; i < A - 1; i++) {
-                const u64 lo = y[j] * k.phat[j][i], hi = __umul64hi(y[j], k.phat[j][i]);
-                u64 t = s[i] + lo;
-                u64 cy = t < lo ? 1ull : 0ull;
-                t += carry;
-                cy += t < carry ? 1ull : 0ull;
-                s[i] = t;
-                carry = hi + cy;   // hi < 2^62
-            }
-            s[A - 1] += carry;     // the partial sums stay below S
-        }
-        int e = 0;
-#pragma unroll
-        for (int m = 0; m < A - 1; m++) {
-            int cmp = 0;
-#pragma unroll
-            for (int i = A - 1; i >= 0; i--)
-                if (cmp == 0) cmp = s[i] > k.kP[m][i] ? 1 : (s[i] < k.kP[m][i] ? -1 : 0);
-            e += cmp >= 0 ? 1 : 0;
-        }
-        return e;
-    }
-}
 
 // C adjacent coefficients per thread (2: 16-byte loads and stores, on
 // launches that fill the GPU; 1 on small ones), a grid stride over (item,
@@ -1395,6 +1352,23 @@ void launch_multsum_multi(Ctx *c, u64 *const *outs, const u64 *digits, const u64
         }
     }
     run(chunk, v, true);
+}
+
+// The inner product with one key on the rows of Q alone: digits [B][ndig][l+1][N]
+// -> out [B][2][l+1][N] (the key without permutation).
+void launch_multsum_q(Ctx *c, u64 *out, const u64 *digits, const u64 *key, int B, int level, cudaStream_t st) {
+    MultiKeys<1> mk;
+    mk.key[0] = key, mk.out[0] = out, mk.ginv[0] = 1;
+    int BI = 8;
+    while (BI > 1 && BI > B) BI >>= 1;
+    const int XW = 256 / BI, nq = level + 1, nd = c->ndig(level);
+    c->n_launch++;
+    cudaEvent_t e0;
+    c->trace_begin(0, e0);
+    k_multsum_vec<1, false, 5><<<dim3((unsigned)((c->N / 2 + XW - 1) / XW), (unsigned)nq, (unsigned)((B + BI - 1) / BI)),
+                                 256, 0, st>>>(mk, digits, B, BI, level, 0, c->L, nd, c->nprimes, c->logN, c->d_mod,
+                                               nullptr, 0, nullptr);
+    c->trace_end(0, e0, 8.0 * c->N * nq * (2.0 * nd + (double)B * (nd + 2)), (double)B * nd * nq * c->N * 2.0);
 }
 
 void launch_multsum(Ctx *c, u64 *out, const u64 *digits, const u64 *key, uint32_t g, int B, int level,
