@@ -255,8 +255,36 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
     R.emplace_back(&c->pool, B * qpct);
     launch_lift_P(c, R[0].p, in, 2 * B, level, (long)nq * N, (long)rows * N, c->stream);
     for (int j = 1; j < n1; j++) R.emplace_back(&c->pool, B * qpct);
-    Buf acc(&c->pool, B * qpct), S(&c->pool, B * qpct), ctmp(&c->pool, (size_t)B * 2 * nq * N),
-        dg2(&c->pool, (size_t)B * c->ndig(level) * rows * N), T(&c->pool, B * qpct);
+    // Giants i != 0 go in groups of G: their sums, ModDowns, Decomposes and
+    // rotations run as one batch of G B items, so that a few ciphertexts fill
+    // the GPU (one giant of one ciphertext at N = 2^15 leaves most of it idle).
+    // 16 items of N = 2^16 bound the digits' memory.
+    std::vector<int> giants;
+    std::vector<PmulTerm> terms;
+    std::vector<int> first(1, 0);
+    int i0 = -1;   // position of giant 0, which needs no rotation: it comes first
+    auto add_giant = [&](int i) {
+        const size_t n0 = terms.size();
+        for (int j = 0; j < n1; j++) {
+            long t = a * ((long)n1 * i + j);
+            if (fac ? !fac->diags.count(mod_pos(t, n2)) : !diag_nonzero(kind, n, t)) continue;
+            terms.push_back({get_pt(c, kind, n, t, mod_pos(-a * n1 * i, n2), value, 0, level, fac), j});
+        }
+        if (terms.size() == n0) return;
+        giants.push_back(i);
+        first.push_back((int)terms.size());
+    };
+    if (gi0 <= 0 && gi1 > 0) {
+        add_giant(0);
+        if (!giants.empty()) i0 = 0;
+    }
+    for (int i = gi0; i < gi1; i++)
+        if (i) add_giant(i);
+    const int ng = (int)giants.size(), nrot = ng - (i0 == 0 ? 1 : 0);
+    const int Gmax = std::min(nrot, (int)std::max<long>(1, std::min<long>(kMaxGiants, (16L << 16) / ((long)B * N))));
+    const size_t dgw = (size_t)B * c->ndig(level) * rows * N;
+    Buf acc(&c->pool, B * qpct), ctmp(&c->pool, std::max(1, Gmax) * (size_t)B * 2 * nq * N),
+        dg2(&c->pool, std::max(1, Gmax) * dgw), S(&c->pool, std::max(1, Gmax) * B * qpct);
     const int head = n1_sub > 1 && n1_sub < n1 ? n1_sub : n1;
     for (int j0 = 1, base = 0; j0 < n1; j0 += head - 1) {
         const u64 *src = in, *sdg = dg.p;
@@ -276,32 +304,27 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
         }
         rot_qp_multi(c, src, B, level, sdg, gs.data(), (int)gs.size(), outs.data());
     }
-    bool have = false;
-    RowMap qp = c->map_qp(level);
-    for (int i = gi0; i < gi1; i++) {
-        std::vector<const u64 *> pts, Rs;
-        for (int j = 0; j < n1; j++) {
-            long t = a * ((long)n1 * i + j);
-            if (fac ? !fac->diags.count(mod_pos(t, n2)) : !diag_nonzero(kind, n, t)) continue;
-            pts.push_back(get_pt(c, kind, n, t, mod_pos(-a * n1 * i, n2), value, 0, level, fac));
-            Rs.push_back(R[j].p);
+    std::vector<const u64 *> Rp;
+    for (auto &r : R) Rp.push_back(r.p);
+    if (i0 == 0) launch_pmul_sums(c, acc.p, (long)(B * qpct), terms.data(), first.data(), 1, Rp.data(), n1, B, level, (long)qpct, c->stream);
+    bool have = i0 == 0;
+    for (int p0 = have ? 1 : 0, G; p0 < ng; p0 += G) {
+        G = std::min(Gmax, ng - p0);
+        launch_pmul_sums(c, S.p, (long)(B * qpct), terms.data(), first.data() + p0, G, Rp.data(), n1, B, level, (long)qpct,
+                         c->stream);
+        moddown(c, S.p, 2 * B * G, level, ctmp.p, (long)nq * N);
+        c->n_md += (long long)B * G;
+        modup(c, ctmp.p + (long)nq * N, 2L * nq * N, B * G, level, dg2.p);
+        std::vector<const u64 *> keys;
+        std::vector<uint32_t> gs;
+        for (int t = 0; t < G; t++) {
+            gs.push_back(galois_of_step(c, mod_pos(a * n1 * giants[p0 + t], n2)));
+            keys.push_back(need_key(c, gs.back()));
         }
-        if (pts.empty()) continue;
-        launch_pmul_acc(c, S.p, pts.data(), Rs.data(), (int)pts.size(), B, level, (long)qpct, c->stream);
-        const u64 *term = S.p;
-        if (i != 0) {
-            moddown(c, S.p, 2 * B, level, ctmp.p, (long)nq * N);
-            c->n_md += B;
-            modup(c, ctmp.p + (long)nq * N, 2L * nq * N, B, level, dg2.p);
-            rot_qp(c, ctmp.p, B, level, dg2.p, galois_of_step(c, mod_pos(a * n1 * i, n2)), T.p);
-            term = T.p;
-        }
-        if (!have) {
-            cudaMemcpyAsync(acc.p, term, B * qpct * 8, cudaMemcpyDeviceToDevice, c->stream);
-            have = true;
-        } else {
-            launch_add(c, acc.p, acc.p, term, 2L * B * rows, qp, c->stream);
-        }
+        launch_multsum_giants(c, acc.p, have ? acc.p : nullptr, dg2.p, keys.data(), gs.data(), G, B, level, ctmp.p,
+                              2L * nq * N, c->stream);
+        c->n_ms += (long long)B * G;
+        have = true;
     }
     moddown_rescale(c, acc.p, B, level, out);
     c->n_md += B;
@@ -424,7 +447,9 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
             launch_lift_P(c, R2.p, Apg.p, 2 * nA, l1, (long)(l1 + 1) * N, (long)rows1 * N, c->stream);
             const u64 *pts[2] = {get_pt(c, 3, n, 0, 0, 1.0, k, l1), get_pt(c, 4, n, 0, 0, 1.0, k, l1)};
             const u64 *Rs[2] = {R1.p, R2.p};
-            launch_pmul_acc(c, SA.p, pts, Rs, 2, nA, l1, (long)qp1, c->stream);
+            const PmulTerm two[2] = {{pts[0], 0}, {pts[1], 1}};
+            const int range[2] = {0, 2};
+            launch_pmul_sums(c, SA.p, 0, two, range, 1, Rs, 2, nA, l1, (long)qp1, c->stream);
         }
         if (nbA <= 0) return;
         // the babies, masked and summed in one pass:

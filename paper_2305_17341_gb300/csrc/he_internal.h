@@ -399,8 +399,18 @@ void launch_multsum_ck(Ctx *c, u64 *const *outs, const u64 *dig1, const u64 *dig
                        const u64 *c01, const u64 *c02, long c0s, cudaStream_t st);
 void launch_multsum_q(Ctx *c, u64 *out, const u64 *digits, const u64 *key, int B, int level, cudaStream_t st);
 void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, cudaStream_t st);
-void launch_pmul_acc(Ctx *c, u64 *out, const u64 *const *pts, const u64 *const *R, int nterms, int B,
-                     int level, long R_item_stride, cudaStream_t st);
+// out[y] ([B][2][rows][N] at stride out_s) = sum of the terms first[y] .. first[y+1]
+// of pt (.) R[r], y < sums; at most 32 terms a sum, nR <= 32.
+struct PmulTerm {
+    const u64 *pt;
+    int r;
+};
+constexpr int kMaxPmulTerms = 256, kMaxPmulSums = 64;
+void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const int *first, int sums,
+                      const u64 *const *R, int nR, int B, int level, long Rs, cudaStream_t st);
+constexpr int kMaxGiants = 64;
+void launch_multsum_giants(Ctx *c, u64 *out, const u64 *in, const u64 *digits, const u64 *const *keys,
+                           const uint32_t *gs, int G, int B, int level, const u64 *c0, long c0s, cudaStream_t st);
 void launch_lift_P(Ctx *c, u64 *out_qp, const u64 *in_q, int items, int level, long in_item_stride,
                    long out_item_stride, cudaStream_t st);
 void launch_rescale_prep(Ctx *c, const u64 *lastcoef, u64 *out, int items, int level, cudaStream_t st);

@@ -1354,6 +1354,83 @@ void launch_multsum_multi(Ctx *c, u64 *const *outs, const u64 *digits, const u64
     run(chunk, v, true);
 }
 
+// MultSum + Permute of the G giants of a BSGS transform, summed: every giant
+// has its own digits, key and automorphism, and
+//   out[x] = in[x] + sum_g (T_g[y_g] + P c0_g[y_g]),  y_g = pi_g(x),
+// T_g as above (keys permuted).  A thread owns the output word, so the sum over
+// giants and digits is one accumulation with one reduction; the words of a
+// giant are read at permuted positions inside aligned 32-word blocks.  digits:
+// [G][B][ndig][rows][N]; c0: [G][B] ciphertexts at stride c0s; in (may be null, or
+// equal out), out: [B][2][rows][N].
+struct GiantArgs {
+    const u64 *key[kMaxGiants];
+    u32 g[kMaxGiants];
+};
+__global__ void __launch_bounds__(256, 4) k_multsum_giants(const __grid_constant__ GiantArgs ga, int G, u64 *out,
+                                                           const u64 *in, const u64 *digits, int B, int BI, int level,
+                                                           int alpha, int L, int ndig, int nprimes, int logN,
+                                                           const ModQ *mods, const u64 *c0, long c0s,
+                                                           const ShoupPair *Pmod) {
+    const int N = 1 << logN;
+    const int XW = 256 / BI;
+    const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
+    const int x = blockIdx.x * XW + tx;
+    const int r = blockIdx.y;
+    const int b = blockIdx.z * BI + ti;
+    if (b >= B || x >= N) return;
+    const int rows = level + 1 + alpha;
+    const int kr = r <= level ? r : L + 1 + (r - level - 1);
+    const ModQ m = mods[kr];
+    const long ds = (long)rows * N, kd = 2L * nprimes * N, kk = (long)nprimes * N;
+    const bool q_row = r <= level;
+    const ShoupPair w = q_row ? Pmod[r] : ShoupPair{0, 0};
+    u64 pc = 0;
+    U128 a0 = {0, 0}, a1 = {0, 0};
+    u32 x0 = 0, x1 = 0, x2 = 0, z0 = 0, z1 = 0, z2 = 0;
+    const bool small = m.q < (1ull << 42);   // uniform over the CTA; G ndig <= 2^12 products below 2^84
+    for (int g = 0; g < G; g++) {
+        const int y = auto_index(x, ga.g[g], logN);
+        const u64 *dp = digits + ((long)g * B + b) * ndig * ds + (long)r * N + y;
+        const u64 *kp = ga.key[g] + (long)kr * N + y;
+        if (small) {
+            for (int d = 0; d < ndig; d++) {
+                const u64 v = __ldg(dp + d * ds);
+                mac96(x0, x1, x2, v, __ldg(kp + d * kd));
+                mac96(z0, z1, z2, v, __ldg(kp + d * kd + kk));
+            }
+        } else {
+            for (int d = 0; d < ndig; d++) {
+                const u64 v = __ldg(dp + d * ds);
+                mac128_q(a0, v, __ldg(kp + d * kd), m.q);
+                mac128_q(a1, v, __ldg(kp + d * kd + kk), m.q);
+            }
+        }
+        if (q_row) pc = addmod(pc, shoup(c0[((long)g * B + b) * c0s + (long)r * N + y], w.w, w.wp, m.q), m.q);
+    }
+    if (small) a0 = U128{((u64)x1 << 32) | x0, x2}, a1 = U128{((u64)z1 << 32) | z0, z2};
+    u64 o0 = addmod(redc(a0.lo, a0.hi, m), pc, m.q), o1 = redc(a1.lo, a1.hi, m);
+    const long o = (long)b * 2 * ds + (long)r * N + x;
+    if (in) o0 = addmod(o0, in[o], m.q), o1 = addmod(o1, in[o + ds], m.q);
+    out[o] = o0;
+    out[o + ds] = o1;
+}
+void launch_multsum_giants(Ctx *c, u64 *out, const u64 *in, const u64 *digits, const u64 *const *keys,
+                           const uint32_t *gs, int G, int B, int level, const u64 *c0, long c0s, cudaStream_t st) {
+    GiantArgs ga;
+    for (int g = 0; g < G; g++) ga.key[g] = keys[g], ga.g[g] = gs[g];
+    int BI = 8;
+    while (BI > 1 && BI > B) BI >>= 1;
+    const int XW = 256 / BI, rows = level + 1 + c->alpha, nd = c->ndig(level);
+    c->n_launch++;
+    cudaEvent_t e0;
+    c->trace_begin(0, e0);
+    k_multsum_giants<<<dim3((unsigned)((c->N + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI)), 256, 0, st>>>(
+        ga, G, out, in, digits, B, BI, level, c->alpha, c->L, nd, c->nprimes, c->logN, c->d_mod, c0, c0s, c->d_Pmod);
+    const double W = 8.0 * c->N;
+    c->trace_end(0, e0, W * (G * 2.0 * nd * rows + (double)B * (G * ((double)nd * rows + level + 1) + (in ? 4.0 : 2.0) * rows)),
+                 (double)B * G * nd * rows * c->N * 2.0);
+}
+
 // The inner product with one key on the rows of Q alone: digits [B][ndig][l+1][N]
 // -> out [B][2][l+1][N] (the key without permutation).
 void launch_multsum_q(Ctx *c, u64 *out, const u64 *digits, const u64 *key, int B, int level, cudaStream_t st) {
@@ -1702,25 +1779,29 @@ void launch_multsum_ck(Ctx *c, u64 *const *outs, const u64 *dig1, const u64 *dig
 
 // ------------------------------------------------------ double hoisting
 // S[b][k][r][x] = sum_t ptM_t[r][x] * R_t[b][k][r][x] over Q_l P (one REDC).
-struct PtrList {
-    const u64 *p[32];
+// One launch for several sums over the same R (blockIdx.y: the sum): term t of
+// sum y is plaintext pt[t] times R[ri[t]], first[y] <= t < first[y + 1]; the R
+// words of a block of coefficients are read by all sums close together.  One
+// REDC per output word: up to 32 products below q^2 stay below q 2^64 for q <
+// 2^59; on wider rows (q_0, the special primes) the sum is kept below it term
+// by term (mac128_q).
+struct PmulArgs {
+    const u64 *pt[kMaxPmulTerms];
+    const u64 *R[32];
+    unsigned char ri[kMaxPmulTerms];
+    short first[kMaxPmulSums + 1];
 };
-// One REDC per output word: up to 32 products below q^2 stay below q 2^64
-// for q < 2^59; on wider rows (q_0, the special primes) the sum is kept
-// below it term by term (mac128_q).
-__global__ void k_pmul_acc(u64 *out, PtrList pts, PtrList R, int nterms, int B, int rows, int N, long Rs,
-                           RowMap qp, const ModQ *mods) {
-    long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    long per = (long)rows * N;
-    if (idx >= per) return;
-    int r = (int)(idx / N);
-    const ModQ m = mods[qp.at(r)];
-    const bool wide = m.q >= (1ull << 59);   // uniform over the CTA (128 | N)
+__global__ void __launch_bounds__(128) k_pmul_acc(u64 *out, long out_s, const __grid_constant__ PmulArgs pa, int B,
+                                                  int rows, int logN, long Rs, RowMap qp, const ModQ *mods) {
+    const long idx = (long)blockIdx.x * 128 + threadIdx.x, per = (long)rows << logN;   // 128 | N
+    const ModQ m = mods[qp.at32((unsigned)(idx >> logN))];
+    const bool wide = m.q >= (1ull << 59);   // uniform over the CTA
+    const int t0 = pa.first[blockIdx.y], t1 = pa.first[blockIdx.y + 1];
     for (int b = 0; b < B; b++) {
         U128 a0 = {0, 0}, a1 = {0, 0};
-        for (int t = 0; t < nterms; t++) {
-            const u64 pv = pts.p[t][idx];
-            const u64 *rb = R.p[t] + b * Rs;
+        for (int t = t0; t < t1; t++) {
+            const u64 pv = pa.pt[t][idx];
+            const u64 *rb = pa.R[pa.ri[t]] + b * Rs;
             if (wide) {
                 mac128_q(a0, pv, rb[idx], m.q);
                 mac128_q(a1, pv, rb[per + idx], m.q);
@@ -1729,19 +1810,25 @@ __global__ void k_pmul_acc(u64 *out, PtrList pts, PtrList R, int nterms, int B, 
                 mac128(a1, pv, rb[per + idx]);
             }
         }
-        u64 *ob = out + (long)b * 2 * per;
+        u64 *ob = out + blockIdx.y * out_s + (long)b * 2 * per;
         ob[idx] = redc(a0.lo, a0.hi, m);
         ob[per + idx] = redc(a1.lo, a1.hi, m);
     }
 }
-void launch_pmul_acc(Ctx *c, u64 *out, const u64 *const *pts, const u64 *const *R, int nterms, int B, int level,
-                     long Rs, cudaStream_t st) {
-    PtrList a, b;
-    for (int t = 0; t < nterms; t++) { a.p[t] = pts[t]; b.p[t] = R[t]; }
-    int rows = level + 1 + c->alpha;
-    long n = (long)rows * c->N;
-    c->n_launch++;
-    k_pmul_acc<<<nblk(n, 128), 128, 0, st>>>(out, a, b, nterms, B, rows, c->N, Rs, c->map_qp(level), c->d_mod);
+void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const int *first, int sums,
+                      const u64 *const *R, int nR, int B, int level, long Rs, cudaStream_t st) {
+    const int rows = level + 1 + c->alpha;
+    for (int y0 = 0, y1; y0 < sums; y0 = y1) {
+        PmulArgs a;
+        for (int j = 0; j < nR; j++) a.R[j] = R[j];
+        for (y1 = y0 + 1; y1 < sums && y1 - y0 < kMaxPmulSums && first[y1 + 1] - first[y0] <= kMaxPmulTerms;) y1++;
+        for (int y = y0; y <= y1; y++) a.first[y - y0] = (short)(first[y] - first[y0]);
+        for (int t = first[y0]; t < first[y1]; t++)
+            a.pt[t - first[y0]] = terms[t].pt, a.ri[t - first[y0]] = (unsigned char)terms[t].r;
+        c->n_launch++;
+        k_pmul_acc<<<dim3(nblk((long)rows * c->N, 128), (unsigned)(y1 - y0)), 128, 0, st>>>(
+            out + y0 * out_s, out_s, a, B, rows, c->logN, Rs, c->map_qp(level), c->d_mod);
+    }
 }
 
 // P * a over Q_l P: rows q_r get (P mod q_r) a_r, the p rows are zero.
