@@ -284,7 +284,11 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
     const int Gmax = std::min(nrot, (int)std::max<long>(1, std::min<long>(kMaxGiants, (16L << 16) / ((long)B * N))));
     const size_t dgw = (size_t)B * c->ndig(level) * rows * N;
     Buf acc(&c->pool, B * qpct), ctmp(&c->pool, std::max(1, Gmax) * (size_t)B * 2 * nq * N),
-        dg2(&c->pool, std::max(1, Gmax) * dgw), S(&c->pool, std::max(1, Gmax) * B * qpct);
+        dg2(&c->pool, std::max(1, Gmax) * dgw);
+    // the plaintext sums of up to 64 items of N = 2^16 at a time: more sums a launch
+    // share more of its reads of R
+    const int Smax = std::max(1, std::min(nrot, (int)std::max<long>(Gmax, (64L << 16) / ((long)B * N))));
+    Buf S(&c->pool, (size_t)Smax * B * qpct);
     const int head = n1_sub > 1 && n1_sub < n1 ? n1_sub : n1;
     for (int j0 = 1, base = 0; j0 < n1; j0 += head - 1) {
         const u64 *src = in, *sdg = dg.p;
@@ -308,11 +312,14 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
     for (auto &r : R) Rp.push_back(r.p);
     if (i0 == 0) launch_pmul_sums(c, acc.p, (long)(B * qpct), terms.data(), first.data(), 1, Rp.data(), n1, B, level, (long)qpct, c->stream);
     bool have = i0 == 0;
-    for (int p0 = have ? 1 : 0, G; p0 < ng; p0 += G) {
-        G = std::min(Gmax, ng - p0);
-        launch_pmul_sums(c, S.p, (long)(B * qpct), terms.data(), first.data() + p0, G, Rp.data(), n1, B, level, (long)qpct,
-                         c->stream);
-        moddown(c, S.p, 2 * B * G, level, ctmp.p, (long)nq * N);
+    for (int p0 = have ? 1 : 0, G, s0 = 0, s1 = 0; p0 < ng; p0 += G) {
+        if (p0 >= s1) {
+            s0 = p0, s1 = std::min(ng, p0 + Smax);
+            launch_pmul_sums(c, S.p, (long)(B * qpct), terms.data(), first.data() + s0, s1 - s0, Rp.data(), n1, B, level,
+                             (long)qpct, c->stream);
+        }
+        G = std::min(Gmax, s1 - p0);
+        moddown(c, S.p + (size_t)(p0 - s0) * B * qpct, 2 * B * G, level, ctmp.p, (long)nq * N);
         c->n_md += (long long)B * G;
         modup(c, ctmp.p + (long)nq * N, 2L * nq * N, B * G, level, dg2.p);
         std::vector<const u64 *> keys;

@@ -328,7 +328,7 @@ struct SubScale {
     const ShoupPair *w = nullptr;
     const ulonglong2 *wf = nullptr;   // the same constants for the float-quotient product
     int rows_per_item = 1;
-    long row0 = 0;   // absolute index of the launch's first row
+    unsigned row0 = 0;   // the launch's first row (counted from item 0)
     const u64 *add = nullptr;   // optional addend, laid out like out (item stride as)
     long as = 0;
 };

@@ -359,19 +359,28 @@ __device__ __forceinline__ void fwd_tile(u64 (&x)[16], u64 *sm, const PassTw<LM,
     __syncthreads();
     if (!on) return;
     if (ROWS && SUBSC) {
-        const long arow = ep.row0 + row;
-        const long it = arow / ep.rows_per_item;
-        const int r = (int)(arow - it * ep.rows_per_item);
+        const u32 arow = ep.row0 + (u32)row;
+        const u32 it = arow / (u32)ep.rows_per_item;
+        const int r = (int)(arow - it * (u32)ep.rows_per_item);
         const long off = (long)r * N + seq * M;
         const u64 *up = ep.u + it * ep.us + off;
         u64 *op = ep.out + it * ep.os + off;
-        const u64 *ap = ep.add ? ep.add + it * ep.as + off : nullptr;
+        // every operand before the first store: a load may not pass a store
+        // that could alias it, so interleaved they would be 16 memory latencies
 #pragma unroll
-        for (int k = 0; k < 16; k++) {
-            u64 o = subscale_value<AR>(ep, r, up[t + T * k], sm[G_::sidx(t + T * k, w)], q, wone, f);
-            if (ap) o = addmod(o, ap[t + T * k], q);
-            op[t + T * k] = o;
+        for (int k = 0; k < 16; k++) x[k] = up[t + T * k];
+#pragma unroll
+        for (int k = 0; k < 16; k++) x[k] = subscale_value<AR>(ep, r, x[k], sm[G_::sidx(t + T * k, w)], q, wone, f);
+        if (ep.add) {
+            const u64 *ap = ep.add + it * ep.as + off;
+            u64 y[16];
+#pragma unroll
+            for (int k = 0; k < 16; k++) y[k] = ap[t + T * k];
+#pragma unroll
+            for (int k = 0; k < 16; k++) x[k] = addmod(x[k], y[k], q);
         }
+#pragma unroll
+        for (int k = 0; k < 16; k++) op[t + T * k] = x[k];
         return;
     }
 #pragma unroll
@@ -470,8 +479,8 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_fwd_fast(u64 *data, RowMap rm
         // the epilogue's operands (this item's sequences of u, and of the
         // addend) are contiguous: have the copy engine bring them into L2
         // while the butterflies run, so the epilogue does not wait on DRAM
-        const long arow = ep.row0 + pm.row, it = arow / ep.rows_per_item;
-        const long off = (arow - it * ep.rows_per_item) * (long)N + pm.seq * M;
+        const u32 arow = ep.row0 + (u32)pm.row, it = arow / (u32)ep.rows_per_item;
+        const long off = (long)(arow - it * (u32)ep.rows_per_item) * N + pm.seq * M;
         const u32 bytes = (u32)(G_::W / items) * M * 8;
         bc_prefetch_l2(ep.u + it * ep.us + off, bytes);
         if (ep.add) bc_prefetch_l2(ep.add + it * ep.as + off, bytes);
@@ -964,8 +973,12 @@ void ntt_fwd_subscale(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStre
         long nr = rows - r0 < chunk ? rows - r0 : chunk;
         u64 *d = data + r0 * (long)ctx->N;
         RowMap m = rm.shifted(r0);
+        // the chunk's rows counted from the item it starts in
         SubScale e = ep;
-        e.row0 = ep.row0 + r0;
+        const long i0 = r0 / ep.rows_per_item;
+        e.u += i0 * ep.us, e.out += i0 * ep.os;
+        if (e.add) e.add += i0 * ep.as;
+        e.row0 = (unsigned)(r0 - i0 * ep.rows_per_item);
         ctx->n_launch += 2;
         cudaEvent_t e0;
         ctx->trace_begin(1, e0);
