@@ -73,6 +73,7 @@ __global__ void k_sample_small(i64 *out, int N, int kind, GaussT gt, u32 obj, u3
 }
 
 __global__ void k_small_to_rns(const i64 *x, u64 *out, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * N) return;
     long row = idx / N;
@@ -206,6 +207,7 @@ void launch_decode(Ctx *c, const double *coef, double scale, double *zre, double
     (void)m;
 
 __global__ void k_add(u64 *o, const u64 *a, const u64 *b, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
     EW_PROLOGUE
     o[idx] = addmod(a[idx], b[idx], m.q);
 }
@@ -308,6 +310,7 @@ void launch_automorph(Ctx *c, u64 *out, const u64 *in, long rows, const RowMap &
 // place, without a level-dropping copy).
 __global__ void k_tensor(u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, int N,
                          long as, long bs, long bps, RowMap rm, const ModQ *mods, int accumulate) {
+    pdl_trigger();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     long per = (long)limbs * N;
     if (idx >= (long)B * per) return;
@@ -390,6 +393,7 @@ __global__ void __launch_bounds__(256) k_modup_bconv(const u64 *coef, u64 *out, 
                                                      RowMap qp, const ModQ *mods, const ModF *modf,
                                                      const ShoupPair *up_inv, const ShoupPair *up_mod,
                                                      const FqPair *up_fq, const u64 *own_ntt, long own_s) {
+    pdl_trigger();
     __shared__ ShoupPair s_mod[A * 64];   // [s][r], rows <= 64
     __shared__ FqPair s_fq[A * 64];
     __shared__ ModF s_f[64];
@@ -602,6 +606,7 @@ __global__ void __launch_bounds__(256) k_moddown_bconv(const u64 *pcoef, u64 *ou
                                                        const ModF *modf, const ShoupPair *pmod, const FqPair *pfq,
                                                        const ShoupPair *Pmod, const ShoupPair *Pinv, const u64 *E,
                                                        int Es, const u64 *El, int L) {
+    pdl_trigger();
     constexpr int S = RS ? A + 1 : A;   // sources: y_j, then t
     __shared__ ShoupPair s_c[S * 64];
     __shared__ FqPair s_fq[S * 64];
@@ -776,6 +781,7 @@ __global__ void __launch_bounds__(256, OCC ? OCC : G <= 2 ? 4 : G <= 5 ? 2 : 1) 
                                                        int alpha, int L, int ndig, int nprimes, int logN,
                                                        const ModQ *mods, const u64 *c0, long c0s,
                                                        const ShoupPair *Pmod) {
+    pdl_trigger();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -866,6 +872,7 @@ __global__ void __launch_bounds__(256, OCC) k_multsum_vec(MultiKeys<G> mk, const
                                                           int alpha, int L, int ndig, int nprimes, int logN,
                                                           const ModQ *mods, const u64 *c0, long c0s,
                                                           const ShoupPair *Pmod) {
+    pdl_trigger();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -951,6 +958,7 @@ __global__ void __launch_bounds__(256, OCC) k_multsum_split(const __grid_constan
                                                             int alpha, int L, int ndig, int nprimes, int logN,
                                                             const ModQ *mods, const u64 *c0, long c0s,
                                                             const ShoupPair *Pmod) {
+    pdl_trigger();
     constexpr int NGRP = G / KG, BI = 8 / NGRP;
     const int N = 1 << logN;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1022,6 +1030,7 @@ __global__ void __launch_bounds__(256, OCC) k_multsum_splitv(const __grid_consta
                                                              const u64 *digits, int B, int level, int alpha, int L,
                                                              int ndig, int nprimes, int logN, const ModQ *mods,
                                                              const u64 *c0, long c0s, const ShoupPair *Pmod) {
+    pdl_trigger();
     constexpr int NGRP = G / KG, BI = 8 / NGRP;
     const int N = 1 << logN;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1371,6 +1380,7 @@ __global__ void __launch_bounds__(256, 4) k_multsum_giants(const __grid_constant
                                                            int alpha, int L, int ndig, int nprimes, int logN,
                                                            const ModQ *mods, const u64 *c0, long c0s,
                                                            const ShoupPair *Pmod) {
+    pdl_trigger();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -1476,6 +1486,7 @@ __global__ void __launch_bounds__(256, G <= 1 ? 4 : G <= 2 ? 3 : 2)
     k_multsum_ck(const __grid_constant__ CkArgs<G> ck, const u64 *dig1, const u64 *dig2, int B, int BI, int level,
                  int alpha, int L, int ndig, int nprimes, int logN, const ModQ *mods, const u64 *c01,
                  const u64 *c02, long c0s, const ShoupPair *Pmod) {
+    pdl_trigger();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -1565,6 +1576,7 @@ __global__ void __launch_bounds__(256, 3)
     k_multsum_cks(const __grid_constant__ CkArgs<G> ck, const u64 *dig1, const u64 *dig2, int B, int level,
                   int alpha, int L, int ndig, int nprimes, int logN, const ModQ *mods, const u64 *c01,
                   const u64 *c02, long c0s, const ShoupPair *Pmod) {
+    pdl_trigger();
     constexpr int BI = 8 / G;
     const int N = 1 << logN;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1825,6 +1837,7 @@ __device__ __forceinline__ void pmul_item(const PmulArgs &pa, int t0, int t1, lo
 }
 __global__ void __launch_bounds__(128) k_pmul_acc(u64 *out, long out_s, const __grid_constant__ PmulArgs pa, int B,
                                                   int rows, int logN, long Rs, RowMap qp, const ModQ *mods) {
+    pdl_trigger();
     const long idx = 2 * ((long)blockIdx.y * 128 + threadIdx.x), per = (long)rows << logN;   // 256 | N
     const ModQ m = mods[qp.at32((unsigned)(idx >> logN))];
     const int t0 = pa.first[blockIdx.x], t1 = pa.first[blockIdx.x + 1];
@@ -1854,6 +1867,7 @@ void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const
 // in: [items][l+1][N] (stride in_s), out: [items][l+1+alpha][N] (stride out_s)
 __global__ void k_lift_P(u64 *out, const u64 *in, int items, int level, int alpha, int N, long is, long os,
                          const ModQ *mods, const ShoupPair *Pmod) {
+    pdl_trigger();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     int rows = level + 1 + alpha;
     long per = (long)rows * N;
@@ -1881,6 +1895,7 @@ void launch_lift_P(Ctx *c, u64 *out_qp, const u64 *in_q, int items, int level, l
 // last: [items][N]; out: [items][l][N]
 __global__ void k_rescale_prep(const u64 *last, u64 *out, int items, int level, int logN, const ModQ *mods,
                                const ModF *modf, const u64 *qlmod) {
+    pdl_trigger();
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long)items << logN) return;
     const int N = 1 << logN, x = (int)(idx & (N - 1)), it = (int)(idx >> logN);

@@ -14,6 +14,15 @@ typedef unsigned long long u64;
 typedef long long i64;
 typedef unsigned int u32;
 
+// Programmatic dependent launch.  A kernel that calls pdl_trigger lets the next
+// kernel of the stream start as soon as all its own CTAs run, if that kernel
+// was launched for it (the NTT passes are): its CTAs take free SMs, form their
+// indexes and stage their tables, and pdl_wait holds them until every earlier
+// kernel has finished and its writes are visible.  Nothing that an earlier
+// kernel writes is touched before pdl_wait.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 struct ModQ {
     u64 q;       // the prime
     u64 qinv;    // -q^-1 mod 2^64 (Montgomery)

@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_fwd_fast(u64 *data, RowMap rm
     extern __shared__ __align__(16) u64 sm[];
     ulonglong2 *stg = (ulonglong2 *)(sm + G_::SM);
     const int N = 1 << logN;
+    pdl_trigger();
     const PassMap<LM, ROWS> pm(rm, nr, items, skip);
     // uniform over the CTA: a column CTA's row, or the first row of all items
     if (ROWS ? pm.row >= nr : !pm.on) return;
@@ -475,6 +476,7 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_fwd_fast(u64 *data, RowMap rm
     if (STG) stage_twiddles<LM, ROWS>(stg, tab, items);
     const PassTw<LM, ROWS, STG> tw{
         STG ? stg + (ROWS ? (w % (G_::W / items)) * M : 0) : ROWS ? tab + 256 + pm.seq * M : tab, t};
+    pdl_wait();
     if (ROWS && SUBSC && pm.on && threadIdx.x % (256 / items) == 0) {
         // the epilogue's operands (this item's sequences of u, and of the
         // addend) are contiguous: have the copy engine bring them into L2
@@ -590,6 +592,7 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_inv_fast(u64 *data, RowMap rm
     extern __shared__ __align__(16) u64 sm[];
     ulonglong2 *stg = (ulonglong2 *)(sm + G_::SM);
     const int N = 1 << logN;
+    pdl_trigger();
     const PassMap<LM, ROWS> pm(rm, nr, items, RowSkip());
     if (ROWS && pm.row >= nr) return;   // uniform over the CTA: the first row of all items
     const int t = pm.t, w = pm.w, pidx = pm.pidx;
@@ -601,6 +604,7 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_inv_fast(u64 *data, RowMap rm
     const PassTw<LM, ROWS, STG> tw{
         STG ? stg + (ROWS ? (w % (G_::W / items)) * M : 0) : ROWS ? tab + 256 + pm.seq * M : tab, t};
     u64 x[16];
+    pdl_wait();
     if (ROWS) {
         const u64 *in = p;
         if (src.src) {
@@ -646,7 +650,13 @@ static void pass_launch(const Ctx *ctx, dim3 grid, size_t smem, cudaStream_t st,
         cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
         raised[ctx->device & 63].store(true, std::memory_order_release);
     }
-    KERN<<<grid, 256, smem, st>>>(args...);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // pdl_wait
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid, cfg.blockDim = dim3(256), cfg.dynamicSmemBytes = smem, cfg.stream = st;
+    cfg.attrs = at, cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, KERN, args...);
 }
 
 template <int LM, int LS, bool ROWS, bool STG, bool SUB>

@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(256) k_tensor_run(u64 *d01, u64 *D2, u64 *d2, 
                                                     int P, int p0, int nA, int nB, int limbs, int logN, long bs,
                                                     long bp, const __grid_constant__ PairIdx ix, const ModQ *mods,
                                                     const ModF *modf, int accumulate) {
+    pdl_trigger();
     const long N = 1L << logN;
     const int x = 2 * (blockIdx.x * 256 + threadIdx.x);   // 256 | N / 2
     const int r = blockIdx.y, p = p0 + blockIdx.z;
@@ -136,6 +137,7 @@ template <int A>
 __global__ void __launch_bounds__(256) k_relin_up(const u64 *d2, u64 *SY, u64 *digP, int K, int P, int level, int ndig,
                                                   int logN, int Lp1, const ModQ *mods, const ShoupPair *up_inv,
                                                   const ShoupPair *up_mod, int accumulate) {
+    pdl_trigger();
     const int nq = level + 1, rows = nq + A, d = blockIdx.y, i0 = d * A, ns = min(A, nq - i0);
     const long N = 1L << logN;
     ShoupPair inv[A], wp[A][A];   // wp[s][j]: (Q_d / q_s) mod p_j
@@ -193,6 +195,7 @@ __global__ void __launch_bounds__(256) k_relin_up(const u64 *d2, u64 *SY, u64 *d
 template <int A>
 __global__ void __launch_bounds__(256, 4) k_relin_ms(u64 *u, const u64 *digP, const u64 *key, int items, int ndig,
                                                      int logN, int Lp1, int nprimes, const ModQ *mods) {
+    pdl_trigger();
     const long N = 1L << logN;
     const int tx = threadIdx.x & 31, ti = threadIdx.x >> 5;
     const int x = 2 * (blockIdx.x * 32 + tx), j = blockIdx.y;
@@ -221,6 +224,7 @@ __global__ void __launch_bounds__(256, 4) k_relin_ms(u64 *u, const u64 *digP, co
 template <int A>
 __global__ void __launch_bounds__(256) k_relin_down(const u64 *uP, u64 *YP, int K, int P, int logN,
                                                     const __grid_constant__ MdExact k, int accumulate) {
+    pdl_trigger();
     const long N = 1L << logN;
     const long idx = (long)blockIdx.x * 256 + threadIdx.x;   // (p, poly, x): 256 | N
     const long pp = idx >> logN;
@@ -287,6 +291,7 @@ template <int A>
 __global__ void __launch_bounds__(256) k_relin_up_fin(u64 *dig, const u64 *SY, const u64 *D2, int P, int level,
                                                       int ndig, int logN, const ulonglong2 *Wf, const ShoupPair *Ws,
                                                       const ModQ *mods, const ModF *modf) {
+    pdl_trigger();
     const int nq = level + 1, d = blockIdx.y, i0 = d * A, ns = min(A, nq - i0);
     const long N = 1L << logN, units = (long)P << logN;
     LinRows L = {};
@@ -314,6 +319,7 @@ template <int A>
 __global__ void __launch_bounds__(256) k_relin_down_fin(u64 *conv, const u64 *YP, int items, int K, int level, int logN,
                                                         int nt, const ulonglong2 *Wf, const ShoupPair *Ws,
                                                         const ModQ *mods, const ModF *modf) {
+    pdl_trigger();
     const int nq = level + 1;
     const long N = 1L << logN, units = (long)items << logN;
     LinRows L = {};
