@@ -305,6 +305,19 @@ int device_status(const Ctx *c);
         }                                                                            \
     } while (0)
 
+// Launches a kernel that calls pdl_wait so that it may start while the kernel
+// before it in the stream finishes (modarith.cuh).
+template <class... P, class... A>
+inline void launch_pdl(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid, cfg.blockDim = dim3(block), cfg.dynamicSmemBytes = smem, cfg.stream = st;
+    cfg.attrs = at, cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // host number theory
 u64 h_mulmod(u64 a, u64 b, u64 q);
 u64 h_powmod(u64 a, u64 e, u64 q);

@@ -55,6 +55,8 @@ struct GaussT {
 // kind 0: ternary from w0 mod 3 -> {0, 1, -1}; kind 1: discrete Gaussian by
 // inversion of the cumulative table T on r = (w1:w0) >> 1, sign = w2 bit 0.
 __global__ void k_sample_small(i64 *out, int N, int kind, GaussT gt, u32 obj, u32 tag, u32 k0, u32 k1) {
+    pdl_trigger();
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     u32 c[4] = {(u32)i, 0u, obj, tag};
@@ -74,6 +76,7 @@ __global__ void k_sample_small(i64 *out, int N, int kind, GaussT gt, u32 obj, u3
 
 __global__ void k_small_to_rns(const i64 *x, u64 *out, long rows, int N, RowMap rm, const ModQ *mods) {
     pdl_trigger();
+    pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * N) return;
     long row = idx / N;
@@ -93,14 +96,14 @@ void launch_sample_small(Ctx *c, i64 *out, int kind, uint32_t obj, uint32_t tag,
     GaussT gt;
     for (int k = 0; k < 20; k++) gt.T[k] = c->gauss_T[k];
     c->n_launch++;
-    k_sample_small<<<nblk(c->N, 256), 256, 0, st>>>(out, c->N, kind, gt, obj, tag, (u32)c->seed,
+    launch_pdl(k_sample_small, dim3(nblk(c->N, 256)), 256, 0, st, out, c->N, kind, gt, obj, tag, (u32)c->seed,
                                                    (u32)(c->seed >> 32));
 }
 
 void launch_small_to_rns(Ctx *c, const i64 *x, u64 *out, int rows, const RowMap &rm, cudaStream_t st) {
     long n = (long)rows * c->N;
     c->n_launch++;
-    k_small_to_rns<<<nblk(n, 256), 256, 0, st>>>(x, out, rows, c->N, rm, c->d_mod);
+    launch_pdl(k_small_to_rns, dim3(nblk(n, 256)), 256, 0, st, x, out, rows, c->N, rm, c->d_mod);
 }
 
 // ------------------------------------------------------ encode / decode
@@ -113,6 +116,8 @@ __device__ __forceinline__ int brev_bits(int x, int bits) { return (int)(__brev(
 
 __global__ void k_enc_permute(const double *zr, const double *zi, double *xr, double *xi, const int *slot_t,
                               int S, int logS) {
+    pdl_trigger();
+    pdl_wait();
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= S) return;
     int t = brev_bits(slot_t[j], logS);
@@ -121,6 +126,8 @@ __global__ void k_enc_permute(const double *zr, const double *zi, double *xr, do
 }
 
 __global__ void k_dft_pass(double *xr, double *xi, const double *zeta, int S, int len, int sign) {
+    pdl_trigger();
+    pdl_wait();
     int e = blockIdx.x * blockDim.x + threadIdx.x;
     int half = len >> 1;
     if (e >= S / 2) return;
@@ -139,6 +146,8 @@ __global__ void k_dft_pass(double *xr, double *xi, const double *zeta, int S, in
 }
 
 __global__ void k_enc_final(const double *xr, const double *xi, const double *zeta, double f, i64 *m, int S) {
+    pdl_trigger();
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S) return;
     double wr = zeta[2 * i], wi = -zeta[2 * i + 1];
@@ -152,6 +161,8 @@ __global__ void k_enc_final(const double *xr, const double *xi, const double *ze
 // length-S DFT with exponent +1, slot j = x[t(j)].
 __global__ void k_dec_twist(const double *coef, double scale, const double *zeta, double *xr, double *xi, int S,
                             int logS) {
+    pdl_trigger();
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= S) return;
     double ur = coef[i] / scale, ui = coef[i + S] / scale;
@@ -162,6 +173,8 @@ __global__ void k_dec_twist(const double *coef, double scale, const double *zeta
 }
 
 __global__ void k_dec_gather(const double *xr, const double *xi, const int *slot_t, double *zr, double *zi, int S) {
+    pdl_trigger();
+    pdl_wait();
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= S) return;
     zr[j] = xr[slot_t[j]];
@@ -173,14 +186,14 @@ void launch_encode(Ctx *c, const double *zre, const double *zim, double scale, i
     Buf tmp(&c->pool, (size_t)S), tmp2(&c->pool, (size_t)S);  // S doubles each
     double *xr = (double *)tmp.p, *xi = (double *)tmp2.p;
     c->n_launch++;
-    k_enc_permute<<<nblk(S, 256), 256, 0, st>>>(zre, zim, xr, xi, c->d_slot_t, S, logS);
+    launch_pdl(k_enc_permute, dim3(nblk(S, 256)), 256, 0, st, zre, zim, xr, xi, c->d_slot_t, S, logS);
     for (int len = 2; len <= S; len <<= 1) {
         c->n_launch++;
-        k_dft_pass<<<nblk(S / 2, 256), 256, 0, st>>>(xr, xi, c->d_zeta, S, len, -1);
+        launch_pdl(k_dft_pass, dim3(nblk(S / 2, 256)), 256, 0, st, xr, xi, c->d_zeta, S, len, -1);
     }
     double f = scale / (double)S;
     c->n_launch++;
-    k_enc_final<<<nblk(S, 256), 256, 0, st>>>(xr, xi, c->d_zeta, f, m_out, S);
+    launch_pdl(k_enc_final, dim3(nblk(S, 256)), 256, 0, st, xr, xi, c->d_zeta, f, m_out, S);
 }
 
 void launch_decode(Ctx *c, const double *coef, double scale, double *zre, double *zim, cudaStream_t st) {
@@ -189,13 +202,13 @@ void launch_decode(Ctx *c, const double *coef, double scale, double *zre, double
     Buf tmp2(&c->pool, (size_t)S);
     double *xr = (double *)tmp.p, *xi = (double *)tmp2.p;
     c->n_launch++;
-    k_dec_twist<<<nblk(S, 256), 256, 0, st>>>(coef, scale, c->d_zeta, xr, xi, S, logS);
+    launch_pdl(k_dec_twist, dim3(nblk(S, 256)), 256, 0, st, coef, scale, c->d_zeta, xr, xi, S, logS);
     for (int len = 2; len <= S; len <<= 1) {
         c->n_launch++;
-        k_dft_pass<<<nblk(S / 2, 256), 256, 0, st>>>(xr, xi, c->d_zeta, S, len, +1);
+        launch_pdl(k_dft_pass, dim3(nblk(S / 2, 256)), 256, 0, st, xr, xi, c->d_zeta, S, len, +1);
     }
     c->n_launch++;
-    k_dec_gather<<<nblk(S, 256), 256, 0, st>>>(xr, xi, c->d_slot_t, zre, zim, S);
+    launch_pdl(k_dec_gather, dim3(nblk(S, 256)), 256, 0, st, xr, xi, c->d_slot_t, zre, zim, S);
 }
 
 // ----------------------------------------------------------- elementwise
@@ -208,31 +221,44 @@ void launch_decode(Ctx *c, const double *coef, double scale, double *zre, double
 
 __global__ void k_add(u64 *o, const u64 *a, const u64 *b, long rows, int N, RowMap rm, const ModQ *mods) {
     pdl_trigger();
+    pdl_wait();
     EW_PROLOGUE
     o[idx] = addmod(a[idx], b[idx], m.q);
 }
 __global__ void k_sub(u64 *o, const u64 *a, const u64 *b, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     EW_PROLOGUE
     o[idx] = submod(a[idx], b[idx], m.q);
 }
 __global__ void k_neg(u64 *o, const u64 *a, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     EW_PROLOGUE
     u64 v = a[idx];
     o[idx] = v ? m.q - v : 0;
 }
 __global__ void k_mul(u64 *o, const u64 *a, const u64 *b, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     EW_PROLOGUE
     o[idx] = mulmod(a[idx], b[idx], m);
 }
 __global__ void k_mulM(u64 *o, const u64 *a, const u64 *bM, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     EW_PROLOGUE
     o[idx] = mulmont(a[idx], bM[idx], m);
 }
 __global__ void k_to_mont(u64 *o, const u64 *a, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     EW_PROLOGUE
     o[idx] = mulmont(a[idx], m.r2, m);  // a R^2 R^-1 = a R
 }
 __global__ void k_from_mont(u64 *o, const u64 *a, long rows, int N, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     EW_PROLOGUE
     o[idx] = redc(a[idx], 0, m);
 }
@@ -240,7 +266,7 @@ __global__ void k_from_mont(u64 *o, const u64 *a, long rows, int N, RowMap rm, c
 #define EW_LAUNCH(kern, ...)                                                         \
     do {                                                                             \
         long n__ = rows * (long)c->N;                                                \
-        if (n__ > 0) c->n_launch++, kern<<<nblk(n__, 256), 256, 0, st>>>(__VA_ARGS__, rows, c->N, rm, c->d_mod); \
+        if (n__ > 0) c->n_launch++, launch_pdl(kern, dim3(nblk(n__, 256)), 256, 0, st, __VA_ARGS__, rows, c->N, rm, c->d_mod); \
     } while (0)
 
 void launch_add(Ctx *c, u64 *out, const u64 *a, const u64 *b, long rows, const RowMap &rm, cudaStream_t st) {
@@ -311,6 +337,7 @@ void launch_automorph(Ctx *c, u64 *out, const u64 *in, long rows, const RowMap &
 __global__ void k_tensor(u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, int N,
                          long as, long bs, long bps, RowMap rm, const ModQ *mods, int accumulate) {
     pdl_trigger();
+    pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     long per = (long)limbs * N;
     if (idx >= (long)B * per) return;
@@ -340,7 +367,7 @@ void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, in
                        const RowMap &rm, cudaStream_t st, bool acc01, bool acc2, long bps) {
     long n = (long)B * limbs * c->N;
     c->n_launch++;
-    k_tensor<<<nblk(n, 256), 256, 0, st>>>(d01, d2, a, b, B, limbs, c->N, as, bs, bps ? bps : (long)limbs * c->N,
+    launch_pdl(k_tensor, dim3(nblk(n, 256)), 256, 0, st, d01, d2, a, b, B, limbs, c->N, as, bs, bps ? bps : (long)limbs * c->N,
                                            rm, c->d_mod, (acc01 ? 1 : 0) | (acc2 ? 2 : 0));
 }
 
@@ -394,6 +421,7 @@ __global__ void __launch_bounds__(256) k_modup_bconv(const u64 *coef, u64 *out, 
                                                      const ShoupPair *up_inv, const ShoupPair *up_mod,
                                                      const FqPair *up_fq, const u64 *own_ntt, long own_s) {
     pdl_trigger();
+    if (!up_fq) pdl_wait();   // constants that the caller uploaded in the stream
     __shared__ ShoupPair s_mod[A * 64];   // [s][r], rows <= 64
     __shared__ FqPair s_fq[A * 64];
     __shared__ ModF s_f[64];
@@ -419,6 +447,7 @@ __global__ void __launch_bounds__(256) k_modup_bconv(const u64 *coef, u64 *out, 
     for (int sd = 0; sd < A; sd++)
         if (sd < ns) inv[sd] = up_inv[d * A + sd], qs[sd] = mods[i0 + sd].q, narrow[sd] = qs[sd] < kNarrow;
     __syncthreads();
+    pdl_wait();
     const int per = N / C;
     const long units = (long)B * per;
     for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < units; idx += (long)gridDim.x * blockDim.x) {
@@ -495,9 +524,9 @@ static void modup_launch_a(Ctx *c, const u64 *coef, u64 *out, int B, int level, 
     const dim3 grid((unsigned)gx, (unsigned)nd);
     const RowMap qp = c->map_qp(level);
     if (wide)
-        k_modup_bconv<A, 2><<<grid, 256, 0, st>>>(coef, out, B, level, nd, c->N, qp, c->d_mod, c->d_modf, up_inv, up_mod, up_fq, own_ntt, own_s);
+        launch_pdl(k_modup_bconv<A, 2>, dim3(grid), 256, 0, st, coef, out, B, level, nd, c->N, qp, c->d_mod, c->d_modf, up_inv, up_mod, up_fq, own_ntt, own_s);
     else
-        k_modup_bconv<A, 1><<<grid, 256, 0, st>>>(coef, out, B, level, nd, c->N, qp, c->d_mod, c->d_modf, up_inv, up_mod, up_fq, own_ntt, own_s);
+        launch_pdl(k_modup_bconv<A, 1>, dim3(grid), 256, 0, st, coef, out, B, level, nd, c->N, qp, c->d_mod, c->d_modf, up_inv, up_mod, up_fq, own_ntt, own_s);
 }
 
 static void modup_launch(Ctx *c, const u64 *coef, u64 *out, int B, int level, int nd, const ShoupPair *up_inv,
@@ -537,6 +566,8 @@ struct ScalarList {
 };
 __global__ void k_scalar_mul_rows(u64 *o, const u64 *a, long rows, int rpi, int N, ScalarList s, RowMap rm,
                                   const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * (long)N) return;
     long row = idx / N;
@@ -549,9 +580,11 @@ void launch_scalar_mul_rows(Ctx *c, u64 *out, const u64 *a, long rows, int rpi, 
     for (int i = 0; i < rpi && i < 64; i++) s.w[i] = vals[i];
     long n = rows * (long)c->N;
     c->n_launch++;
-    k_scalar_mul_rows<<<nblk(n, 256), 256, 0, st>>>(out, a, rows, rpi, c->N, s, rm, c->d_mod);
+    launch_pdl(k_scalar_mul_rows, dim3(nblk(n, 256)), 256, 0, st, out, a, rows, rpi, c->N, s, rm, c->d_mod);
 }
 __global__ void k_scalar_add_rows(u64 *o, long rows, int N, ScalarList s, RowMap rm, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * (long)N) return;
     long row = idx / N;
@@ -563,10 +596,12 @@ void launch_scalar_add_rows(Ctx *c, u64 *data, long rows, const u64 *vals, const
     for (int i = 0; i < rows && i < 64; i++) s.w[i].w = vals[i];
     long n = rows * (long)c->N;
     c->n_launch++;
-    k_scalar_add_rows<<<nblk(n, 256), 256, 0, st>>>(data, rows, c->N, s, rm, c->d_mod);
+    launch_pdl(k_scalar_add_rows, dim3(nblk(n, 256)), 256, 0, st, data, rows, c->N, s, rm, c->d_mod);
 }
 // centred lift of a residue mod q_0 to a signed integer
 __global__ void k_centre_i64_q0(const u64 *a, i64 *out, int N, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= N) return;
     u64 q = mods[0].q, v = a[x];
@@ -574,7 +609,7 @@ __global__ void k_centre_i64_q0(const u64 *a, i64 *out, int N, const ModQ *mods)
 }
 void launch_centre_i64_q0(Ctx *c, const u64 *a, i64 *out, cudaStream_t st) {
     c->n_launch++;
-    k_centre_i64_q0<<<nblk(c->N, 256), 256, 0, st>>>(a, out, c->N, c->d_mod);
+    launch_pdl(k_centre_i64_q0, dim3(nblk(c->N, 256)), 256, 0, st, a, out, c->N, c->d_mod);
 }
 
 // ------------------------------------------------------------- ModDown
@@ -626,6 +661,7 @@ __global__ void __launch_bounds__(256) k_moddown_bconv(const u64 *pcoef, u64 *ou
     if (RS && threadIdx.x < A) s_El[threadIdx.x] = El[threadIdx.x * (L + 1) + level];
     const ShoupPair pil = RS ? Pinv[level] : ShoupPair{0, 0};
     __syncthreads();
+    pdl_wait();
     const int per = N / C;
     const long units = (long)items * per;
     // sum_j y_j w_jr + e for the first n sources
@@ -696,9 +732,9 @@ static void moddown_launch_a(Ctx *c, const u64 *pcoef, u64 *out, int items, int 
     const u64 *E = RS ? c->lc(level).d_mr_E : c->d_dn_E;
     const int Es = RS ? level : c->L + 1;
     if (wide)
-        k_moddown_bconv<A, 2, RS><<<grid, 256, 0, st>>>(pcoef, out, items, level, c->N, k, c->d_mod, c->d_modf, c->d_dn_pmod, c->d_dn_fq, c->d_Pmod, c->d_dn_Pinv, E, Es, c->d_dn_E, c->L);
+        launch_pdl(k_moddown_bconv<A, 2, RS>, dim3(grid), 256, 0, st, pcoef, out, items, level, c->N, k, c->d_mod, c->d_modf, c->d_dn_pmod, c->d_dn_fq, c->d_Pmod, c->d_dn_Pinv, E, Es, c->d_dn_E, c->L);
     else
-        k_moddown_bconv<A, 1, RS><<<grid, 256, 0, st>>>(pcoef, out, items, level, c->N, k, c->d_mod, c->d_modf, c->d_dn_pmod, c->d_dn_fq, c->d_Pmod, c->d_dn_Pinv, E, Es, c->d_dn_E, c->L);
+        launch_pdl(k_moddown_bconv<A, 1, RS>, dim3(grid), 256, 0, st, pcoef, out, items, level, c->N, k, c->d_mod, c->d_modf, c->d_dn_pmod, c->d_dn_fq, c->d_Pmod, c->d_dn_Pinv, E, Es, c->d_dn_E, c->L);
 }
 
 template <bool RS>
@@ -726,6 +762,8 @@ void launch_moddown_rescale_bconv(Ctx *c, const u64 *pcoef, u64 *out, int items,
 // out_r = (u_r - conv_r) P^-1 mod q_r (+ addend_r), NTT domain, r <= level.
 __global__ void k_moddown_final(u64 *out, const u64 *u, const u64 *conv, const u64 *add, int items, int level,
                                 int N, long us, long os, long as, const ModQ *mods, const ShoupPair *Pinv) {
+    pdl_trigger();
+    pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     long per = (long)(level + 1) * N;
     if (idx >= (long)items * per) return;
@@ -742,7 +780,7 @@ void launch_moddown_final(Ctx *c, u64 *out, const u64 *u, const u64 *conv, const
                           long us, long os, long as, cudaStream_t st) {
     long n = (long)items * (level + 1) * c->N;
     c->n_launch++;
-    k_moddown_final<<<nblk(n, 256), 256, 0, st>>>(out, u, conv, addend, items, level, c->N, us, os, as, c->d_mod,
+    launch_pdl(k_moddown_final, dim3(nblk(n, 256)), 256, 0, st, out, u, conv, addend, items, level, c->N, us, os, as, c->d_mod,
                                                   c->d_dn_Pinv);
 }
 
@@ -782,6 +820,7 @@ __global__ void __launch_bounds__(256, OCC ? OCC : G <= 2 ? 4 : G <= 5 ? 2 : 1) 
                                                        const ModQ *mods, const u64 *c0, long c0s,
                                                        const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -873,6 +912,7 @@ __global__ void __launch_bounds__(256, OCC) k_multsum_vec(MultiKeys<G> mk, const
                                                           const ModQ *mods, const u64 *c0, long c0s,
                                                           const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -959,6 +999,7 @@ __global__ void __launch_bounds__(256, OCC) k_multsum_split(const __grid_constan
                                                             const ModQ *mods, const u64 *c0, long c0s,
                                                             const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     constexpr int NGRP = G / KG, BI = 8 / NGRP;
     const int N = 1 << logN;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1031,6 +1072,7 @@ __global__ void __launch_bounds__(256, OCC) k_multsum_splitv(const __grid_consta
                                                              int ndig, int nprimes, int logN, const ModQ *mods,
                                                              const u64 *c0, long c0s, const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     constexpr int NGRP = G / KG, BI = 8 / NGRP;
     const int N = 1 << logN;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1183,11 +1225,11 @@ static void multsum_launch_g(Ctx *c, int v, u64 *const *outs, const u64 *digits,
             const int rows = level + 1 + c->alpha, XW = 256 / BI;
             dim3 grid((unsigned)((c->N / 2 + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI));
             if (stream)
-                k_multsum_vec<G, true, OCCV><<<grid, 256, 0, st>>>(mk, digits, B, BI, level, c->alpha, c->L,
+                launch_pdl(k_multsum_vec<G, true, OCCV>, dim3(grid), 256, 0, st, mk, digits, B, BI, level, c->alpha, c->L,
                                                                    c->ndig(level), c->nprimes, c->logN, c->d_mod, c0,
                                                                    c0s, c->d_Pmod);
             else
-                k_multsum_vec<G, false, OCCV><<<grid, 256, 0, st>>>(mk, digits, B, BI, level, c->alpha, c->L,
+                launch_pdl(k_multsum_vec<G, false, OCCV>, dim3(grid), 256, 0, st, mk, digits, B, BI, level, c->alpha, c->L,
                                                                     c->ndig(level), c->nprimes, c->logN, c->d_mod, c0,
                                                                     c0s, c->d_Pmod);
             c->n_launch++;
@@ -1200,7 +1242,7 @@ static void multsum_launch_g(Ctx *c, int v, u64 *const *outs, const u64 *digits,
         const int rows = level + 1 + c->alpha;
         auto go = [&](auto kern, int bi) {
             dim3 grid((unsigned)((c->N / 2 + 31) / 32), (unsigned)rows, (unsigned)((B + bi - 1) / bi));
-            kern<<<grid, 256, 0, st>>>(mk, digits, B, level, c->alpha, c->L, c->ndig(level), c->nprimes, c->logN,
+            launch_pdl(kern, grid, 256, 0, st, mk, digits, B, level, c->alpha, c->L, c->ndig(level), c->nprimes, c->logN,
                                        c->d_mod, c0, c0s, c->d_Pmod);
         };
         if (v == 97 && G % 2 == 0 && G >= 2) {
@@ -1225,7 +1267,7 @@ static void multsum_launch_g(Ctx *c, int v, u64 *const *outs, const u64 *digits,
         const int rows = level + 1 + c->alpha;
         auto go = [&](auto kern, int bi) {
             dim3 grid((unsigned)((c->N + 31) / 32), (unsigned)rows, (unsigned)((B + bi - 1) / bi));
-            kern<<<grid, 256, 0, st>>>(mk, digits, B, level, c->alpha, c->L, c->ndig(level), c->nprimes, c->logN,
+            launch_pdl(kern, grid, 256, 0, st, mk, digits, B, level, c->alpha, c->L, c->ndig(level), c->nprimes, c->logN,
                                        c->d_mod, c0, c0s, c->d_Pmod);
         };
         if (v == 65 && G % 2 == 0 && G >= 2) {
@@ -1261,7 +1303,7 @@ static void multsum_launch_g(Ctx *c, int v, u64 *const *outs, const u64 *digits,
     constexpr int OCC_HI = G <= 1 ? 8 : G <= 2 ? 6 : G <= 4 ? 4 : 3;
     const bool hi = (v & 32) != 0;
 #define MS_LAUNCH(STR, PFD, OCC)                                                                           \
-    k_multsum_multi<G, STR, PFD, OCC><<<grid, 256, 0, st>>>(mk, digits, B, BI, level, c->alpha, c->L,          \
+    launch_pdl(k_multsum_multi<G, STR, PFD, OCC>, dim3(grid), 256, 0, st, mk, digits, B, BI, level, c->alpha, c->L,          \
                                                             c->ndig(level), c->nprimes, c->logN, c->d_mod, c0, c0s, \
                                                             c->d_Pmod)
     if (hi) {
@@ -1381,6 +1423,7 @@ __global__ void __launch_bounds__(256, 4) k_multsum_giants(const __grid_constant
                                                            const ModQ *mods, const u64 *c0, long c0s,
                                                            const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -1434,7 +1477,7 @@ void launch_multsum_giants(Ctx *c, u64 *out, const u64 *in, const u64 *digits, c
     c->n_launch++;
     cudaEvent_t e0;
     c->trace_begin(0, e0);
-    k_multsum_giants<<<dim3((unsigned)((c->N + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI)), 256, 0, st>>>(
+    launch_pdl(k_multsum_giants, dim3((unsigned)((c->N + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI)), 256, 0, st, 
         ga, G, out, in, digits, B, BI, level, c->alpha, c->L, nd, c->nprimes, c->logN, c->d_mod, c0, c0s, c->d_Pmod);
     const double W = 8.0 * c->N;
     c->trace_end(0, e0, W * (G * 2.0 * nd * rows + (double)B * (G * ((double)nd * rows + level + 1) + (in ? 4.0 : 2.0) * rows)),
@@ -1452,8 +1495,7 @@ void launch_multsum_q(Ctx *c, u64 *out, const u64 *digits, const u64 *key, int B
     c->n_launch++;
     cudaEvent_t e0;
     c->trace_begin(0, e0);
-    k_multsum_vec<1, false, 5><<<dim3((unsigned)((c->N / 2 + XW - 1) / XW), (unsigned)nq, (unsigned)((B + BI - 1) / BI)),
-                                 256, 0, st>>>(mk, digits, B, BI, level, 0, c->L, nd, c->nprimes, c->logN, c->d_mod,
+    launch_pdl(k_multsum_vec<1, false, 5>, dim3((unsigned)((c->N / 2 + XW - 1) / XW), (unsigned)nq, (unsigned)((B + BI - 1) / BI)), 256, 0, st, mk, digits, B, BI, level, 0, c->L, nd, c->nprimes, c->logN, c->d_mod,
                                                nullptr, 0, nullptr);
     c->trace_end(0, e0, 8.0 * c->N * nq * (2.0 * nd + (double)B * (nd + 2)), (double)B * nd * nq * c->N * 2.0);
 }
@@ -1487,6 +1529,7 @@ __global__ void __launch_bounds__(256, G <= 1 ? 4 : G <= 2 ? 3 : 2)
                  int alpha, int L, int ndig, int nprimes, int logN, const ModQ *mods, const u64 *c01,
                  const u64 *c02, long c0s, const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     const int N = 1 << logN;
     const int XW = 256 / BI;
     const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
@@ -1577,6 +1620,7 @@ __global__ void __launch_bounds__(256, 3)
                   int alpha, int L, int ndig, int nprimes, int logN, const ModQ *mods, const u64 *c01,
                   const u64 *c02, long c0s, const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     constexpr int BI = 8 / G;
     const int N = 1 << logN;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1690,7 +1734,7 @@ static void multsum_ck_launch_g(Ctx *c, int BI, u64 *const *outs, const u64 *dig
             const unsigned xblocks = (unsigned)((c->N / 2 + 31) / 32);
             const dim3 grid = SBI == 1 ? dim3(xblocks * (unsigned)B, (unsigned)rows, 1)
                                        : dim3(xblocks, (unsigned)rows, (unsigned)((B + SBI - 1) / SBI));
-            k_multsum_cks<G><<<grid, 256, 0, st>>>(ck, dig1, dig2, B, level, c->alpha, c->L, c->ndig(level),
+            launch_pdl(k_multsum_cks<G>, dim3(grid), 256, 0, st, ck, dig1, dig2, B, level, c->alpha, c->L, c->ndig(level),
                                                    c->nprimes, c->logN, c->d_mod, c01, c02, c0s, c->d_Pmod);
             c->n_launch++;
             return;
@@ -1700,7 +1744,7 @@ static void multsum_ck_launch_g(Ctx *c, int BI, u64 *const *outs, const u64 *dig
         if (BI == 0) BI = 8;   // G does not divide the warps
         const int XW = 256 / BI;
         dim3 grid((unsigned)((c->N + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI));
-        k_multsum_ck<G><<<grid, 256, 0, st>>>(ck, dig1, dig2, B, BI, level, c->alpha, c->L, c->ndig(level),
+        launch_pdl(k_multsum_ck<G>, dim3(grid), 256, 0, st, ck, dig1, dig2, B, BI, level, c->alpha, c->L, c->ndig(level),
                                               c->nprimes, c->logN, c->d_mod, c01, c02, c0s, c->d_Pmod);
         c->n_launch++;
     }
@@ -1838,6 +1882,7 @@ __device__ __forceinline__ void pmul_item(const PmulArgs &pa, int t0, int t1, lo
 __global__ void __launch_bounds__(128) k_pmul_acc(u64 *out, long out_s, const __grid_constant__ PmulArgs pa, int B,
                                                   int rows, int logN, long Rs, RowMap qp, const ModQ *mods) {
     pdl_trigger();
+    pdl_wait();
     const long idx = 2 * ((long)blockIdx.y * 128 + threadIdx.x), per = (long)rows << logN;   // 256 | N
     const ModQ m = mods[qp.at32((unsigned)(idx >> logN))];
     const int t0 = pa.first[blockIdx.x], t1 = pa.first[blockIdx.x + 1];
@@ -1858,7 +1903,7 @@ void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const
         for (int t = first[y0]; t < first[y1]; t++)
             a.pt[t - first[y0]] = terms[t].pt, a.ri[t - first[y0]] = (unsigned char)terms[t].r;
         c->n_launch++;
-        k_pmul_acc<<<dim3((unsigned)(y1 - y0), (unsigned)((long)rows * c->N / 256)), 128, 0, st>>>(
+        launch_pdl(k_pmul_acc, dim3((unsigned)(y1 - y0), (unsigned)((long)rows * c->N / 256)), 128, 0, st, 
             out + y0 * out_s, out_s, a, B, rows, c->logN, Rs, c->map_qp(level), c->d_mod);
     }
 }
@@ -1868,6 +1913,7 @@ void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const
 __global__ void k_lift_P(u64 *out, const u64 *in, int items, int level, int alpha, int N, long is, long os,
                          const ModQ *mods, const ShoupPair *Pmod) {
     pdl_trigger();
+    pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     int rows = level + 1 + alpha;
     long per = (long)rows * N;
@@ -1885,7 +1931,7 @@ __global__ void k_lift_P(u64 *out, const u64 *in, int items, int level, int alph
 void launch_lift_P(Ctx *c, u64 *out_qp, const u64 *in_q, int items, int level, long is, long os, cudaStream_t st) {
     long n = (long)items * (level + 1 + c->alpha) * c->N;
     c->n_launch++;
-    k_lift_P<<<nblk(n, 256), 256, 0, st>>>(out_qp, in_q, items, level, c->alpha, c->N, is, os, c->d_mod,
+    launch_pdl(k_lift_P, dim3(nblk(n, 256)), 256, 0, st, out_qp, in_q, items, level, c->alpha, c->N, is, os, c->d_mod,
                                            c->d_Pmod);
 }
 
@@ -1896,6 +1942,7 @@ void launch_lift_P(Ctx *c, u64 *out_qp, const u64 *in_q, int items, int level, l
 __global__ void k_rescale_prep(const u64 *last, u64 *out, int items, int level, int logN, const ModQ *mods,
                                const ModF *modf, const u64 *qlmod) {
     pdl_trigger();
+    pdl_wait();
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long)items << logN) return;
     const int N = 1 << logN, x = (int)(idx & (N - 1)), it = (int)(idx >> logN);
@@ -1921,13 +1968,15 @@ void launch_rescale_prep(Ctx *c, const u64 *lastcoef, u64 *out, int items, int l
     const LevelConsts &L = c->lc(level);
     long n = (long)items * c->N;
     c->n_launch++;
-    k_rescale_prep<<<nblk(n, 256), 256, 0, st>>>(lastcoef, out, items, level, c->logN, c->d_mod, c->d_modf, L.d_rs_qlmod);
+    launch_pdl(k_rescale_prep, dim3(nblk(n, 256)), 256, 0, st, lastcoef, out, items, level, c->logN, c->d_mod, c->d_modf, L.d_rs_qlmod);
 }
 
 // out_i = (c_i - t_i) q_l^-1 mod q_i (NTT domain), i < l.
 // in: [items][l+1][N] stride is; t: [items][l][N]; out: [items][l][N] stride os
 __global__ void k_rescale_final(u64 *out, const u64 *in, const u64 *t, int items, int level, int N, long is, long os,
                                 const ModQ *mods, const ShoupPair *inv) {
+    pdl_trigger();
+    pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     long per = (long)level * N;
     if (idx >= (long)items * per) return;
@@ -1943,18 +1992,22 @@ void launch_rescale_final(Ctx *c, u64 *out, const u64 *in, const u64 *t, int ite
     const LevelConsts &L = c->lc(level);
     long n = (long)items * level * c->N;
     c->n_launch++;
-    k_rescale_final<<<nblk(n, 256), 256, 0, st>>>(out, in, t, items, level, c->N, is, os, c->d_mod, L.d_rs_inv);
+    launch_pdl(k_rescale_final, dim3(nblk(n, 256)), 256, 0, st, out, in, t, items, level, c->N, is, os, c->d_mod, L.d_rs_inv);
 }
 
 // ------------------------------------------------------------- decrypt
 // m = c0 + c1 s on limb q_0 (NTT domain), written into out (u64 view).
 __global__ void k_dec_q0(const u64 *c0, const u64 *c1, const u64 *skM, u64 *out, int N, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= N) return;
     const ModQ &m = mods[0];
     out[x] = addmod(c0[x], mulmont(c1[x], skM[x], m), m.q);
 }
 __global__ void k_centre_q0(const u64 *a, double *out, int N, const ModQ *mods) {
+    pdl_trigger();
+    pdl_wait();
     int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= N) return;
     u64 q = mods[0].q, v = a[x];
@@ -2011,10 +2064,10 @@ void launch_copy_rows(u64 *dst, long dst_stride, const u64 *src, long src_stride
 namespace he {
 void launch_dec_q0(Ctx *c, const u64 *c0, const u64 *c1, u64 *out, cudaStream_t st) {
     c->n_launch++;
-    k_dec_q0<<<nblk(c->N, 256), 256, 0, st>>>(c0, c1, c->d_skM, out, c->N, c->d_mod);
+    launch_pdl(k_dec_q0, dim3(nblk(c->N, 256)), 256, 0, st, c0, c1, c->d_skM, out, c->N, c->d_mod);
 }
 void launch_centre_q0(Ctx *c, const u64 *a, double *out, cudaStream_t st) {
     c->n_launch++;
-    k_centre_q0<<<nblk(c->N, 256), 256, 0, st>>>(a, out, c->N, c->d_mod);
+    launch_pdl(k_centre_q0, dim3(nblk(c->N, 256)), 256, 0, st, a, out, c->N, c->d_mod);
 }
 }  // namespace he

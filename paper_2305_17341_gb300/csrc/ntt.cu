@@ -650,13 +650,7 @@ static void pass_launch(const Ctx *ctx, dim3 grid, size_t smem, cudaStream_t st,
         cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
         raised[ctx->device & 63].store(true, std::memory_order_release);
     }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // pdl_wait
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = grid, cfg.blockDim = dim3(256), cfg.dynamicSmemBytes = smem, cfg.stream = st;
-    cfg.attrs = at, cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, KERN, args...);
+    launch_pdl(KERN, grid, 256, smem, st, args...);
 }
 
 template <int LM, int LS, bool ROWS, bool STG, bool SUB>

@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(256) k_tensor_run(u64 *d01, u64 *D2, u64 *d2, 
                                                     long bp, const __grid_constant__ PairIdx ix, const ModQ *mods,
                                                     const ModF *modf, int accumulate) {
     pdl_trigger();
+    pdl_wait();
     const long N = 1L << logN;
     const int x = 2 * (blockIdx.x * 256 + threadIdx.x);   // 256 | N / 2
     const int r = blockIdx.y, p = p0 + blockIdx.z;
@@ -121,10 +122,10 @@ void launch_tensor_run(Ctx *c, u64 *d01, u64 *D2, u64 *d2, const u64 *a, const u
         const dim3 grid((unsigned)(c->N / 512), (unsigned)limbs, (unsigned)n);
         c->n_launch++;
         if (d2)
-            k_tensor_run<true><<<grid, 256, 0, c->stream>>>(d01, D2, d2, a, b, K, P, p0, nA, nB, limbs, c->logN, bs, bp,
+            launch_pdl(k_tensor_run<true>, dim3(grid), 256, 0, c->stream, d01, D2, d2, a, b, K, P, p0, nA, nB, limbs, c->logN, bs, bp,
                                                             ix, c->d_mod, c->d_modf, accumulate);
         else
-            k_tensor_run<false><<<grid, 256, 0, c->stream>>>(d01, D2, d2, a, b, K, P, p0, nA, nB, limbs, c->logN, bs,
+            launch_pdl(k_tensor_run<false>, dim3(grid), 256, 0, c->stream, d01, D2, d2, a, b, K, P, p0, nA, nB, limbs, c->logN, bs,
                                                              bp, ix, c->d_mod, c->d_modf, accumulate);
     }
 }
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(256) k_relin_up(const u64 *d2, u64 *SY, u64 *d
                                                   int logN, int Lp1, const ModQ *mods, const ShoupPair *up_inv,
                                                   const ShoupPair *up_mod, int accumulate) {
     pdl_trigger();
+    pdl_wait();
     const int nq = level + 1, rows = nq + A, d = blockIdx.y, i0 = d * A, ns = min(A, nq - i0);
     const long N = 1L << logN;
     ShoupPair inv[A], wp[A][A];   // wp[s][j]: (Q_d / q_s) mod p_j
@@ -196,6 +198,7 @@ template <int A>
 __global__ void __launch_bounds__(256, 4) k_relin_ms(u64 *u, const u64 *digP, const u64 *key, int items, int ndig,
                                                      int logN, int Lp1, int nprimes, const ModQ *mods) {
     pdl_trigger();
+    pdl_wait();
     const long N = 1L << logN;
     const int tx = threadIdx.x & 31, ti = threadIdx.x >> 5;
     const int x = 2 * (blockIdx.x * 32 + tx), j = blockIdx.y;
@@ -225,6 +228,7 @@ template <int A>
 __global__ void __launch_bounds__(256) k_relin_down(const u64 *uP, u64 *YP, int K, int P, int logN,
                                                     const __grid_constant__ MdExact k, int accumulate) {
     pdl_trigger();
+    pdl_wait();
     const long N = 1L << logN;
     const long idx = (long)blockIdx.x * 256 + threadIdx.x;   // (p, poly, x): 256 | N
     const long pp = idx >> logN;
@@ -292,6 +296,7 @@ __global__ void __launch_bounds__(256) k_relin_up_fin(u64 *dig, const u64 *SY, c
                                                       int ndig, int logN, const ulonglong2 *Wf, const ShoupPair *Ws,
                                                       const ModQ *mods, const ModF *modf) {
     pdl_trigger();
+    pdl_wait();
     const int nq = level + 1, d = blockIdx.y, i0 = d * A, ns = min(A, nq - i0);
     const long N = 1L << logN, units = (long)P << logN;
     LinRows L = {};
@@ -320,6 +325,7 @@ __global__ void __launch_bounds__(256) k_relin_down_fin(u64 *conv, const u64 *YP
                                                         int nt, const ulonglong2 *Wf, const ShoupPair *Ws,
                                                         const ModQ *mods, const ModF *modf) {
     pdl_trigger();
+    pdl_wait();
     const int nq = level + 1;
     const long N = 1L << logN, units = (long)items << logN;
     LinRows L = {};
@@ -347,19 +353,19 @@ static void run_a(Ctx *c, RelinSum &S, u64 *d2, int K) {
     c->n_launch++;
     cudaEvent_t e0;
     c->trace_begin(3, e0);
-    k_relin_up<A><<<dim3(gx, nd), 256, 0, c->stream>>>(d2, S.SY.p, digP.p, K, P, S.level, nd, c->logN, c->L + 1, c->d_mod,
+    launch_pdl(k_relin_up<A>, dim3(gx, nd), 256, 0, c->stream, d2, S.SY.p, digP.p, K, P, S.level, nd, c->logN, c->L + 1, c->d_mod,
                                                        lc.d_up_inv, lc.d_up_mod, acc);
     c->trace_end(3, e0, 8.0 * N * P * (K * (nq + (double)nd * A) + (acc ? 4.0 : 2.0) * nq));
     ntt_fwd(c, digP.p, (long)K * P * nd * A, c->map_p(), c->stream);
     c->n_launch++;
     c->trace_begin(0, e0);
-    k_relin_ms<A><<<dim3((unsigned)(N / 64), A, (unsigned)((K * P + 7) / 8)), 256, 0, c->stream>>>(
+    launch_pdl(k_relin_ms<A>, dim3((unsigned)(N / 64), A, (unsigned)((K * P + 7) / 8)), 256, 0, c->stream, 
         uP.p, digP.p, c->rlk, K * P, nd, c->logN, c->L + 1, c->nprimes, c->d_mod);
     c->trace_end(0, e0, 8.0 * N * A * (2.0 * nd + (double)K * P * (nd + 2)), (double)K * P * nd * A * N * 2.0);
     ntt_inv(c, uP.p, (long)K * P * 2 * A, c->map_p(), c->stream);
     c->n_launch++;
     c->trace_begin(4, e0);
-    k_relin_down<A><<<(unsigned)(2L * P * N / 256), 256, 0, c->stream>>>(uP.p, S.YP.p, K, P, c->logN, c->md_exact, acc);
+    launch_pdl(k_relin_down<A>, dim3((unsigned)(2L * P * N / 256)), 256, 0, c->stream, uP.p, S.YP.p, K, P, c->logN, c->md_exact, acc);
     c->trace_end(4, e0, 8.0 * N * 2 * P * (K * A + (acc ? 2.0 : 1.0) * (2 * A + 1)));
     S.terms += K;
 }
@@ -374,7 +380,7 @@ static void finish_a(Ctx *c, RelinSum &S, const u64 *D2, u64 *out) {
     c->n_launch++;
     cudaEvent_t e0;
     c->trace_begin(3, e0);
-    k_relin_up_fin<A><<<dim3(gx, nd), 256, 0, c->stream>>>(dig.p, S.SY.p, D2, P, S.level, nd, c->logN, lc.d_su_f,
+    launch_pdl(k_relin_up_fin<A>, dim3(gx, nd), 256, 0, c->stream, dig.p, S.SY.p, D2, P, S.level, nd, c->logN, lc.d_su_f,
                                                            lc.d_su_s, c->d_mod, c->d_modf);
     c->trace_end(3, e0, 8.0 * N * P * (3.0 * nq + (double)nd * nq));
     RowSkip sk;
@@ -383,7 +389,7 @@ static void finish_a(Ctx *c, RelinSum &S, const u64 *D2, u64 *out) {
     launch_multsum_q(c, u.p, dig.p, c->rlk, P, S.level, c->stream);
     c->n_launch++;
     c->trace_begin(4, e0);
-    k_relin_down_fin<A><<<(unsigned)std::min<long>(2L * P * N / 256, (long)c->nsm * 8), 256, 0, c->stream>>>(
+    launch_pdl(k_relin_down_fin<A>, dim3((unsigned)std::min<long>(2L * P * N / 256, (long)c->nsm * 8)), 256, 0, c->stream, 
         conv.p, S.YP.p, 2 * P, S.terms, S.level, c->logN, c->L + 1, c->d_sd_f, c->d_sd_s, c->d_mod, c->d_modf);
     c->trace_end(4, e0, 8.0 * N * 2 * P * (2 * A + 1 + nq));
     SubScale ep;
