@@ -123,13 +123,15 @@ void rescale(Ctx *c, const u64 *in, int B, int level, u64 *out) {
 // ModDown then Rescale of items over Q_l P ([2 B][rows][N]) -> [B][2][l][N]:
 // the words of moddown and rescale in a row, with one forward NTT of l rows per
 // polynomial for the two (k_moddown_bconv, RS).
-void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out) {
+void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out, u64 *const *outs) {
     const int N = c->N, rows = c->qp_rows(level), a1 = c->alpha + 1;
     if (level < 1) throw HeError(HE_ERR_LEVEL, "rescale at level 0");
     if (c->logN < 14 || c->logN > 16) {
         Buf t(&c->pool, (size_t)B * 2 * (level + 1) * N);
         moddown(c, u, 2 * B, level, t.p, (long)(level + 1) * N);
-        rescale(c, t.p, B, level, out);
+        if (!outs) rescale(c, t.p, B, level, out);
+        else
+            for (int b = 0; b < B; b++) rescale(c, t.p + (size_t)b * 2 * (level + 1) * N, 1, level, outs[b]);
         return;
     }
     Buf pc(&c->pool, (size_t)2 * B * a1 * N), z(&c->pool, (size_t)2 * B * level * N);
@@ -138,6 +140,10 @@ void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out) {
     SubScale ep;
     ep.u = u, ep.us = (long)rows * N, ep.out = out, ep.os = (long)level * N;
     ep.w = c->lc(level).d_mr_inv, ep.wf = c->lc(level).d_mr_invf, ep.rows_per_item = level;
+    if (outs) {
+        ep.n_out = B;
+        for (int b = 0; b < B; b++) ep.outs[b] = outs[b];
+    }
     ntt_fwd_subscale(c, z.p, 2L * B * level, c->map_q(level - 1), c->stream, ep);
 }
 
@@ -337,14 +343,22 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
     c->n_md += B;
 }
 
+// The ModDown's last store adds into ct in place.
+void rotate_add(Ctx *c, u64 *ct, int B, int level, uint32_t g) {
+    const int rows = c->qp_rows(level);
+    const size_t N = c->N;
+    const long nq = level + 1;
+    Buf dg(&c->pool, (size_t)B * c->ndig(level) * rows * N), u(&c->pool, (size_t)B * 2 * rows * N);
+    modup(c, ct + nq * N, 2L * nq * N, B, level, dg.p);
+    rot_qp(c, ct, B, level, dg.p, g, u.p);
+    moddown(c, u.p, 2 * B, level, ct, nq * N, ct, nq * N);
+    c->n_md += B;
+}
+
 // ct <- ct + Rot(ct, -n^2 2^j) for j = 0 .. log2(S/n^2)-1 (period n^2).
 void replicate(Ctx *c, u64 *ct, int B, int level, int n) {
     const long n2 = (long)n * n;
-    Buf r(&c->pool, (size_t)B * 2 * (level + 1) * c->N);
-    for (long s = n2; s < c->S; s *= 2) {
-        rotate(c, ct, B, level, galois_of_step(c, c->S - s), r.p);
-        add(c, ct, r.p, B, level, ct);
-    }
+    for (long s = n2; s < c->S; s *= 2) rotate_add(c, ct, B, level, galois_of_step(c, c->S - s));
 }
 
 // JKLS product (eq. 4) with the hoisting of Sec. 4.1; A, B: [Bn][2][l+1][N]

@@ -31,7 +31,13 @@ void rot_qp_multi(Ctx *c, const u64 *ct, int B, int level, const u64 *digits, co
 void rotate_digits(Ctx *c, const u64 *ct, int B, int level, const u64 *digits, uint32_t g, u64 *out);
 void rotate(Ctx *c, const u64 *ct, int B, int level, uint32_t g, u64 *out);
 void rescale(Ctx *c, const u64 *in, int B, int level, u64 *out);
-void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out);
+// out: [B][2][l][N], or outs[b] for each of at most 8 items
+void moddown_rescale(Ctx *c, const u64 *u, int B, int level, u64 *out, u64 *const *outs = nullptr);
+constexpr int kMultMany = 8;
+void mult_rescale_many(Ctx *c, const u64 *const *a, const int *a_level, const u64 *const *b, const int *b_level, int n,
+                       int level, u64 *const *out);
+// ct [B][2][l+1][N] += Rot(ct; g)
+void rotate_add(Ctx *c, u64 *ct, int B, int level, uint32_t g);
 void drop(Ctx *c, const u64 *in, int B, int level, int to, u64 *out);
 // b may sit at a higher level b_level (its first level + 1 limbs are used in place)
 void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out, bool accumulate = false,

@@ -342,6 +342,8 @@ struct SubScale {
     const ulonglong2 *wf = nullptr;   // the same constants for the float-quotient product
     int rows_per_item = 1;
     unsigned row0 = 0;   // the launch's first row (counted from item 0)
+    u64 *outs[8] = {};   // when set (n_out > 0): item it goes to outs[it / 2] + (it & 1) os
+    int n_out = 0;
     const u64 *add = nullptr;   // optional addend, laid out like out (item stride as)
     long as = 0;
 };
@@ -384,6 +386,8 @@ void launch_automorph(Ctx *c, u64 *out, const u64 *in, long rows, const RowMap &
 // polynomial to its second (0: limbs * N).
 void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, long as, long bs,
                        const RowMap &rm, cudaStream_t st, bool acc01, bool acc2, long b_poly_stride = 0);
+// u [B][2][rows][N] over Q_l P += P d on the rows of Q, d [B][2][l+1][N]
+void launch_add_lifted(Ctx *c, u64 *u, const u64 *d, int B, int level, cudaStream_t st);
 // key switching pieces
 // own_ntt (may be null): the input in the NTT domain, item stride own_s; the
 // digit's own rows are then copied from it (and the forward NTT must skip

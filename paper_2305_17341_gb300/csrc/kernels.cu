@@ -1908,6 +1908,23 @@ void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const
     }
 }
 
+__global__ void k_add_lifted(u64 *u, const u64 *d, int level, int rows, int logN, const ModQ *mods,
+                             const ShoupPair *Pmod) {
+    pdl_trigger();
+    pdl_wait();
+    const long N = 1L << logN, x = (long)blockIdx.x * 256 + threadIdx.x;   // 256 | N
+    const int r = blockIdx.y;
+    const u64 q = mods[r].q;
+    const ShoupPair w = Pmod[r];
+    u64 *o = u + ((long)blockIdx.z * rows + r) * N + x;
+    *o = addmod(*o, shoup(d[((long)blockIdx.z * (level + 1) + r) * N + x], w.w, w.wp, q), q);
+}
+void launch_add_lifted(Ctx *c, u64 *u, const u64 *d, int B, int level, cudaStream_t st) {
+    c->n_launch++;
+    launch_pdl(k_add_lifted, dim3((unsigned)(c->N / 256), (unsigned)(level + 1), (unsigned)(2 * B)), 256, 0, st, u, d, level,
+               c->qp_rows(level), c->logN, c->d_mod, c->d_Pmod);
+}
+
 // P * a over Q_l P: rows q_r get (P mod q_r) a_r, the p rows are zero.
 // in: [items][l+1][N] (stride in_s), out: [items][l+1+alpha][N] (stride out_s)
 __global__ void k_lift_P(u64 *out, const u64 *in, int items, int level, int alpha, int N, long is, long os,

@@ -364,7 +364,7 @@ __device__ __forceinline__ void fwd_tile(u64 (&x)[16], u64 *sm, const PassTw<LM,
         const int r = (int)(arow - it * (u32)ep.rows_per_item);
         const long off = (long)r * N + seq * M;
         const u64 *up = ep.u + it * ep.us + off;
-        u64 *op = ep.out + it * ep.os + off;
+        u64 *op = (ep.n_out ? ep.outs[it >> 1] + (it & 1) * ep.os : ep.out + it * ep.os) + off;
         // every operand before the first store: a load may not pass a store
         // that could alias it, so interleaved they would be 16 memory latencies
 #pragma unroll
@@ -972,7 +972,7 @@ void ntt_fwd_subscale(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStre
     int logN = ctx->logN, logN1, C, R;
     split(logN, logN1, C, R);
     if (logN < 14 || logN > 16) throw std::logic_error("the fused NTT epilogue needs the register-blocked NTT");
-    const long chunk = ctx->ntt_chunk > 0 && ctx->ntt_chunk < 65535 ? ctx->ntt_chunk : 65535;
+    const long chunk = ctx->ntt_chunk > 0 && ctx->ntt_chunk < 65535 && !ep.n_out ? ctx->ntt_chunk : 65535;
     for (long r0 = 0; r0 < rows; r0 += chunk) {
         long nr = rows - r0 < chunk ? rows - r0 : chunk;
         u64 *d = data + r0 * (long)ctx->N;
@@ -980,6 +980,7 @@ void ntt_fwd_subscale(Ctx *ctx, u64 *data, long rows, const RowMap &rm, cudaStre
         // the chunk's rows counted from the item it starts in
         SubScale e = ep;
         const long i0 = r0 / ep.rows_per_item;
+        if (ep.n_out && r0) throw std::logic_error("separate outputs take one launch");
         e.u += i0 * ep.us, e.out += i0 * ep.os;
         if (e.add) e.add += i0 * ep.as;
         e.row0 = (unsigned)(r0 - i0 * ep.rows_per_item);

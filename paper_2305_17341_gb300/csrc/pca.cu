@@ -128,13 +128,43 @@ public:
     HC mult(HC a, HC b) {
         a = need(std::move(a), 1);
         b = need(std::move(b), 1);
-        auto ab = align(std::move(a), std::move(b));
-        const he_ct *x = ab.first.p, *y = ab.second.p;
-        HC t = make(x->level, x->scale * y->scale, std::min(x->period, y->period));
-        mult_relin(c, x->d, y->d, 1, x->level, t->d);
-        return rescale_ct(t.p, false);
+        return std::move(mult_all({{a.p, b.p}})[0]);
     }
-    HC mult(const he_ct *a, const he_ct *b) { return mult(clone(a), clone(b)); }
+    HC mult(const he_ct *a, const he_ct *b) {
+        if (a->level >= 1 && b->level >= 1) return std::move(mult_all({{a, b}})[0]);
+        return mult(clone(a), clone(b));
+    }
+
+    // Rescaled products of pairs of ciphertexts with at least one level, each at
+    // the lower of its operands' levels.  Consecutive pairs of one level go
+    // through the key switch together.
+    std::vector<HC> mult_all(const std::vector<std::pair<const he_ct *, const he_ct *>> &ps) {
+        std::vector<HC> out;
+        for (size_t i = 0, j; i < ps.size(); i = j) {
+            const int lv = std::min(ps[i].first->level, ps[i].second->level);
+            const u64 *a[kMultMany], *b[kMultMany];
+            int al[kMultMany], bl[kMultMany];
+            u64 *o[kMultMany];
+            for (j = i; j < ps.size() && j - i < kMultMany && std::min(ps[j].first->level, ps[j].second->level) == lv; j++) {
+                const he_ct *x = ps[j].first, *y = ps[j].second;
+                a[j - i] = x->d, al[j - i] = x->level, b[j - i] = y->d, bl[j - i] = y->level;
+                out.push_back(make(lv - 1, (x->scale * y->scale) / (double)c->primes[lv], std::min(x->period, y->period)));
+                o[j - i] = out.back()->d;
+            }
+            mult_rescale_many(c, a, al, b, bl, (int)(j - i), lv, o);
+        }
+        return out;
+    }
+    // the same for operands that may need a refresh, which happens in order
+    std::vector<HC> mult_list(const std::vector<std::pair<const he_ct *, const he_ct *>> &ps) {
+        for (auto &p : ps)
+            if (p.first->level < 1 || p.second->level < 1) {
+                std::vector<HC> out;
+                for (auto &q : ps) out.push_back(mult(q.first, q.second));
+                return out;
+            }
+        return mult_all(ps);
+    }
 
     void scalar_mul(const he_ct *a, long long m, u64 *out) {
         std::vector<ShoupPair> w(a->level + 1);
@@ -230,26 +260,75 @@ public:
     }
 
     // Aggregate (Sec. 5.2)
-    HC aggregate(const he_ct *in, int axis, int n) {
+    HC aggregate(const he_ct *in, int axis, int n) { return std::move(aggregate_all({in}, axis, n)[0]); }
+
+    std::vector<HC> aggregate_list(const std::vector<HC> &in, int axis, int n) {
+        std::vector<const he_ct *> p;
+        for (auto &x : in) p.push_back(x.p);
+        return aggregate_all(p, axis, n);
+    }
+
+    // of several ciphertexts: those of one level and period (with the level that
+    // axis 1's mask takes) as one batch
+    std::vector<HC> aggregate_all(const std::vector<const he_ct *> &in, int axis, int n) {
         const long n2 = (long)n * n;
-        HC A = replicated(in, n);
+        const int lv = in[0]->level, per = in[0]->period, B = (int)in.size();
+        bool same = true;
+        for (auto *x : in) same = same && x->level == lv && x->period == per;
+        if (B > 1 && (!same || (axis == 1 && lv < 1))) {
+            std::vector<HC> out;
+            for (auto *x : in) out.push_back(aggregate(x, axis, n));
+            return out;
+        }
+        const size_t w = ct_words(c, lv);
+        std::vector<HC> out;
+        Buf buf;
+        u64 *d;
+        int level = lv;
+        if (B == 1) {
+            out.push_back(clone(in[0]));
+            d = out[0]->d;
+        } else {
+            buf = Buf(&c->pool, B * w);
+            d = buf.p;
+            for (int i = 0; i < B; i++)
+                cudaMemcpyAsync(d + i * w, in[i]->d, w * 8, cudaMemcpyDeviceToDevice, c->stream);
+        }
+        if (per != n2) replicate(c, d, B, level, n);
+        auto spread = [&](long from, long to, long sign) {
+            for (long i = from; i < to; i <<= 1)
+                rotate_add(c, d, B, level, galois_of_step(c, ((sign * i) % n2 + n2) % n2));
+        };
         if (axis == 0) {
-            for (long i = n; i < n2; i <<= 1) {
-                HC r = rot(A.p, i % n2);
-                A = add_ct(A.p, r.p);
+            spread(n, n2, 1);
+        } else {
+            spread(1, n, 1);
+            if (B == 1) {
+                out[0]->period = (int)n2;
+                out[0] = mul_mask(std::move(out[0]), 6, n);
+                d = out[0]->d, level = out[0]->level;
+            } else {
+                const u64 *pt = get_pt(c, 6, n, 0, 0, 1.0, 0, level);
+                const long nq = (long)(level + 1) * c->N;
+                for (int i = 0; i < 2 * B; i++)
+                    launch_mulM(c, d + i * nq, d + i * nq, pt, level + 1, c->map_q(level), c->stream);
+                Buf r(&c->pool, B * ct_words(c, level - 1));
+                rescale(c, d, B, level, r.p);
+                buf = std::move(r);
+                d = buf.p, level--;
             }
-            return A;
+            spread(1, n, -1);
         }
-        for (long i = 1; i < n; i <<= 1) {
-            HC r = rot(A.p, i % n2);
-            A = add_ct(A.p, r.p);
+        if (B == 1) {
+            out[0]->period = (int)n2;
+            return out;
         }
-        A = mul_mask(std::move(A), 6, n);
-        for (long i = -1; i > -n; i *= 2) {
-            HC r = rot(A.p, ((i % n2) + n2) % n2);
-            A = add_ct(A.p, r.p);
+        for (int i = 0; i < B; i++) {
+            HC o = make(level, in[i]->scale, (int)n2);
+            cudaMemcpyAsync(o->d, d + i * ct_words(c, level), ct_words(c, level) * 8, cudaMemcpyDeviceToDevice, c->stream);
+            out.push_back(std::move(o));
         }
-        return A;
+        return out;
     }
 
     HC transpose(const he_ct *a, int n, int n1, double prescale) {
@@ -462,14 +541,19 @@ public:
         for (int it = 0; it < iters; it++) {
             y = need(std::move(y), 3);
             x = need(std::move(x), 3);
-            HC t1 = mult(y.p, y.p);
-            HC t2 = mult(y.p, x.p);
-            HC t3 = mult(std::move(t1), std::move(t2));
+            std::vector<HC> t = mult_all({{y.p, y.p}, {y.p, x.p}});
+            HC t3 = mult(std::move(t[0]), std::move(t[1]));
             HC y3 = to_scale(mul_const_int(y.p, 3), t3->level, t3->scale);
             HC d = sub_ct(y3.p, t3.p);
             y = mul_const(std::move(d), 0.5, &delta);
         }
         return y;
+    }
+
+    HC sum(std::vector<HC> v) {
+        HC acc = std::move(v[0]);
+        for (size_t i = 1; i < v.size(); i++) acc = add_aligned(std::move(acc), std::move(v[i]));
+        return acc;
     }
 
     HC add_aligned(HC a, HC b) {
@@ -539,26 +623,42 @@ public:
         std::vector<HC> hold;
         std::vector<const he_ct *> V;
         for (auto &v : V0) V.push_back(once(v.p, hold));
+        std::vector<std::pair<const he_ct *, const he_ct *>> ps;
+        for (int i = 0; i < k; i++)
+            for (int j = 0; j < k; j++) ps.push_back({axis == 0 ? C[i * k + j] : C[j * k + i], V[j]});
+        bool fresh = true;   // no product refreshes an operand
+        for (auto &p : ps) fresh = fresh && p.first->level >= 1 && p.second->level >= 1;
         std::vector<HC> out;
-        for (int i = 0; i < k; i++) {
-            HC acc;
-            for (int j = 0; j < k; j++) {
-                const he_ct *blk = axis == 0 ? C[i * k + j] : C[j * k + i];
-                HC p = mult(blk, V[j]);
-                acc = acc.p ? add_aligned(std::move(acc), std::move(p)) : std::move(p);
+        if (!fresh) {   // refreshes in the order of the circuit: a row's products, its Aggregate
+            for (int i = 0; i < k; i++) {
+                HC acc;
+                for (int j = 0; j < k; j++) {
+                    HC p = mult(ps[i * k + j].first, ps[i * k + j].second);
+                    acc = acc.p ? add_aligned(std::move(acc), std::move(p)) : std::move(p);
+                }
+                out.push_back(aggregate(acc.p, (axis + 1) % 2, n));
             }
-            out.push_back(aggregate(acc.p, (axis + 1) % 2, n));
+            return out;
         }
-        return out;
+        std::vector<HC> pr = mult_all(ps), sums;
+        for (int i = 0; i < k; i++) {
+            HC acc = std::move(pr[i * k]);
+            for (int j = 1; j < k; j++) acc = add_aligned(std::move(acc), std::move(pr[i * k + j]));
+            sums.push_back(std::move(acc));
+        }
+        return aggregate_list(sums, (axis + 1) % 2, n);
     }
 
     std::vector<HC> axis_flip(const std::vector<HC> &V, int axis, int n) {
-        std::vector<HC> out;
+        const int ax = (axis + 1) % 2;
+        bool fresh = true;   // neither the mask nor axis 1's Aggregate refreshes
+        for (auto &v : V) fresh = fresh && v->level >= 1 + ax;
+        std::vector<HC> w, out;
         for (auto &v : V) {
-            HC w = mul_mask(replicated(v.p, n), 7, n);
-            out.push_back(aggregate(w.p, (axis + 1) % 2, n));
+            w.push_back(mul_mask(replicated(v.p, n), 7, n));
+            if (!fresh) out.push_back(aggregate(w.back().p, ax, n));
         }
-        return out;
+        return fresh ? aggregate_list(w, ax, n) : std::move(out);
     }
 
     void power_method(he_ct *const *C, int k, int n, he_ct *const *V0, int axis, int l_P, const int *counts,
@@ -570,25 +670,21 @@ public:
             std::vector<HC> Vn = cov_apply(C, k, V, axis, n);
             int axis_n = (axis + 1) % 2;
             if (t < l_P) {
-                HC acc;
-                for (auto &v : Vn) {
-                    HC p = mult(v.p, v.p);
-                    acc = acc.p ? add_aligned(std::move(acc), std::move(p)) : std::move(p);
-                }
+                std::vector<std::pair<const he_ct *, const he_ct *>> sq;
+                for (auto &v : Vn) sq.push_back({v.p, v.p});
+                HC acc = sum(mult_list(sq));
                 HC norm2 = aggregate(acc.p, (axis_n + 1) % 2, n);
                 HC g = taylor_init(need(clone(norm2.p), 1), B2);
                 HC inv = newton(std::move(norm2), std::move(g), counts[t]);
-                std::vector<HC> Vs;
-                for (auto &v : Vn) Vs.push_back(mult(v.p, inv.p));
-                V = std::move(Vs);
+                std::vector<std::pair<const he_ct *, const he_ct *>> sc;
+                for (auto &v : Vn) sc.push_back({v.p, inv.p});
+                V = mult_list(sc);
                 axis = axis_n;
             } else {
                 std::vector<HC> Vf = axis_flip(V, axis, n);
-                HC acc;
-                for (int i = 0; i < k; i++) {
-                    HC p = mult(Vn[i].p, Vf[i].p);
-                    acc = acc.p ? add_aligned(std::move(acc), std::move(p)) : std::move(p);
-                }
+                std::vector<std::pair<const he_ct *, const he_ct *>> dp;
+                for (int i = 0; i < k; i++) dp.push_back({Vn[i].p, Vf[i].p});
+                HC acc = sum(mult_list(dp));
                 lam = aggregate(acc.p, (axis_n + 1) % 2, n);
                 Vout = std::move(V);
                 VT = std::move(Vf);

@@ -130,6 +130,66 @@ void launch_tensor_run(Ctx *c, u64 *d01, u64 *D2, u64 *d2, const u64 *a, const u
     }
 }
 
+// Tensors of separate ciphertexts: d01 [n][2][limbs][N], d2 [n][limbs][N] of
+// a[i] b[i], each given by its first polynomial and the distance of its second.
+struct MultPtrs {
+    const u64 *a[kMultMany], *b[kMultMany];
+    long as[kMultMany], bs[kMultMany];
+};
+__global__ void __launch_bounds__(256) k_tensor_ptrs(u64 *d01, u64 *d2, const __grid_constant__ MultPtrs mp, int limbs,
+                                                     int logN, const ModQ *mods, const ModF *modf) {
+    pdl_trigger();
+    pdl_wait();
+    const long N = 1L << logN;
+    const int r = blockIdx.y, i = blockIdx.z;
+    const long ro = (long)r * N + blockIdx.x * 256 + threadIdx.x;   // 256 | N
+    const ModQ m = mods[r];
+    const ModF f = modf[r];
+    const u64 a0 = mp.a[i][ro], a1 = mp.a[i][ro + mp.as[i]], b0 = mp.b[i][ro], b1 = mp.b[i][ro + mp.bs[i]];
+    u64 o0, o1, o2;
+    if (f.on) {   // uniform over the CTA
+        const float c = f.qi * 1.4901161193847656e-08f;   // 2^6 / q
+        const ulonglong2 v0 = fq_var(b0, c), v1 = fq_var(b1, c);
+        o0 = fq_pos(fq_mul(a0, v0, f), m.q);
+        o1 = fq_pos(fq_red(fq_mul(a0, v1, f) + fq_mul(a1, v0, f), f), m.q);
+        o2 = fq_pos(fq_mul(a1, v1, f), m.q);
+    } else {
+        o0 = mulmod(a0, b0, m);
+        o1 = addmod(mulmod(a0, b1, m), mulmod(a1, b0, m), m.q);
+        o2 = mulmod(a1, b1, m);
+    }
+    d01[((long)i * 2 * limbs) * N + ro] = o0;
+    d01[((long)i * 2 * limbs + limbs) * N + ro] = o1;
+    d2[(long)i * limbs * N + ro] = o2;
+}
+
+// out[i] [2][level][N] = Rescale(Mult(a[i], b[i])) at level `level` for n <= kMultMany
+// pairs of ciphertexts at levels >= level: the words of mult_relin and rescale,
+// with (d0, d1) lifted into the key switch's Q_l P sum (ModDown(u + P d) = d +
+// ModDown(u)) so that one ModDown + rescale ends both.
+void mult_rescale_many(Ctx *c, const u64 *const *a, const int *a_level, const u64 *const *b, const int *b_level, int n,
+                       int level, u64 *const *out) {
+    if (!c->rlk) throw HeError(HE_ERR_KEY_MISSING, "relinearisation key missing");
+    const int nq = level + 1, rows = c->qp_rows(level);
+    const size_t N = c->N;
+    Buf d01(&c->pool, n * 2 * nq * N), d2(&c->pool, n * nq * N), dg(&c->pool, (size_t)n * c->ndig(level) * rows * N),
+        u(&c->pool, n * 2 * rows * N);
+    MultPtrs mp = {};
+    for (int i = 0; i < n; i++) {
+        mp.a[i] = a[i], mp.as[i] = (long)(a_level[i] + 1) * N;
+        mp.b[i] = b[i], mp.bs[i] = (long)(b_level[i] + 1) * N;
+    }
+    c->n_launch++;
+    launch_pdl(k_tensor_ptrs, dim3((unsigned)(N / 256), (unsigned)nq, (unsigned)n), 256, 0, c->stream, d01.p, d2.p, mp, nq,
+               c->logN, c->d_mod, c->d_modf);
+    modup(c, d2.p, (long)(nq * N), n, level, dg.p);
+    launch_multsum(c, u.p, dg.p, c->rlk, 1u, n, level, nullptr, 0, c->stream);
+    c->n_ms += n;
+    launch_add_lifted(c, u.p, d01.p, n, level, c->stream);
+    moddown_rescale(c, u.p, n, level, nullptr, out);
+    c->n_md += n;
+}
+
 // ------------------------------------------------------- per-term conversions
 // Decompose's integers of a run: d2 [K][P][nq][N] (coefficient form) -> SY
 // [P][2][nq][N] (+)= sum_kk (low, high words of y_{kk,i}), and the P rows of the
