@@ -658,9 +658,8 @@ static u64 *gen_swk(Ctx *c, const u64 *sprime, uint32_t obj) {
             launch_mulconst_rows(c, t.p, sprime + (size_t)i * N, c->d_Pmod + i, 1, 1, one, c->stream);
             launch_add(c, k0 + (size_t)i * N, k0 + (size_t)i * N, t.p, 1, one, c->stream);
         }
-        launch_to_mont(c, k0, k0, np, all, c->stream);
-        launch_to_mont(c, k1, k1, np, all, c->stream);
     }
+    launch_key_form(c, key, (long)c->dnum * 2 * np, all, c->stream);
     return key;
 }
 

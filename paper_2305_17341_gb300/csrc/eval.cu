@@ -214,7 +214,10 @@ const u64 *get_pt(Ctx *c, int kind, int n, long t, long rot, double value, int k
     RowMap qp = c->map_qp(level);
     launch_small_to_rns(c, (const i64 *)m.p, pt, rows, qp, c->stream);
     ntt_fwd(c, pt, rows, qp, c->stream);
-    launch_to_mont(c, pt, pt, rows, qp, c->stream);
+    // the PowerMethod's masks (kinds 6, 7, 10, 11) multiply by themselves, in
+    // Montgomery form; diagonals and column masks enter sums
+    if (kind == 6 || kind == 7 || kind == 10 || kind == 11) launch_to_mont(c, pt, pt, rows, qp, c->stream);
+    else launch_key_form(c, pt, rows, qp, c->stream);
     c->ptcache[key] = pt;
     c->ptcache_bytes += (size_t)rows * N * 8;
     return pt;

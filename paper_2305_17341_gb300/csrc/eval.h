@@ -6,11 +6,6 @@
 
 namespace he {
 
-struct HeError : std::runtime_error {
-    int code;
-    HeError(int c, const std::string &m) : std::runtime_error(m), code(c) {}
-};
-
 uint32_t galois_of_step(const Ctx *c, long step);
 void create_keys(Ctx *c);
 u64 *gen_rotation_key(Ctx *c, uint32_t g);

@@ -7,6 +7,7 @@
 #include <map>
 #include <set>
 #include <mutex>
+#include <stdexcept>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -240,11 +241,11 @@ struct Ctx {
     // vector's segments refreshed as one packed ciphertext
     bool newton_compose = false;
     bool pack_refresh = false;
-    // >= 0: every MultSum launch uses this variant (keys per launch 8), no tuning
+    // >= 0: every MultSum launch uses this split (modulo their number), no tuning
     int force_multsum = -1;
-    // (level, items, keys) -> (keys per launch << 8) | variant
+    // (level and rows, items, keys) -> split of the launch (msum_cfgs)
     std::map<std::tuple<int, int, int>, int> tune_multsum;
-    std::map<std::tuple<int, int, int>, int> tune_ck;   // fused C^k babies: (keys per launch << 8) | items per CTA
+    std::map<std::tuple<int, int, int>, int> tune_ck;   // fused C^k babies
     std::string tune_log;   // every timed plan, one line each
     TraceClass tr[5];   // 0 MultSum, 1 NTT forward, 2 NTT inverse, 3 ModUp BConv, 4 ModDown BConv
     std::vector<cudaEvent_t> ev_free;
@@ -305,6 +306,11 @@ int device_status(const Ctx *c);
         }                                                                            \
     } while (0)
 
+struct HeError : std::runtime_error {
+    int code;
+    HeError(int c, const std::string &m) : std::runtime_error(m), code(c) {}
+};
+
 // Launches a kernel that calls pdl_wait so that it may start while the kernel
 // before it in the stream finishes (modarith.cuh).
 template <class... P, class... A>
@@ -315,7 +321,8 @@ inline void launch_pdl(void (*kern)(P...), dim3 grid, unsigned block, size_t sme
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = grid, cfg.blockDim = dim3(block), cfg.dynamicSmemBytes = smem, cfg.stream = st;
     cfg.attrs = at, cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
+    if (e != cudaSuccess) throw HeError(HE_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
 }
 
 // host number theory
@@ -404,9 +411,7 @@ void launch_moddown_final(Ctx *c, u64 *out, const u64 *u, const u64 *conv, const
                           cudaStream_t st);
 void launch_multsum(Ctx *c, u64 *out, const u64 *digits, const u64 *key, uint32_t g, int B, int level,
                     const u64 *c0_for_P, long c0_item_stride, cudaStream_t st);
-// Up to kMultSumMaxKeys rotations per launch share one read of the digits
-// (longer lists are split); keys must be in the permuted layout.
-constexpr int kMultSumMaxKeys = 8;
+// G rotations that share one read of the digits; keys must be in the permuted layout.
 void launch_multsum_multi(Ctx *c, u64 *const *outs, const u64 *digits, const u64 *const *keys, const uint32_t *gs,
                           int G, int B, int level, const u64 *c0_for_P, long c0s, cudaStream_t st);
 // G hoisted rotations of two sources with the same keys, each output the
@@ -415,6 +420,9 @@ void launch_multsum_ck(Ctx *c, u64 *const *outs, const u64 *dig1, const u64 *dig
                        const uint32_t *gs, const u64 *const *m1, const u64 *const *m2, int G, int B, int level,
                        const u64 *c01, const u64 *c02, long c0s, cudaStream_t st);
 void launch_multsum_q(Ctx *c, u64 *out, const u64 *digits, const u64 *key, int B, int level, cudaStream_t st);
+void launch_relin_ms(Ctx *c, u64 *u, const u64 *digP, int items, int ndig, cudaStream_t st);
+// rows into the form that MultSum and the plaintext sums read (msum.cu)
+void launch_key_form(Ctx *c, u64 *key, long rows, const RowMap &rm, cudaStream_t st);
 void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, cudaStream_t st);
 // out[y] ([B][2][rows][N] at stride out_s) = sum of the terms first[y] .. first[y+1]
 // of pt (.) R[r], y < sums; at most 32 terms a sum, nR <= 32.

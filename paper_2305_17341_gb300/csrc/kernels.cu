@@ -9,7 +9,6 @@
 #include <set>
 #include <stdexcept>
 
-#include "bulkcopy.cuh"
 #include "he_internal.h"
 #include "kernels.cuh"
 
@@ -784,371 +783,7 @@ void launch_moddown_final(Ctx *c, u64 *out, const u64 *u, const u64 *conv, const
                                                   c->d_dn_Pinv);
 }
 
-// ------------------------------------------------------------- MultSum
-// MultSum + Permute (Sec. 3.3.1) for G rotations that share one Decompose
-// output (hoisting).  Rotation keys are stored permuted, K'_g[y] = K_g[x]
-// with y = pi_g(x) the NTT-domain index of kappa_g, so that
-//   out_g[x] = sum_d D[d][pi_g(x)] K_g[d][x] = T_g[pi_g(x)],
-//   T_g[y]   = sum_d D[d][y] K'_g[d][y]
-// (the same products, summed in the same order, for every output word).
-// Each digit word is loaded once and multiplied into all G accumulators; the
-// result is written to x = pi_g^{-1}(y), which stays inside the aligned
-// 32-word block of y (kappa permutes the low bits of the bit-reversed index
-// only), so stores remain coalesced.  Keys in Montgomery form (one REDC per
-// output).  With c0 given, P * c0[y] is added on the Q rows of poly 0 (the
-// hoisted rotation kept in Q_l P of double hoisting).
-// digits: [B][ndig][rows][N]; key_k: [dnum][2][nprimes][N];
-// out_k: [B][2][rows][N].
-template <int G>
-struct MultiKeys {
-    const u64 *key[G];
-    u64 *out[G];
-    u32 ginv[G];   // pi_g^{-1} = pi_{g^{-1} mod 2N}; 1 = identity
-};
-
-// Each digit word is loaded once and multiplied into the 2G accumulators of
-// the G keys (2G independent accumulation chains per thread).
-// With PF > 0 every thread also asks L2 for its digit word PF digits ahead,
-// and the threads of the first item for their key words, so that more DRAM
-// requests are in flight than the loads themselves keep (no registers held).
-__device__ __forceinline__ void l2_prefetch(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
-// OCC: resident CTAs per SM the launch bound asks for (0: by G).
-template <int G, bool STREAM, int PF = 0, int OCC = 0>
-__global__ void __launch_bounds__(256, OCC ? OCC : G <= 2 ? 4 : G <= 5 ? 2 : 1) k_multsum_multi(MultiKeys<G> mk, const u64 *digits, int B, int BI, int level,
-                                                       int alpha, int L, int ndig, int nprimes, int logN,
-                                                       const ModQ *mods, const u64 *c0, long c0s,
-                                                       const ShoupPair *Pmod) {
-    pdl_trigger();
-    pdl_wait();
-    const int N = 1 << logN;
-    const int XW = 256 / BI;
-    const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
-    const int y = blockIdx.x * XW + tx;
-    const int r = blockIdx.y;
-    const int b = blockIdx.z * BI + ti;
-    if (b >= B || y >= N) return;
-    const int rows = level + 1 + alpha;
-    const int kr = r <= level ? r : L + 1 + (r - level - 1);   // the row's global prime
-    const ModQ m = mods[kr];
-    const long dstride = (long)rows * N;
-    const u64 *dp = digits + (long)b * ndig * dstride + (long)r * N + y;
-    const long koff = (long)kr * N + y, kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    U128 a0[G], a1[G];
-    if (m.q < (1ull << 42)) {
-        // residues below 2^42 (uniform over the CTA): 96-bit accumulation
-        u32 x0[2 * G], x1[2 * G], x2[2 * G];
-#pragma unroll
-        for (int k = 0; k < 2 * G; k++) x0[k] = 0, x1[k] = 0, x2[k] = 0;
-        for (int d = 0; d < ndig; d++) {
-            if (PF && d + PF < ndig) {
-                l2_prefetch(dp + (long)(d + PF) * dstride);
-                if (ti == 0)
-#pragma unroll
-                    for (int k = 0; k < G; k++) {
-                        l2_prefetch(mk.key[k] + (long)(d + PF) * kd + koff);
-                        l2_prefetch(mk.key[k] + (long)(d + PF) * kd + koff + kk);
-                    }
-            }
-            const u64 v = STREAM ? __ldcs(dp + (long)d * dstride) : __ldg(dp + (long)d * dstride);
-#pragma unroll
-            for (int k = 0; k < G; k++) {
-                const u64 *kp = mk.key[k] + (long)d * kd + koff;
-                mac96(x0[2 * k], x1[2 * k], x2[2 * k], v, __ldg(kp));
-                mac96(x0[2 * k + 1], x1[2 * k + 1], x2[2 * k + 1], v, __ldg(kp + kk));
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < G; k++) {
-            a0[k] = U128{((u64)x1[2 * k] << 32) | x0[2 * k], x2[2 * k]};
-            a1[k] = U128{((u64)x1[2 * k + 1] << 32) | x0[2 * k + 1], x2[2 * k + 1]};
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < G; k++) a0[k] = U128{0, 0}, a1[k] = U128{0, 0};
-        for (int d = 0; d < ndig; d++) {
-            if (PF && d + PF < ndig) {
-                l2_prefetch(dp + (long)(d + PF) * dstride);
-                if (ti == 0)
-#pragma unroll
-                    for (int k = 0; k < G; k++) {
-                        l2_prefetch(mk.key[k] + (long)(d + PF) * kd + koff);
-                        l2_prefetch(mk.key[k] + (long)(d + PF) * kd + koff + kk);
-                    }
-            }
-            const u64 v = STREAM ? __ldcs(dp + (long)d * dstride) : __ldg(dp + (long)d * dstride);
-#pragma unroll
-            for (int k = 0; k < G; k++) {
-                const u64 *kp = mk.key[k] + (long)d * kd + koff;
-                mac128_q(a0[k], v, __ldg(kp), m.q);
-                mac128_q(a1[k], v, __ldg(kp + kk), m.q);
-            }
-        }
-    }
-    u64 pc0 = 0;
-    const bool with_c0 = c0 && r <= level;
-    if (with_c0) {
-        ShoupPair w = Pmod[r];
-        pc0 = shoup(c0[b * c0s + (long)r * N + y], w.w, w.wp, m.q);
-    }
-#pragma unroll
-    for (int k = 0; k < G; k++) {
-        u64 o0 = redc(a0[k].lo, a0[k].hi, m), o1 = redc(a1[k].lo, a1[k].hi, m);
-        if (with_c0) o0 = addmod(o0, pc0, m.q);
-        const int x = mk.ginv[k] == 1u ? y : auto_index(y, mk.ginv[k], logN);
-        u64 *ob = mk.out[k] + (long)b * 2 * rows * N;
-        ob[(long)r * N + x] = o0;
-        ob[(long)(rows + r) * N + x] = o1;
-    }
-}
-
-// The thread-per-word MultSum with two adjacent coefficients per thread:
-// every digit and key load is 16 bytes (ulonglong2), so twice the bytes are
-// in flight per load at the same number of resident warps.  For launches of
-// at most two rotations (the per-thread accumulators double).
-template <int G, bool STREAM, int OCC>
-__global__ void __launch_bounds__(256, OCC) k_multsum_vec(MultiKeys<G> mk, const u64 *digits, int B, int BI, int level,
-                                                          int alpha, int L, int ndig, int nprimes, int logN,
-                                                          const ModQ *mods, const u64 *c0, long c0s,
-                                                          const ShoupPair *Pmod) {
-    pdl_trigger();
-    pdl_wait();
-    const int N = 1 << logN;
-    const int XW = 256 / BI;
-    const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
-    const int y = 2 * (blockIdx.x * XW + tx);
-    const int r = blockIdx.y;
-    const int b = blockIdx.z * BI + ti;
-    if (b >= B || y >= N) return;
-    const int rows = level + 1 + alpha;
-    const int kr = r <= level ? r : L + 1 + (r - level - 1);
-    const ModQ m = mods[kr];
-    const long dstride = (long)rows * N;
-    const ulonglong2 *dp = (const ulonglong2 *)(digits + (long)b * ndig * dstride + (long)r * N + y);
-    const long koff = (long)kr * N + y, kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    U128 acc[2][2 * G];   // [coefficient][key, polynomial]
-    if (m.q < (1ull << 42)) {
-        u32 x0[2][2 * G], x1[2][2 * G], x2[2][2 * G];
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int k = 0; k < 2 * G; k++) x0[c][k] = 0, x1[c][k] = 0, x2[c][k] = 0;
-        for (int d = 0; d < ndig; d++) {
-            const ulonglong2 v = STREAM ? __ldcs(dp + (long)d * dstride / 2) : __ldg(dp + (long)d * dstride / 2);
-#pragma unroll
-            for (int k = 0; k < G; k++) {
-                const ulonglong2 *kp = (const ulonglong2 *)(mk.key[k] + (long)d * kd + koff);
-                const ulonglong2 k0 = __ldg(kp), k1 = __ldg(kp + kk / 2);
-                mac96(x0[0][2 * k], x1[0][2 * k], x2[0][2 * k], v.x, k0.x);
-                mac96(x0[1][2 * k], x1[1][2 * k], x2[1][2 * k], v.y, k0.y);
-                mac96(x0[0][2 * k + 1], x1[0][2 * k + 1], x2[0][2 * k + 1], v.x, k1.x);
-                mac96(x0[1][2 * k + 1], x1[1][2 * k + 1], x2[1][2 * k + 1], v.y, k1.y);
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int k = 0; k < 2 * G; k++) acc[c][k] = U128{((u64)x1[c][k] << 32) | x0[c][k], x2[c][k]};
-    } else {
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int k = 0; k < 2 * G; k++) acc[c][k] = U128{0, 0};
-        for (int d = 0; d < ndig; d++) {
-            const ulonglong2 v = STREAM ? __ldcs(dp + (long)d * dstride / 2) : __ldg(dp + (long)d * dstride / 2);
-#pragma unroll
-            for (int k = 0; k < G; k++) {
-                const ulonglong2 *kp = (const ulonglong2 *)(mk.key[k] + (long)d * kd + koff);
-                const ulonglong2 k0 = __ldg(kp), k1 = __ldg(kp + kk / 2);
-                mac128_q(acc[0][2 * k], v.x, k0.x, m.q);
-                mac128_q(acc[1][2 * k], v.y, k0.y, m.q);
-                mac128_q(acc[0][2 * k + 1], v.x, k1.x, m.q);
-                mac128_q(acc[1][2 * k + 1], v.y, k1.y, m.q);
-            }
-        }
-    }
-    const bool with_c0 = c0 && r <= level;
-    const ShoupPair w = with_c0 ? Pmod[r] : ShoupPair{0, 0};
-#pragma unroll
-    for (int c = 0; c < 2; c++) {
-        const int yc = y + c;
-        u64 pc0 = 0;
-        if (with_c0) pc0 = shoup(c0[b * c0s + (long)r * N + yc], w.w, w.wp, m.q);
-#pragma unroll
-        for (int k = 0; k < G; k++) {
-            u64 o0 = redc(acc[c][2 * k].lo, acc[c][2 * k].hi, m), o1 = redc(acc[c][2 * k + 1].lo, acc[c][2 * k + 1].hi, m);
-            if (with_c0) o0 = addmod(o0, pc0, m.q);
-            const int x = mk.ginv[k] == 1u ? yc : auto_index(yc, mk.ginv[k], logN);
-            u64 *ob = mk.out[k] + (long)b * 2 * rows * N;
-            ob[(long)r * N + x] = o0;
-            ob[(long)(rows + r) * N + x] = o1;
-        }
-    }
-}
-
-// The same MultSum with the G keys split over the CTA's warps: 8 warps =
-// (G / KG) key groups x BI = 8 KG / G items, 32 coefficients of one row per
-// CTA; each thread accumulates KG keys of one item, so its state (2 KG
-// accumulators) does not grow with G and more CTAs fit on an SM.  A digit
-// word is loaded by the warps of every key group (one DRAM read, L1 for the
-// others), a key word by the warps of every item; every output word is
-// still the sum over the digits of the same products, reduced once.
-template <int G, int KG, int OCC>
-__global__ void __launch_bounds__(256, OCC) k_multsum_split(const __grid_constant__ MultiKeys<G> mk, const u64 *digits, int B, int level,
-                                                            int alpha, int L, int ndig, int nprimes, int logN,
-                                                            const ModQ *mods, const u64 *c0, long c0s,
-                                                            const ShoupPair *Pmod) {
-    pdl_trigger();
-    pdl_wait();
-    constexpr int NGRP = G / KG, BI = 8 / NGRP;
-    const int N = 1 << logN;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int kg0 = (wid / BI) * KG, bi = wid % BI;
-    const int y = blockIdx.x * 32 + lane;
-    const int r = blockIdx.y;
-    const int b = blockIdx.z * BI + bi;
-    if (b >= B || y >= N) return;
-    const int rows = level + 1 + alpha;
-    const int kr = r <= level ? r : L + 1 + (r - level - 1);
-    const ModQ m = mods[kr];
-    const long dstride = (long)rows * N;
-    const u64 *dp = digits + (long)b * ndig * dstride + (long)r * N + y;
-    const long koff = (long)kr * N + y, kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    U128 a0[KG], a1[KG];
-    if (m.q < (1ull << 42)) {
-        u32 x0[2 * KG], x1[2 * KG], x2[2 * KG];
-#pragma unroll
-        for (int k = 0; k < 2 * KG; k++) x0[k] = 0, x1[k] = 0, x2[k] = 0;
-        for (int d = 0; d < ndig; d++) {
-            const u64 v = __ldg(dp + (long)d * dstride);
-#pragma unroll
-            for (int k = 0; k < KG; k++) {
-                const u64 *kp = mk.key[kg0 + k] + (long)d * kd + koff;
-                mac96(x0[2 * k], x1[2 * k], x2[2 * k], v, __ldg(kp));
-                mac96(x0[2 * k + 1], x1[2 * k + 1], x2[2 * k + 1], v, __ldg(kp + kk));
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < KG; k++) {
-            a0[k] = U128{((u64)x1[2 * k] << 32) | x0[2 * k], x2[2 * k]};
-            a1[k] = U128{((u64)x1[2 * k + 1] << 32) | x0[2 * k + 1], x2[2 * k + 1]};
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < KG; k++) a0[k] = U128{0, 0}, a1[k] = U128{0, 0};
-        for (int d = 0; d < ndig; d++) {
-            const u64 v = __ldg(dp + (long)d * dstride);
-#pragma unroll
-            for (int k = 0; k < KG; k++) {
-                const u64 *kp = mk.key[kg0 + k] + (long)d * kd + koff;
-                mac128_q(a0[k], v, __ldg(kp), m.q);
-                mac128_q(a1[k], v, __ldg(kp + kk), m.q);
-            }
-        }
-    }
-    u64 pc0 = 0;
-    const bool with_c0 = c0 && r <= level;
-    if (with_c0) {
-        ShoupPair w = Pmod[r];
-        pc0 = shoup(c0[b * c0s + (long)r * N + y], w.w, w.wp, m.q);
-    }
-#pragma unroll
-    for (int k = 0; k < KG; k++) {
-        u64 o0 = redc(a0[k].lo, a0[k].hi, m), o1 = redc(a1[k].lo, a1[k].hi, m);
-        if (with_c0) o0 = addmod(o0, pc0, m.q);
-        const u32 gi = mk.ginv[kg0 + k];
-        const int x = gi == 1u ? y : auto_index(y, gi, logN);
-        u64 *ob = mk.out[kg0 + k] + (long)b * 2 * rows * N;
-        ob[(long)r * N + x] = o0;
-        ob[(long)(rows + r) * N + x] = o1;
-    }
-}
-
-// The key-split MultSum with two adjacent coefficients per thread and
-// 16-byte digit and key loads (each warp covers 64 coefficients).
-template <int G, int KG, int OCC>
-__global__ void __launch_bounds__(256, OCC) k_multsum_splitv(const __grid_constant__ MultiKeys<G> mk,
-                                                             const u64 *digits, int B, int level, int alpha, int L,
-                                                             int ndig, int nprimes, int logN, const ModQ *mods,
-                                                             const u64 *c0, long c0s, const ShoupPair *Pmod) {
-    pdl_trigger();
-    pdl_wait();
-    constexpr int NGRP = G / KG, BI = 8 / NGRP;
-    const int N = 1 << logN;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int kg0 = (wid / BI) * KG, bi = wid % BI;
-    const int y = 2 * (blockIdx.x * 32 + lane);
-    const int r = blockIdx.y;
-    const int b = blockIdx.z * BI + bi;
-    if (b >= B || y >= N) return;
-    const int rows = level + 1 + alpha;
-    const int kr = r <= level ? r : L + 1 + (r - level - 1);
-    const ModQ m = mods[kr];
-    const long dstride = (long)rows * N;
-    const ulonglong2 *dp = (const ulonglong2 *)(digits + (long)b * ndig * dstride + (long)r * N + y);
-    const long koff = (long)kr * N + y, kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    U128 acc[2][2 * KG];
-    if (m.q < (1ull << 42)) {
-        u32 x0[2][2 * KG], x1[2][2 * KG], x2[2][2 * KG];
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int k = 0; k < 2 * KG; k++) x0[c][k] = 0, x1[c][k] = 0, x2[c][k] = 0;
-        for (int d = 0; d < ndig; d++) {
-            const ulonglong2 v = __ldg(dp + (long)d * dstride / 2);
-#pragma unroll
-            for (int k = 0; k < KG; k++) {
-                const ulonglong2 *kp = (const ulonglong2 *)(mk.key[kg0 + k] + (long)d * kd + koff);
-                const ulonglong2 k0 = __ldg(kp), k1 = __ldg(kp + kk / 2);
-                mac96(x0[0][2 * k], x1[0][2 * k], x2[0][2 * k], v.x, k0.x);
-                mac96(x0[1][2 * k], x1[1][2 * k], x2[1][2 * k], v.y, k0.y);
-                mac96(x0[0][2 * k + 1], x1[0][2 * k + 1], x2[0][2 * k + 1], v.x, k1.x);
-                mac96(x0[1][2 * k + 1], x1[1][2 * k + 1], x2[1][2 * k + 1], v.y, k1.y);
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int k = 0; k < 2 * KG; k++) acc[c][k] = U128{((u64)x1[c][k] << 32) | x0[c][k], x2[c][k]};
-    } else {
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int k = 0; k < 2 * KG; k++) acc[c][k] = U128{0, 0};
-        for (int d = 0; d < ndig; d++) {
-            const ulonglong2 v = __ldg(dp + (long)d * dstride / 2);
-#pragma unroll
-            for (int k = 0; k < KG; k++) {
-                const ulonglong2 *kp = (const ulonglong2 *)(mk.key[kg0 + k] + (long)d * kd + koff);
-                const ulonglong2 k0 = __ldg(kp), k1 = __ldg(kp + kk / 2);
-                mac128_q(acc[0][2 * k], v.x, k0.x, m.q);
-                mac128_q(acc[1][2 * k], v.y, k0.y, m.q);
-                mac128_q(acc[0][2 * k + 1], v.x, k1.x, m.q);
-                mac128_q(acc[1][2 * k + 1], v.y, k1.y, m.q);
-            }
-        }
-    }
-    const bool with_c0 = c0 && r <= level;
-    const ShoupPair w = with_c0 ? Pmod[r] : ShoupPair{0, 0};
-#pragma unroll
-    for (int c = 0; c < 2; c++) {
-        const int yc = y + c;
-        u64 pc0 = 0;
-        if (with_c0) pc0 = shoup(c0[b * c0s + (long)r * N + yc], w.w, w.wp, m.q);
-#pragma unroll
-        for (int k = 0; k < KG; k++) {
-            u64 o0 = redc(acc[c][2 * k].lo, acc[c][2 * k].hi, m), o1 = redc(acc[c][2 * k + 1].lo, acc[c][2 * k + 1].hi, m);
-            if (with_c0) o0 = addmod(o0, pc0, m.q);
-            const u32 gi = mk.ginv[kg0 + k];
-            const int x = gi == 1u ? yc : auto_index(yc, gi, logN);
-            u64 *ob = mk.out[kg0 + k] + (long)b * 2 * rows * N;
-            ob[(long)r * N + x] = o0;
-            ob[(long)(rows + r) * N + x] = o1;
-        }
-    }
-}
-
-// Permutes key rows into the layout above: out[row][pi_g(x)] = in[row][x].
+// Permutes key rows into the layout of msum.cu: out[row][pi_g(x)] = in[row][x].
 __global__ void k_permute_key(u64 *out, const u64 *in, long rows, int logN, u32 g) {
     const int N = 1 << logN;
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1161,676 +796,6 @@ void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, 
     long n = rows * (long)c->N;
     c->n_launch++;
     k_permute_key<<<nblk(n, 256), 256, 0, st>>>(out, in, rows, c->logN, g);
-}
-
-#include "multsum_tma.cuh"
-
-// Launch of the bulk-copy MultSum, persistent: as many CTAs as fit on the
-// GPU at once.  Variants: 8: 64-coefficient segments of 8 items, 8 stages;
-// 9: 128 of 4, 6 stages; 10: 256 of 2, 4 stages.
-template <int G, int S, int TW, int BI>
-static void multsum_tma_launch(Ctx *c, const MultiKeys<G> &mk, const u64 *digits, int B, int level, const u64 *c0,
-                               long c0s, cudaStream_t st) {
-    static_assert(TW * BI == 2 * MST_CONSUMERS, "two items per consumer thread");
-    static int occ[64];   // resident CTAs per SM, per device
-    const size_t smem = (size_t)S * (BI + 2 * G) * TW * 8;
-    const int dev = c->device & 63;
-    if (!occ[dev]) {
-        cudaFuncSetAttribute(k_multsum_tma<G, S, TW, BI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int nb = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_multsum_tma<G, S, TW, BI>, MST_THREADS, smem);
-        occ[dev] = nb > 0 ? nb : 1;
-    }
-    int nsm = 0;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
-    MstGeom g;
-    g.N = c->N, g.logN = c->logN, g.rows = level + 1 + c->alpha, g.level = level, g.L = c->L;
-    g.ndig = c->ndig(level), g.nprimes = c->nprimes, g.ntx = c->N / TW, g.nig = (B + BI - 1) / BI;
-    g.B = B;
-    g.ntiles = (long)g.ntx * g.rows * g.nig;
-    const long grid = std::min<long>(g.ntiles, (long)nsm * occ[dev]);
-    k_multsum_tma<G, S, TW, BI><<<(unsigned)grid, MST_THREADS, smem, st>>>(mk, digits, g, c->d_mod, c0, c0s,
-                                                                            c->d_Pmod, c->d_err);
-}
-
-// MultSum launch variants: items per CTA (BI), streaming digit loads.
-static void multsum_variant(int v, int B, int &BI, bool &stream) {
-    static const int bis[4] = {8, 4, 2, 1};
-    BI = bis[v & 3];
-    while (BI > 1 && BI > B) BI >>= 1;
-    stream = (v >> 2) & 1;
-}
-
-template <int G>
-static void multsum_launch_g(Ctx *c, int v, u64 *const *outs, const u64 *digits, const u64 *const *keys,
-                             const uint32_t *gs, int B, int level, const u64 *c0, long c0s, cudaStream_t st) {
-    MultiKeys<G> mk;
-    const u32 M = 2u * (u32)c->N;
-    for (int k = 0; k < G; k++) {
-        mk.key[k] = keys[k];
-        mk.out[k] = outs[k];
-        // inverse of the odd g modulo 2N: Newton iteration on 32-bit words
-        u32 g = gs[k], inv = g;
-        for (int it = 0; it < 5; it++) inv *= 2u - g * inv;
-        mk.ginv[k] = inv & (M - 1);
-    }
-    if ((v == 80 || v == 84) && G <= 2) {
-        // two coefficients per thread, 16-byte loads, more resident CTAs
-        if constexpr (G <= 2) {
-            constexpr int OCCV = G == 1 ? 5 : 3;
-            int BI;
-            bool stream;
-            multsum_variant(0, B, BI, stream);
-            stream = v == 84;
-            const int rows = level + 1 + c->alpha, XW = 256 / BI;
-            dim3 grid((unsigned)((c->N / 2 + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI));
-            if (stream)
-                launch_pdl(k_multsum_vec<G, true, OCCV>, dim3(grid), 256, 0, st, mk, digits, B, BI, level, c->alpha, c->L,
-                                                                   c->ndig(level), c->nprimes, c->logN, c->d_mod, c0,
-                                                                   c0s, c->d_Pmod);
-            else
-                launch_pdl(k_multsum_vec<G, false, OCCV>, dim3(grid), 256, 0, st, mk, digits, B, BI, level, c->alpha, c->L,
-                                                                    c->ndig(level), c->nprimes, c->logN, c->d_mod, c0,
-                                                                    c0s, c->d_Pmod);
-            c->n_launch++;
-            return;
-        }
-    }
-    if (v == 80 || v == 84) v = v == 80 ? 32 : 36;   // more than two rotations: the one-coefficient kernel
-    if (v == 96 || v == 97) {
-        // rotations split over warps (1 or 2 per thread), two coefficients per thread
-        const int rows = level + 1 + c->alpha;
-        auto go = [&](auto kern, int bi) {
-            dim3 grid((unsigned)((c->N / 2 + 31) / 32), (unsigned)rows, (unsigned)((B + bi - 1) / bi));
-            launch_pdl(kern, grid, 256, 0, st, mk, digits, B, level, c->alpha, c->L, c->ndig(level), c->nprimes, c->logN,
-                                       c->d_mod, c0, c0s, c->d_Pmod);
-        };
-        if (v == 97 && G % 2 == 0 && G >= 2) {
-            constexpr int KG2 = (G % 2 == 0 && G >= 2) ? 2 : 1;
-            constexpr int NG2 = G / KG2;
-            if constexpr (8 % NG2 == 0) {
-                go(k_multsum_splitv<G, KG2, 3>, 8 / NG2);
-                c->n_launch++;
-                return;
-            }
-        }
-        if constexpr (8 % G == 0) {
-            go(k_multsum_splitv<G, 1, 5>, 8 / G);
-            c->n_launch++;
-            return;
-        }
-        v = 80;   // G does not divide the warps
-    }
-    if ((v == 80 || v == 84) && G > 2) v = v == 80 ? 32 : 36;
-    if (v == 64 || v == 65) {
-        // keys split over warps: KG = 1 (64) or 2 (65, G even)
-        const int rows = level + 1 + c->alpha;
-        auto go = [&](auto kern, int bi) {
-            dim3 grid((unsigned)((c->N + 31) / 32), (unsigned)rows, (unsigned)((B + bi - 1) / bi));
-            launch_pdl(kern, grid, 256, 0, st, mk, digits, B, level, c->alpha, c->L, c->ndig(level), c->nprimes, c->logN,
-                                       c->d_mod, c0, c0s, c->d_Pmod);
-        };
-        if (v == 65 && G % 2 == 0 && G >= 2) {
-            constexpr int KG2 = (G % 2 == 0 && G >= 2) ? 2 : 1;
-            constexpr int NG2 = G / KG2;
-            if constexpr (8 % NG2 == 0) {
-                go(k_multsum_split<G, KG2, 4>, 8 / NG2);
-                c->n_launch++;
-                return;
-            }
-        }
-        if constexpr (8 % G == 0) {
-            go(k_multsum_split<G, 1, 6>, 8 / G);
-            c->n_launch++;
-            return;
-        }
-        v = 32;   // G does not divide the warps: the high-occupancy thread-per-word kernel
-    }
-    if (v >= 8 && v <= 10) {
-        if (v == 8) multsum_tma_launch<G, 8, 64, 8>(c, mk, digits, B, level, c0, c0s, st);
-        else if (v == 9) multsum_tma_launch<G, 6, 128, 4>(c, mk, digits, B, level, c0, c0s, st);
-        else multsum_tma_launch<G, 4, 256, 2>(c, mk, digits, B, level, c0, c0s, st);
-        c->n_launch++;
-        return;
-    }
-    int BI;
-    bool stream;
-    multsum_variant(v & 15, B, BI, stream);
-    const bool pf = (v & 16) != 0;
-    const int rows = level + 1 + c->alpha, XW = 256 / BI;
-    dim3 grid((unsigned)((c->N + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI));
-    // bit 5: the launch bound asks for more resident CTAs (fewer registers)
-    constexpr int OCC_HI = G <= 1 ? 8 : G <= 2 ? 6 : G <= 4 ? 4 : 3;
-    const bool hi = (v & 32) != 0;
-#define MS_LAUNCH(STR, PFD, OCC)                                                                           \
-    launch_pdl(k_multsum_multi<G, STR, PFD, OCC>, dim3(grid), 256, 0, st, mk, digits, B, BI, level, c->alpha, c->L,          \
-                                                            c->ndig(level), c->nprimes, c->logN, c->d_mod, c0, c0s, \
-                                                            c->d_Pmod)
-    if (hi) {
-        if (pf) MS_LAUNCH(false, 2, OCC_HI);
-        else if (stream) MS_LAUNCH(true, 0, OCC_HI);
-        else MS_LAUNCH(false, 0, OCC_HI);
-    } else if (stream) {
-        if (pf) MS_LAUNCH(true, 2, 0); else MS_LAUNCH(true, 0, 0);
-    } else {
-        if (pf) MS_LAUNCH(false, 2, 0); else MS_LAUNCH(false, 0, 0);
-    }
-#undef MS_LAUNCH
-    c->n_launch++;
-}
-
-static void multsum_launch(Ctx *c, int v, int G, u64 *const *outs, const u64 *digits, const u64 *const *keys,
-                           const uint32_t *gs, int B, int level, const u64 *c0, long c0s, cudaStream_t st) {
-    switch (G) {
-    case 1: multsum_launch_g<1>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    case 2: multsum_launch_g<2>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    case 3: multsum_launch_g<3>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    case 4: multsum_launch_g<4>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    case 5: multsum_launch_g<5>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    case 6: multsum_launch_g<6>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    case 7: multsum_launch_g<7>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    default: multsum_launch_g<8>(c, v, outs, digits, keys, gs, B, level, c0, c0s, st); break;
-    }
-}
-
-void launch_multsum_multi(Ctx *c, u64 *const *outs, const u64 *digits, const u64 *const *keys, const uint32_t *gs,
-                          int G, int B, int level, const u64 *c0_for_P, long c0s, cudaStream_t st) {
-    if (G <= 0) return;
-    const int rows = level + 1 + c->alpha;
-    // a launch plan: keys per launch (chunk) and the launch variant
-    auto run = [&](int chunk, int v, bool traced) {
-        for (int k0 = 0; k0 < G; k0 += chunk) {
-            const int g = std::min(chunk, G - k0);
-            cudaEvent_t e0 = nullptr;
-            if (traced) c->trace_begin(0, e0);
-            multsum_launch(c, v, g, outs + k0, digits, keys + k0, gs + k0, B, level, c0_for_P, c0s, st);
-            if (traced) {
-                // algorithmic bytes: every key (2 polys x ndig digits x rows
-                // limbs) read once, every item's digits read once for the g
-                // keys, both output polys of every (item, key) written, c0
-                // read once if fused
-                double nd = c->ndig(level), W = (double)c->N * 8.0;
-                double bytes = g * 2.0 * nd * rows * W +
-                               (double)B * (nd * rows * W + g * 2.0 * rows * W + (c0_for_P ? (level + 1) * W : 0));
-                c->trace_end(0, e0, bytes, (double)B * nd * rows * c->N * 2.0 * g);
-            }
-        }
-    };
-    int chunk = std::min(G, kMultSumMaxKeys), v = 0;  // default: 8 keys, 8 items per CTA, cached loads
-    if (c->force_multsum >= 0) {
-        v = c->force_multsum;
-    } else if (c->autotune) {
-        auto key3 = std::make_tuple(level, B, G);
-        auto it = c->tune_multsum.find(key3);
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        cudaStreamIsCapturing(st, &cap);
-        if (it != c->tune_multsum.end()) {
-            chunk = it->second >> 8, v = it->second & 255;
-        } else if (cap == cudaStreamCaptureStatusNone) {
-            // time every (keys per launch, variant) twice on these very
-            // launches (the outputs do not depend on the plan); keep the fastest
-            cudaEvent_t a = c->ev_get(), b = c->ev_get();
-            float best = 1e30f;
-            std::set<std::tuple<int, int, bool>> seen;
-            for (int ch : {8, 4, 2, 1}) {
-                const int cc = std::min(ch, G);
-                for (int cand : {0, 1, 2, 3, 4, 5, 6, 7, 16, 20, 32, 36, 48, 64, 65, 80, 84, 96, 97, 8, 9, 10}) {
-                    int BI;
-                    bool stream;
-                    multsum_variant(cand & 15, B, BI, stream);
-                    if (cand >= 8) BI = 100 + cand;   // the bulk-copy and prefetching kernels: their own entries
-                    if (!seen.insert(std::make_tuple(cc, BI, stream)).second) continue;
-                    float t = 1e30f;
-                    for (int rep = 0; rep < 2; rep++) {
-                        cudaEventRecord(a, st);
-                        run(cc, cand, false);
-                        cudaEventRecord(b, st);
-                        cudaEventSynchronize(b);
-                        float ms = 0;
-                        cudaEventElapsedTime(&ms, a, b);
-                        t = std::min(t, ms);
-                    }
-                    if (t < best) best = t, chunk = cc, v = cand;
-                    char line[128];
-                    snprintf(line, sizeof line, "multsum level %d B %d G %d chunk %d BI %d stream %d ms %.4f\n",
-                             level, B, G, cc, BI, (int)stream, t);
-                    c->tune_log += line;
-                }
-            }
-            c->ev_free.push_back(a);
-            c->ev_free.push_back(b);
-            c->tune_multsum[key3] = (chunk << 8) | v;
-        }
-    }
-    run(chunk, v, true);
-}
-
-// MultSum + Permute of the G giants of a BSGS transform, summed: every giant
-// has its own digits, key and automorphism, and
-//   out[x] = in[x] + sum_g (T_g[y_g] + P c0_g[y_g]),  y_g = pi_g(x),
-// T_g as above (keys permuted).  A thread owns the output word, so the sum over
-// giants and digits is one accumulation with one reduction; the words of a
-// giant are read at permuted positions inside aligned 32-word blocks.  digits:
-// [G][B][ndig][rows][N]; c0: [G][B] ciphertexts at stride c0s; in (may be null, or
-// equal out), out: [B][2][rows][N].
-struct GiantArgs {
-    const u64 *key[kMaxGiants];
-    u32 g[kMaxGiants];
-};
-__global__ void __launch_bounds__(256, 4) k_multsum_giants(const __grid_constant__ GiantArgs ga, int G, u64 *out,
-                                                           const u64 *in, const u64 *digits, int B, int BI, int level,
-                                                           int alpha, int L, int ndig, int nprimes, int logN,
-                                                           const ModQ *mods, const u64 *c0, long c0s,
-                                                           const ShoupPair *Pmod) {
-    pdl_trigger();
-    pdl_wait();
-    const int N = 1 << logN;
-    const int XW = 256 / BI;
-    const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
-    const int x = blockIdx.x * XW + tx;
-    const int r = blockIdx.y;
-    const int b = blockIdx.z * BI + ti;
-    if (b >= B || x >= N) return;
-    const int rows = level + 1 + alpha;
-    const int kr = r <= level ? r : L + 1 + (r - level - 1);
-    const ModQ m = mods[kr];
-    const long ds = (long)rows * N, kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    const bool q_row = r <= level;
-    const ShoupPair w = q_row ? Pmod[r] : ShoupPair{0, 0};
-    u64 pc = 0;
-    U128 a0 = {0, 0}, a1 = {0, 0};
-    u32 x0 = 0, x1 = 0, x2 = 0, z0 = 0, z1 = 0, z2 = 0;
-    const bool small = m.q < (1ull << 42);   // uniform over the CTA; G ndig <= 2^12 products below 2^84
-    for (int g = 0; g < G; g++) {
-        const int y = auto_index(x, ga.g[g], logN);
-        const u64 *dp = digits + ((long)g * B + b) * ndig * ds + (long)r * N + y;
-        const u64 *kp = ga.key[g] + (long)kr * N + y;
-        if (small) {
-            for (int d = 0; d < ndig; d++) {
-                const u64 v = __ldg(dp + d * ds);
-                mac96(x0, x1, x2, v, __ldg(kp + d * kd));
-                mac96(z0, z1, z2, v, __ldg(kp + d * kd + kk));
-            }
-        } else {
-            for (int d = 0; d < ndig; d++) {
-                const u64 v = __ldg(dp + d * ds);
-                mac128_q(a0, v, __ldg(kp + d * kd), m.q);
-                mac128_q(a1, v, __ldg(kp + d * kd + kk), m.q);
-            }
-        }
-        if (q_row) pc = addmod(pc, shoup(c0[((long)g * B + b) * c0s + (long)r * N + y], w.w, w.wp, m.q), m.q);
-    }
-    if (small) a0 = U128{((u64)x1 << 32) | x0, x2}, a1 = U128{((u64)z1 << 32) | z0, z2};
-    u64 o0 = addmod(redc(a0.lo, a0.hi, m), pc, m.q), o1 = redc(a1.lo, a1.hi, m);
-    const long o = (long)b * 2 * ds + (long)r * N + x;
-    if (in) o0 = addmod(o0, in[o], m.q), o1 = addmod(o1, in[o + ds], m.q);
-    out[o] = o0;
-    out[o + ds] = o1;
-}
-void launch_multsum_giants(Ctx *c, u64 *out, const u64 *in, const u64 *digits, const u64 *const *keys,
-                           const uint32_t *gs, int G, int B, int level, const u64 *c0, long c0s, cudaStream_t st) {
-    GiantArgs ga;
-    for (int g = 0; g < G; g++) ga.key[g] = keys[g], ga.g[g] = gs[g];
-    int BI = 8;
-    while (BI > 1 && BI > B) BI >>= 1;
-    const int XW = 256 / BI, rows = level + 1 + c->alpha, nd = c->ndig(level);
-    c->n_launch++;
-    cudaEvent_t e0;
-    c->trace_begin(0, e0);
-    launch_pdl(k_multsum_giants, dim3((unsigned)((c->N + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI)), 256, 0, st, 
-        ga, G, out, in, digits, B, BI, level, c->alpha, c->L, nd, c->nprimes, c->logN, c->d_mod, c0, c0s, c->d_Pmod);
-    const double W = 8.0 * c->N;
-    c->trace_end(0, e0, W * (G * 2.0 * nd * rows + (double)B * (G * ((double)nd * rows + level + 1) + (in ? 4.0 : 2.0) * rows)),
-                 (double)B * G * nd * rows * c->N * 2.0);
-}
-
-// The inner product with one key on the rows of Q alone: digits [B][ndig][l+1][N]
-// -> out [B][2][l+1][N] (the key without permutation).
-void launch_multsum_q(Ctx *c, u64 *out, const u64 *digits, const u64 *key, int B, int level, cudaStream_t st) {
-    MultiKeys<1> mk;
-    mk.key[0] = key, mk.out[0] = out, mk.ginv[0] = 1;
-    int BI = 8;
-    while (BI > 1 && BI > B) BI >>= 1;
-    const int XW = 256 / BI, nq = level + 1, nd = c->ndig(level);
-    c->n_launch++;
-    cudaEvent_t e0;
-    c->trace_begin(0, e0);
-    launch_pdl(k_multsum_vec<1, false, 5>, dim3((unsigned)((c->N / 2 + XW - 1) / XW), (unsigned)nq, (unsigned)((B + BI - 1) / BI)), 256, 0, st, mk, digits, B, BI, level, 0, c->L, nd, c->nprimes, c->logN, c->d_mod,
-                                               nullptr, 0, nullptr);
-    c->trace_end(0, e0, 8.0 * c->N * nq * (2.0 * nd + (double)B * (nd + 2)), (double)B * nd * nq * c->N * 2.0);
-}
-
-void launch_multsum(Ctx *c, u64 *out, const u64 *digits, const u64 *key, uint32_t g, int B, int level,
-                    const u64 *c0_for_P, long c0s, cudaStream_t st) {
-    launch_multsum_multi(c, &out, digits, &key, &g, 1, B, level, c0_for_P, c0s, st);
-}
-
-// ------------------------------------------------- C^k babies with masks
-// For k = n1 g + b (b >= 1) the product's C^k step (Sec. 4.1, Table 1
-// "Optimized C^k") needs, over Q_l P,
-//   S_b = m_k (.) rot_qp(A_g; b) + m'_k (.) rot_qp(A'_g; b),
-// rot_qp(X; b) = <kappa_b(digits of X), rtk_b> + (P kappa_b(c0 of X), 0), m_k
-// and m'_k the two column masks (Montgomery form).  The two sources use the
-// same rotation keys: each key word is loaded once for both, and the two
-// hoisted rotations stay in registers, so only S_b reaches memory.  The
-// words equal those of two MultSum launches followed by the masked sum
-// (every value is a canonical residue).
-template <int G>
-struct CkArgs {
-    const u64 *key[G];
-    u64 *out[G];
-    const u64 *m1[G], *m2[G];   // masks over Q_l P, [rows][N]
-    u32 ginv[G];
-};
-
-template <int G>
-__global__ void __launch_bounds__(256, G <= 1 ? 4 : G <= 2 ? 3 : 2)
-    k_multsum_ck(const __grid_constant__ CkArgs<G> ck, const u64 *dig1, const u64 *dig2, int B, int BI, int level,
-                 int alpha, int L, int ndig, int nprimes, int logN, const ModQ *mods, const u64 *c01,
-                 const u64 *c02, long c0s, const ShoupPair *Pmod) {
-    pdl_trigger();
-    pdl_wait();
-    const int N = 1 << logN;
-    const int XW = 256 / BI;
-    const int tx = threadIdx.x % XW, ti = threadIdx.x / XW;
-    const int y = blockIdx.x * XW + tx;
-    const int r = blockIdx.y;
-    const int b = blockIdx.z * BI + ti;
-    if (b >= B || y >= N) return;
-    const int rows = level + 1 + alpha;
-    const int kr = r <= level ? r : L + 1 + (r - level - 1);   // the row's global prime
-    const ModQ m = mods[kr];
-    const long dstride = (long)rows * N;
-    const u64 *dp1 = dig1 + (long)b * ndig * dstride + (long)r * N + y;
-    const u64 *dp2 = dig2 + (long)b * ndig * dstride + (long)r * N + y;
-    const long koff = (long)kr * N + y, kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    U128 acc[G][4];   // (source 1: poly 0, poly 1; source 2: poly 0, poly 1) per key
-    if (m.q < (1ull << 42)) {
-        // residues below 2^42 (uniform over the CTA): 96-bit accumulation
-        u32 x0[4 * G], x1[4 * G], x2[4 * G];
-#pragma unroll
-        for (int k = 0; k < 4 * G; k++) x0[k] = 0, x1[k] = 0, x2[k] = 0;
-        for (int d = 0; d < ndig; d++) {
-            const u64 v1 = __ldg(dp1 + (long)d * dstride), v2 = __ldg(dp2 + (long)d * dstride);
-#pragma unroll
-            for (int k = 0; k < G; k++) {
-                const u64 *kp = ck.key[k] + (long)d * kd + koff;
-                const u64 k0 = __ldg(kp), k1 = __ldg(kp + kk);
-                mac96(x0[4 * k], x1[4 * k], x2[4 * k], v1, k0);
-                mac96(x0[4 * k + 1], x1[4 * k + 1], x2[4 * k + 1], v1, k1);
-                mac96(x0[4 * k + 2], x1[4 * k + 2], x2[4 * k + 2], v2, k0);
-                mac96(x0[4 * k + 3], x1[4 * k + 3], x2[4 * k + 3], v2, k1);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < G; k++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) acc[k][j] = U128{((u64)x1[4 * k + j] << 32) | x0[4 * k + j], x2[4 * k + j]};
-    } else {
-#pragma unroll
-        for (int k = 0; k < G; k++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) acc[k][j] = U128{0, 0};
-        for (int d = 0; d < ndig; d++) {
-            const u64 v1 = __ldg(dp1 + (long)d * dstride), v2 = __ldg(dp2 + (long)d * dstride);
-#pragma unroll
-            for (int k = 0; k < G; k++) {
-                const u64 *kp = ck.key[k] + (long)d * kd + koff;
-                const u64 k0 = __ldg(kp), k1 = __ldg(kp + kk);
-                mac128_q(acc[k][0], v1, k0, m.q);
-                mac128_q(acc[k][1], v1, k1, m.q);
-                mac128_q(acc[k][2], v2, k0, m.q);
-                mac128_q(acc[k][3], v2, k1, m.q);
-            }
-        }
-    }
-    u64 pc1 = 0, pc2 = 0;
-    if (r <= level) {
-        const ShoupPair w = Pmod[r];
-        pc1 = shoup(c01[b * c0s + (long)r * N + y], w.w, w.wp, m.q);
-        pc2 = shoup(c02[b * c0s + (long)r * N + y], w.w, w.wp, m.q);
-    }
-#pragma unroll
-    for (int k = 0; k < G; k++) {
-        const u64 a10 = addmod(redc(acc[k][0].lo, acc[k][0].hi, m), pc1, m.q);
-        const u64 a11 = redc(acc[k][1].lo, acc[k][1].hi, m);
-        const u64 a20 = addmod(redc(acc[k][2].lo, acc[k][2].hi, m), pc2, m.q);
-        const u64 a21 = redc(acc[k][3].lo, acc[k][3].hi, m);
-        const int x = ck.ginv[k] == 1u ? y : auto_index(y, ck.ginv[k], logN);
-        const u64 w1 = __ldg(ck.m1[k] + (long)r * N + x), w2 = __ldg(ck.m2[k] + (long)r * N + x);
-        U128 s0 = {0, 0}, s1 = {0, 0};   // two products below q^2: below q 2^64
-        mac128(s0, w1, a10);
-        mac128(s0, w2, a20);
-        mac128(s1, w1, a11);
-        mac128(s1, w2, a21);
-        u64 *ob = ck.out[k] + (long)b * 2 * rows * N;
-        ob[(long)r * N + x] = redc(s0.lo, s0.hi, m);
-        ob[(long)(rows + r) * N + x] = redc(s1.lo, s1.hi, m);
-    }
-}
-
-// The same with the rotations split over the warps: warp w takes rotation
-// w / BI of items blockIdx.z BI + w % BI (BI = 8 / G), two adjacent
-// coefficients per thread with 16-byte digit, key and store accesses, so a
-// thread holds 8 accumulators whatever G is (more resident warps than
-// k_multsum_ck at G >= 2).
-template <int G>
-__global__ void __launch_bounds__(256, 3)
-    k_multsum_cks(const __grid_constant__ CkArgs<G> ck, const u64 *dig1, const u64 *dig2, int B, int level,
-                  int alpha, int L, int ndig, int nprimes, int logN, const ModQ *mods, const u64 *c01,
-                  const u64 *c02, long c0s, const ShoupPair *Pmod) {
-    pdl_trigger();
-    pdl_wait();
-    constexpr int BI = 8 / G;
-    const int N = 1 << logN;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int kq = wid / BI, bi = wid % BI;
-    // one item per CTA (G = 8): the items are the fastest grid index, so the
-    // CTAs of the B items that read the same key words run together
-    const int xb = BI == 1 ? (int)(blockIdx.x / B) : (int)blockIdx.x;
-    const int y = 2 * (xb * 32 + lane);
-    const int r = blockIdx.y;
-    const int b = BI == 1 ? (int)(blockIdx.x % B) : (int)blockIdx.z * BI + bi;
-    if (b >= B || y >= N) return;
-    const int rows = level + 1 + alpha;
-    const int kr = r <= level ? r : L + 1 + (r - level - 1);
-    const ModQ m = mods[kr];
-    const long dstride = (long)rows * N;
-    const ulonglong2 *dp1 = (const ulonglong2 *)(dig1 + (long)b * ndig * dstride + (long)r * N + y);
-    const ulonglong2 *dp2 = (const ulonglong2 *)(dig2 + (long)b * ndig * dstride + (long)r * N + y);
-    const long koff = (long)kr * N + y, kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    const u64 *key = ck.key[kq];
-    U128 acc[2][4];   // [coefficient][source 1 poly 0, poly 1, source 2 poly 0, poly 1]
-    if (m.q < (1ull << 42)) {
-        u32 x0[2][4], x1[2][4], x2[2][4];
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) x0[c][j] = 0, x1[c][j] = 0, x2[c][j] = 0;
-        for (int d = 0; d < ndig; d++) {
-            const ulonglong2 v1 = __ldg(dp1 + (long)d * dstride / 2), v2 = __ldg(dp2 + (long)d * dstride / 2);
-            const ulonglong2 *kp = (const ulonglong2 *)(key + (long)d * kd + koff);
-            const ulonglong2 k0 = __ldg(kp), k1 = __ldg(kp + kk / 2);
-            mac96(x0[0][0], x1[0][0], x2[0][0], v1.x, k0.x);
-            mac96(x0[1][0], x1[1][0], x2[1][0], v1.y, k0.y);
-            mac96(x0[0][1], x1[0][1], x2[0][1], v1.x, k1.x);
-            mac96(x0[1][1], x1[1][1], x2[1][1], v1.y, k1.y);
-            mac96(x0[0][2], x1[0][2], x2[0][2], v2.x, k0.x);
-            mac96(x0[1][2], x1[1][2], x2[1][2], v2.y, k0.y);
-            mac96(x0[0][3], x1[0][3], x2[0][3], v2.x, k1.x);
-            mac96(x0[1][3], x1[1][3], x2[1][3], v2.y, k1.y);
-        }
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) acc[c][j] = U128{((u64)x1[c][j] << 32) | x0[c][j], x2[c][j]};
-    } else {
-#pragma unroll
-        for (int c = 0; c < 2; c++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) acc[c][j] = U128{0, 0};
-        for (int d = 0; d < ndig; d++) {
-            const ulonglong2 v1 = __ldg(dp1 + (long)d * dstride / 2), v2 = __ldg(dp2 + (long)d * dstride / 2);
-            const ulonglong2 *kp = (const ulonglong2 *)(key + (long)d * kd + koff);
-            const ulonglong2 k0 = __ldg(kp), k1 = __ldg(kp + kk / 2);
-            mac128_q(acc[0][0], v1.x, k0.x, m.q);
-            mac128_q(acc[1][0], v1.y, k0.y, m.q);
-            mac128_q(acc[0][1], v1.x, k1.x, m.q);
-            mac128_q(acc[1][1], v1.y, k1.y, m.q);
-            mac128_q(acc[0][2], v2.x, k0.x, m.q);
-            mac128_q(acc[1][2], v2.y, k0.y, m.q);
-            mac128_q(acc[0][3], v2.x, k1.x, m.q);
-            mac128_q(acc[1][3], v2.y, k1.y, m.q);
-        }
-    }
-    const ShoupPair wP = r <= level ? Pmod[r] : ShoupPair{0, 0};
-    u64 *ob = ck.out[kq] + (long)b * 2 * rows * N;
-    const u32 gi = ck.ginv[kq];
-#pragma unroll
-    for (int c = 0; c < 2; c++) {
-        const int yc = y + c;
-        u64 pc1 = 0, pc2 = 0;
-        if (r <= level) {
-            pc1 = shoup(c01[b * c0s + (long)r * N + yc], wP.w, wP.wp, m.q);
-            pc2 = shoup(c02[b * c0s + (long)r * N + yc], wP.w, wP.wp, m.q);
-        }
-        const u64 a10 = addmod(redc(acc[c][0].lo, acc[c][0].hi, m), pc1, m.q);
-        const u64 a11 = redc(acc[c][1].lo, acc[c][1].hi, m);
-        const u64 a20 = addmod(redc(acc[c][2].lo, acc[c][2].hi, m), pc2, m.q);
-        const u64 a21 = redc(acc[c][3].lo, acc[c][3].hi, m);
-        const int x = gi == 1u ? yc : auto_index(yc, gi, logN);
-        const u64 w1 = __ldg(ck.m1[kq] + (long)r * N + x), w2 = __ldg(ck.m2[kq] + (long)r * N + x);
-        U128 s0 = {0, 0}, s1 = {0, 0};
-        mac128(s0, w1, a10);
-        mac128(s0, w2, a20);
-        mac128(s1, w1, a11);
-        mac128(s1, w2, a21);
-        ob[(long)r * N + x] = redc(s0.lo, s0.hi, m);
-        ob[(long)(rows + r) * N + x] = redc(s1.lo, s1.hi, m);
-    }
-}
-
-template <int G>
-static void multsum_ck_launch_g(Ctx *c, int BI, u64 *const *outs, const u64 *dig1, const u64 *dig2,
-                                const u64 *const *keys, const uint32_t *gs, const u64 *const *m1,
-                                const u64 *const *m2, int B, int level, const u64 *c01, const u64 *c02, long c0s,
-                                cudaStream_t st) {
-    CkArgs<G> ck;
-    const u32 M = 2u * (u32)c->N;
-    for (int k = 0; k < G; k++) {
-        ck.key[k] = keys[k];
-        ck.out[k] = outs[k];
-        ck.m1[k] = m1[k];
-        ck.m2[k] = m2[k];
-        u32 g = gs[k], inv = g;   // inverse of the odd g modulo 2N (Newton on 32-bit words)
-        for (int it = 0; it < 5; it++) inv *= 2u - g * inv;
-        ck.ginv[k] = inv & (M - 1);
-    }
-    const int rows = level + 1 + c->alpha;
-    if constexpr (G > 4) BI = 0;   // eight rotations: the split form only
-    if constexpr (8 % G == 0) {
-        if (BI == 0) {   // rotations split over the warps
-            constexpr int SBI = 8 / G;
-            const unsigned xblocks = (unsigned)((c->N / 2 + 31) / 32);
-            const dim3 grid = SBI == 1 ? dim3(xblocks * (unsigned)B, (unsigned)rows, 1)
-                                       : dim3(xblocks, (unsigned)rows, (unsigned)((B + SBI - 1) / SBI));
-            launch_pdl(k_multsum_cks<G>, dim3(grid), 256, 0, st, ck, dig1, dig2, B, level, c->alpha, c->L, c->ndig(level),
-                                                   c->nprimes, c->logN, c->d_mod, c01, c02, c0s, c->d_Pmod);
-            c->n_launch++;
-            return;
-        }
-    }
-    if constexpr (G <= 4) {
-        if (BI == 0) BI = 8;   // G does not divide the warps
-        const int XW = 256 / BI;
-        dim3 grid((unsigned)((c->N + XW - 1) / XW), (unsigned)rows, (unsigned)((B + BI - 1) / BI));
-        launch_pdl(k_multsum_ck<G>, dim3(grid), 256, 0, st, ck, dig1, dig2, B, BI, level, c->alpha, c->L, c->ndig(level),
-                                              c->nprimes, c->logN, c->d_mod, c01, c02, c0s, c->d_Pmod);
-        c->n_launch++;
-    }
-}
-
-void launch_multsum_ck(Ctx *c, u64 *const *outs, const u64 *dig1, const u64 *dig2, const u64 *const *keys,
-                       const uint32_t *gs, const u64 *const *m1, const u64 *const *m2, int G, int B, int level,
-                       const u64 *c01, const u64 *c02, long c0s, cudaStream_t st) {
-    if (G <= 0) return;
-    const int rows = level + 1 + c->alpha;
-    auto run = [&](int chunk, int BI, bool traced) {
-        for (int k0 = 0, g = 0; k0 < G; k0 += g) {
-            g = std::min(chunk, G - k0);
-            if (g > 4 && g != 8) g = 4;   // launches of 1..4 or 8 rotations
-            cudaEvent_t e0 = nullptr;
-            if (traced) c->trace_begin(0, e0);
-            switch (g) {
-            case 8: multsum_ck_launch_g<8>(c, 0, outs + k0, dig1, dig2, keys + k0, gs + k0, m1 + k0, m2 + k0, B, level, c01, c02, c0s, st); break;
-            case 1: multsum_ck_launch_g<1>(c, BI, outs + k0, dig1, dig2, keys + k0, gs + k0, m1 + k0, m2 + k0, B, level, c01, c02, c0s, st); break;
-            case 2: multsum_ck_launch_g<2>(c, BI, outs + k0, dig1, dig2, keys + k0, gs + k0, m1 + k0, m2 + k0, B, level, c01, c02, c0s, st); break;
-            case 3: multsum_ck_launch_g<3>(c, BI, outs + k0, dig1, dig2, keys + k0, gs + k0, m1 + k0, m2 + k0, B, level, c01, c02, c0s, st); break;
-            default: multsum_ck_launch_g<4>(c, BI, outs + k0, dig1, dig2, keys + k0, gs + k0, m1 + k0, m2 + k0, B, level, c01, c02, c0s, st); break;
-            }
-            if (traced) {
-                // algorithmic bytes: every key and every mask read once, both
-                // sources' digits and c0 read once per item, one output per
-                // (item, key)
-                const double nd = c->ndig(level), W = (double)c->N * 8.0;
-                const double bytes = g * (2.0 * nd * rows + 2.0 * rows) * W +
-                                     (double)B * (2.0 * nd * rows * W + 2.0 * (level + 1) * W + g * 2.0 * rows * W);
-                c->trace_end(0, e0, bytes, (double)B * nd * rows * c->N * 4.0 * g);
-            }
-        }
-    };
-    int chunk = std::min(G, 4), BI = std::min(B, 8);
-    while (BI > 1 && BI > B) BI >>= 1;
-    if (c->force_multsum >= 0) {
-        // a pinned MultSum variant: 96 / 97 (rotations split over the warps)
-        // select the split form here too (97: launches of 8 rotations where 8
-        // remain), every other one the thread-per-word form
-        if (c->force_multsum == 96 || c->force_multsum == 97) BI = 0;
-        if (c->force_multsum == 97) chunk = std::min(G, 8);
-    } else if (c->autotune) {
-        auto key3 = std::make_tuple(level, B, G);
-        auto it = c->tune_ck.find(key3);
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        cudaStreamIsCapturing(st, &cap);
-        if (it != c->tune_ck.end()) {
-            chunk = it->second >> 8, BI = it->second & 255;
-        } else if (cap == cudaStreamCaptureStatusNone) {
-            // time every (keys per launch, items per CTA) twice on these very
-            // launches (the outputs do not depend on the plan); keep the fastest
-            cudaEvent_t a = c->ev_get(), b = c->ev_get();
-            float best = 1e30f;
-            std::set<std::pair<int, int>> seen;
-            for (int ch : {8, 4, 2, 1}) {
-                for (int bi : {8, 4, 2, 1, 0}) {   // 0: rotations split over the warps
-                    const int cc = std::min(ch, G);
-                    int bb = bi;
-                    while (bb > 1 && bb > B) bb >>= 1;
-                    if (bi == 0 && (8 % cc) && cc <= 4) continue;
-                    if (cc > 4 && bi != 0) continue;   // more than 4 rotations: the split form only
-                    if (!seen.insert(std::make_pair(cc, bb)).second) continue;
-                    float t = 1e30f;
-                    for (int rep = 0; rep < 2; rep++) {
-                        cudaEventRecord(a, st);
-                        run(cc, bb, false);
-                        cudaEventRecord(b, st);
-                        cudaEventSynchronize(b);
-                        float ms = 0;
-                        cudaEventElapsedTime(&ms, a, b);
-                        t = std::min(t, ms);
-                    }
-                    if (t < best) best = t, chunk = cc, BI = bb;
-                    char line[128];
-                    snprintf(line, sizeof line, "multsum_ck level %d B %d G %d chunk %d BI %d ms %.4f\n", level, B,
-                             G, cc, bb, t);
-                    c->tune_log += line;
-                }
-            }
-            c->ev_free.push_back(a);
-            c->ev_free.push_back(b);
-            c->tune_ck[key3] = (chunk << 8) | BI;
-        }
-    }
-    run(chunk, BI, true);
 }
 
 // ------------------------------------------------------ double hoisting
@@ -1851,10 +816,10 @@ struct PmulArgs {
     unsigned char ri[kMaxPmulTerms];
     short first[kMaxPmulSums + 1];
 };
-template <bool WIDE>
+// FQ: plaintexts plain and centred, sums as in MultSum; else in Montgomery form.
+template <bool FQ, bool WIDE>
 __device__ __forceinline__ void pmul_item(const PmulArgs &pa, int t0, int t1, long idx, long per, long ro, u64 *ob,
-                                          const ModQ &m) {
-    U128 a[2][2] = {};
+                                          const ModQ &m, const ModF &f) {
     ulonglong2 p, r0, r1;
     auto load = [&](int t) {
         p = __ldg((const ulonglong2 *)(pa.pt[t] + idx));
@@ -1862,34 +827,60 @@ __device__ __forceinline__ void pmul_item(const PmulArgs &pa, int t0, int t1, lo
         r0 = __ldg((const ulonglong2 *)rb);
         r1 = __ldg((const ulonglong2 *)(rb + per));
     };
+    u64 o[2][2];
     if (t0 < t1) load(t0);
-    for (int t = t0; t < t1; t++) {
-        const ulonglong2 pv = p, v0 = r0, v1 = r1;
-        if (t + 1 < t1) load(t + 1);
-        if (WIDE) {
-            mac128_q(a[0][0], pv.x, v0.x, m.q), mac128_q(a[0][1], pv.y, v0.y, m.q);
-            mac128_q(a[1][0], pv.x, v1.x, m.q), mac128_q(a[1][1], pv.y, v1.y, m.q);
-        } else {
-            mac128(a[0][0], pv.x, v0.x), mac128(a[0][1], pv.y, v0.y);
-            mac128(a[1][0], pv.x, v1.x), mac128(a[1][1], pv.y, v1.y);
+    if constexpr (FQ) {
+        const FqMacC c(f, m.q);
+        FqMac a[2][2] = {};
+        for (int t = t0, run = 0; t < t1; t++, run++) {
+            const ulonglong2 pv = p, v0 = r0, v1 = r1;
+            if (t + 1 < t1) load(t + 1);
+            if (run == c.lim) {
+                run = 0;
+#pragma unroll
+                for (int i = 0; i < 4; i++) a[i >> 1][i & 1].fold(c, f);
+            }
+            const float p0 = FqMac::part(pv.x), p1 = FqMac::part(pv.y);
+            a[0][0].add(v0.x, FqMac::part(v0.x), pv.x, p0), a[0][1].add(v0.y, FqMac::part(v0.y), pv.y, p1);
+            a[1][0].add(v1.x, FqMac::part(v1.x), pv.x, p0), a[1][1].add(v1.y, FqMac::part(v1.y), pv.y, p1);
         }
+#pragma unroll
+        for (int i = 0; i < 4; i++) o[i >> 1][i & 1] = a[i >> 1][i & 1].get(c, m.q, f);
+    } else {
+        U128 a[2][2] = {};
+        for (int t = t0; t < t1; t++) {
+            const ulonglong2 pv = p, v0 = r0, v1 = r1;
+            if (t + 1 < t1) load(t + 1);
+            if (WIDE) {
+                mac128_q(a[0][0], pv.x, v0.x, m.q), mac128_q(a[0][1], pv.y, v0.y, m.q);
+                mac128_q(a[1][0], pv.x, v1.x, m.q), mac128_q(a[1][1], pv.y, v1.y, m.q);
+            } else {
+                mac128(a[0][0], pv.x, v0.x), mac128(a[0][1], pv.y, v0.y);
+                mac128(a[1][0], pv.x, v1.x), mac128(a[1][1], pv.y, v1.y);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++) o[i >> 1][i & 1] = redc(a[i >> 1][i & 1].lo, a[i >> 1][i & 1].hi, m);
     }
 #pragma unroll
-    for (int c = 0; c < 2; c++)
-        *(ulonglong2 *)(ob + c * per + idx) =
-            make_ulonglong2(redc(a[c][0].lo, a[c][0].hi, m), redc(a[c][1].lo, a[c][1].hi, m));
+    for (int c = 0; c < 2; c++) *(ulonglong2 *)(ob + c * per + idx) = make_ulonglong2(o[c][0], o[c][1]);
 }
 __global__ void __launch_bounds__(128) k_pmul_acc(u64 *out, long out_s, const __grid_constant__ PmulArgs pa, int B,
-                                                  int rows, int logN, long Rs, RowMap qp, const ModQ *mods) {
+                                                  int rows, int logN, long Rs, RowMap qp, const ModQ *mods,
+                                                  const ModF *modf) {
     pdl_trigger();
     pdl_wait();
     const long idx = 2 * ((long)blockIdx.y * 128 + threadIdx.x), per = (long)rows << logN;   // 256 | N
-    const ModQ m = mods[qp.at32((unsigned)(idx >> logN))];
+    const int pi = qp.at32((unsigned)(idx >> logN));
+    const ModQ m = mods[pi];
+    const ModF f = modf[pi];
     const int t0 = pa.first[blockIdx.x], t1 = pa.first[blockIdx.x + 1];
     u64 *o = out + blockIdx.x * out_s;
-    for (int b = 0; b < B; b++) {
-        if (m.q >= (1ull << 59)) pmul_item<true>(pa, t0, t1, idx, per, b * Rs, o + (long)b * 2 * per, m);   // uniform
-        else pmul_item<false>(pa, t0, t1, idx, per, b * Rs, o + (long)b * 2 * per, m);
+    for (int b = 0; b < B; b++) {   // the branches are uniform over the CTA
+        u64 *ob = o + (long)b * 2 * per;
+        if (f.on) pmul_item<true, false>(pa, t0, t1, idx, per, b * Rs, ob, m, f);
+        else if (m.q >= (1ull << 59)) pmul_item<false, true>(pa, t0, t1, idx, per, b * Rs, ob, m, f);
+        else pmul_item<false, false>(pa, t0, t1, idx, per, b * Rs, ob, m, f);
     }
 }
 void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const int *first, int sums,
@@ -1904,7 +895,7 @@ void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const
             a.pt[t - first[y0]] = terms[t].pt, a.ri[t - first[y0]] = (unsigned char)terms[t].r;
         c->n_launch++;
         launch_pdl(k_pmul_acc, dim3((unsigned)(y1 - y0), (unsigned)((long)rows * c->N / 256)), 128, 0, st, 
-            out + y0 * out_s, out_s, a, B, rows, c->logN, Rs, c->map_qp(level), c->d_mod);
+            out + y0 * out_s, out_s, a, B, rows, c->logN, Rs, c->map_qp(level), c->d_mod, c->d_modf);
     }
 }
 

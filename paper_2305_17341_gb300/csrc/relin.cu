@@ -34,12 +34,6 @@ struct PairIdx {
     short a[kPairs], b[kPairs];
 };
 
-// bits of b / (q 2^8) for 0 <= b < 2^41: c = 2^6 / q
-__device__ __forceinline__ ulonglong2 fq_var(u64 b, float c) {
-    const float f = __fmul_rn(__int2float_rn((int)__funnelshift_r((u32)b, (u32)(b >> 32), 14)), c);
-    return make_ulonglong2(b, __float_as_uint(f));
-}
-
 template <bool D2K>
 __global__ void __launch_bounds__(256) k_tensor_run(u64 *d01, u64 *D2, u64 *d2, const u64 *a, const u64 *b, int K,
                                                     int P, int p0, int nA, int nB, int limbs, int logN, long bs,
@@ -66,7 +60,7 @@ __global__ void __launch_bounds__(256) k_tensor_run(u64 *d01, u64 *D2, u64 *d2, 
 #pragma unroll
             for (int j = 0; j < 2; j++) {
                 const u64 u0 = j ? a0.y : a0.x, u1 = j ? a1.y : a1.x;
-                const ulonglong2 v0 = fq_var(j ? b0.y : b0.x, c), v1 = fq_var(j ? b1.y : b1.x, c);
+                const ulonglong2 v0 = fq_svar(j ? b0.y : b0.x, c), v1 = fq_svar(j ? b1.y : b1.x, c);
                 // each product below q in magnitude: 16 terms stay below 17 q
                 if (k && !(k & 7)) s0[j] = fq_red(s0[j], f), s1[j] = fq_red(s1[j], f), s2[j] = fq_red(s2[j], f);
                 s0[j] += fq_mul(u0, v0, f);
@@ -149,7 +143,7 @@ __global__ void __launch_bounds__(256) k_tensor_ptrs(u64 *d01, u64 *d2, const __
     u64 o0, o1, o2;
     if (f.on) {   // uniform over the CTA
         const float c = f.qi * 1.4901161193847656e-08f;   // 2^6 / q
-        const ulonglong2 v0 = fq_var(b0, c), v1 = fq_var(b1, c);
+        const ulonglong2 v0 = fq_svar(b0, c), v1 = fq_svar(b1, c);
         o0 = fq_pos(fq_mul(a0, v0, f), m.q);
         o1 = fq_pos(fq_red(fq_mul(a0, v1, f) + fq_mul(a1, v0, f), f), m.q);
         o2 = fq_pos(fq_mul(a1, v1, f), m.q);
@@ -249,37 +243,6 @@ __global__ void __launch_bounds__(256) k_relin_up(const u64 *d2, u64 *SY, u64 *d
                 SY[(((long)p * 2 + 1) * nq + i0 + s) * N + x] = hi[s];
             }
     }
-}
-
-// The inner product with the relinearisation key on the P rows: u [items][2]
-// [A][N] = sum_d digP[item][d][j] key[d][poly][L + 1 + j], two adjacent words per
-// thread, 8 items per CTA sharing the key words.
-template <int A>
-__global__ void __launch_bounds__(256, 4) k_relin_ms(u64 *u, const u64 *digP, const u64 *key, int items, int ndig,
-                                                     int logN, int Lp1, int nprimes, const ModQ *mods) {
-    pdl_trigger();
-    pdl_wait();
-    const long N = 1L << logN;
-    const int tx = threadIdx.x & 31, ti = threadIdx.x >> 5;
-    const int x = 2 * (blockIdx.x * 32 + tx), j = blockIdx.y;
-    const long it = (long)blockIdx.z * 8 + ti;
-    if (it >= items) return;
-    const ModQ m = mods[Lp1 + j];
-    const u64 *kp = key + (long)(Lp1 + j) * N + x, *dp = digP + (it * ndig * A + j) * N + x;
-    const long kd = 2L * nprimes * N, kk = (long)nprimes * N;
-    U128 a[2][2] = {};
-    for (int d = 0; d < ndig; d++) {
-        const ulonglong2 v = __ldg((const ulonglong2 *)(dp + (long)d * A * N));
-        const ulonglong2 k0 = __ldg((const ulonglong2 *)(kp + d * kd)), k1 = __ldg((const ulonglong2 *)(kp + d * kd + kk));
-        mac128_q(a[0][0], v.x, k0.x, m.q);
-        mac128_q(a[0][1], v.y, k0.y, m.q);
-        mac128_q(a[1][0], v.x, k1.x, m.q);
-        mac128_q(a[1][1], v.y, k1.y, m.q);
-    }
-#pragma unroll
-    for (int c = 0; c < 2; c++)
-        *(ulonglong2 *)(u + ((it * 2 + c) * A + j) * N + x) =
-            make_ulonglong2(redc(a[c][0].lo, a[c][0].hi, m), redc(a[c][1].lo, a[c][1].hi, m));
 }
 
 // ModDown's integers of a run: uP [K][P][2][A][N] (coefficient form) -> YP
@@ -417,10 +380,8 @@ static void run_a(Ctx *c, RelinSum &S, u64 *d2, int K) {
                                                        lc.d_up_inv, lc.d_up_mod, acc);
     c->trace_end(3, e0, 8.0 * N * P * (K * (nq + (double)nd * A) + (acc ? 4.0 : 2.0) * nq));
     ntt_fwd(c, digP.p, (long)K * P * nd * A, c->map_p(), c->stream);
-    c->n_launch++;
     c->trace_begin(0, e0);
-    launch_pdl(k_relin_ms<A>, dim3((unsigned)(N / 64), A, (unsigned)((K * P + 7) / 8)), 256, 0, c->stream, 
-        uP.p, digP.p, c->rlk, K * P, nd, c->logN, c->L + 1, c->nprimes, c->d_mod);
+    launch_relin_ms(c, uP.p, digP.p, K * P, nd, c->stream);
     c->trace_end(0, e0, 8.0 * N * A * (2.0 * nd + (double)K * P * (nd + 2)), (double)K * P * nd * A * N * 2.0);
     ntt_inv(c, uP.p, (long)K * P * 2 * A, c->map_p(), c->stream);
     c->n_launch++;
