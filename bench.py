@@ -455,12 +455,12 @@ def run_ours(args, rank, world, dist):
 
     def mac_roof(t):
         # the second ceiling of MultSum: its digit-key products against the
-        # measured rate of the 96-bit product accumulation
+        # measured rate of its product accumulation
         if not t["count"] or not t.get("ops"):
             return None
         rate = t["ops"] / (t["ms"] / 1e3) / 1e9
         return {"achieved": rate, "peak": mac_peak / 1e9, "unit": "G products/s", "frac": rate / (mac_peak / 1e9),
-                "peak_source": "measured 96-bit product-accumulate microbenchmark on this GPU"}
+                "peak_source": "measured product-accumulate microbenchmark on this GPU"}
 
     def ntt_roof(t, ratio=None):
         if not t["count"]:
@@ -542,7 +542,8 @@ def run_ours(args, rank, world, dist):
 def multsum_picks(log):
     """The MultSum launch plan the tuner kept for each (level, items, rotations):
     the fastest of its timed candidates (log lines "multsum level L B b G g
-    chunk c BI v stream s ms t"; BI above 100 names launch variant BI - 100)."""
+    chunk c BI v stream s ms t": c keys and v items per CTA; BI above 100 would
+    name launch variant BI - 100)."""
     best = {}
     for ln in log.splitlines():
         f = ln.split()
@@ -1396,7 +1397,7 @@ def main():
     ap.add_argument("--ntt-chunk", type=int, default=None,
                     help="ntt: rows per launch pair of the two-pass NTT (default: the tuner's)")
     ap.add_argument("--ms-variant", type=int, default=None,
-                    help="matmul / keyswitch: pin every MultSum launch to one variant (default: the tuner)")
+                    help="matmul / keyswitch: pin every MultSum launch to one split of its warps (default: the tuner)")
     ap.add_argument("--rate", type=float, default=4.0, help="served: arrivals per second")
     ap.add_argument("--duration", type=float, default=120.0, help="served: seconds of arrivals")
     ap.add_argument("--served-dcd", type=int, default=32,

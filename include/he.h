@@ -113,37 +113,21 @@ int he_ctx_destroy(he_ctx *ctx);
 int he_ctx_set_stream(he_ctx *ctx, void *stream);
 
 /* Launch-geometry autotuner (on by default): the first MultSum of each
- * (level, batch size, number of hoisted rotations) times its launch plans --
- * rotations per launch (1, 2, 4 or 8 sharing one read of the digits), items
- * per CTA, cached or streaming digit loads -- on those very launches and keeps
- * the fastest for the context; the first NTT of the context times the NTT
- * passes compiled for 2 and for 3 CTAs per SM on scratch rows.  Plans compute
- * identical words; only speed differs.  on = 0 uses the fixed defaults (8
- * rotations per launch, 8 items per CTA, cached loads; 2 NTT CTAs per SM). */
+ * (level, batch size, number of hoisted rotations) times the splits of a CTA's
+ * warps over items, keys and coefficients on those very launches and keeps the
+ * fastest for the context; the first NTT of the context times the NTT passes
+ * compiled for 2 and for 3 CTAs per SM on scratch rows.  Plans compute
+ * identical words; only speed differs.  on = 0 uses the fixed defaults (the
+ * split that stages the fewest rows per CTA; 2 NTT CTAs per SM). */
 int he_ctx_set_autotune(he_ctx *ctx, int on);
 
-/* Pins every MultSum launch of the context to one launch variant, with up to
- * 8 hoisted rotations per launch and no tuning (-1 returns to the tuner /
- * defaults).  Variants compute identical words; this is for tests and
- * measurement.  0..7: one thread per (item, coefficient, row), digit and key
- * words loaded by the threads (bits 0-1: 8/4/2/1 items per CTA, bit 2:
- * streaming digit loads); 8, 9, 10: persistent CTAs fed by bulk
- * asynchronous global->shared copies of digit and key segments issued by a
- * producer warp, tiles of 64 coefficients x 8 items (8 stages), 128 x 4 (6)
- * and 256 x 2 (4).
- * 16, 20: variants 0 and 4 with an L2 prefetch of the digit and key words
- * two digits ahead; 32, 36: variants 0 and 4 compiled for more resident CTAs
- * per SM (fewer registers), 48 the same with the prefetch of 16; 64, 65:
- * the rotations of a launch split over the CTA's warps, 1 or 2 per thread (a
- * thread's state no longer grows with the number of rotations; where that
- * number does not divide the 8 warps, as 32); 80, 84: two adjacent
- * coefficients per thread with 16-byte digit and key loads (cached /
- * streaming digit loads), more CTAs per SM, for at most two rotations per
- * launch (more: as 32 / 36); 96, 97: as 64, 65 with two coefficients per
- * thread and 16-byte loads.  The fused MultSum of a product's C^k babies
- * (both sources of a giant with their masks) follows: 96 and 97 pin its
- * rotations-split-over-warps form (97 with launches of 8 rotations where 8
- * remain), every other variant its thread-per-word form.  Errors: HE_ERR_ARG for other values. */
+/* Pins every MultSum launch of the context to one launch variant without
+ * tuning (-1 returns to the tuner / defaults).  Variants compute identical
+ * words; this is for tests and measurement.  Accepted: 0..10, 16, 20, 32, 36,
+ * 48, 64, 65, 80, 84, 96 and 97.  Variant v runs split v mod n of the n ways
+ * in which the launch's shape allows a CTA's warps to be split over items,
+ * keys and coefficients, those that stage the fewest rows first.  Errors:
+ * HE_ERR_ARG for other values. */
 int he_ctx_set_multsum_variant(he_ctx *ctx, int variant);
 
 /* Pins the context's NTT passes (N = 2^14 .. 2^16) to one variant, without
@@ -479,9 +463,8 @@ int he_trace_read(he_ctx *ctx, int cls, long long *count, double *total_ms, doub
 int he_trace_ops(he_ctx *ctx, int cls, double *ops);
 
 /* Integer roofline of MultSum: measured rate (products per second) of the
- * 96-bit product accumulation of its 40-bit limbs (eight 32-bit
- * multiply-adds with carries per product) with register operands on the
- * current device, `iters` rounds of 16 products per thread over 8 CTAs of
+ * product accumulation of its 40-bit limbs (a wrapping 64-bit sum and an FP32
+ * estimate of the quotient) with register operands on the current device, `iters` rounds of 16 products per thread over 8 CTAs of
  * 256 threads per SM.  Errors: HE_ERR_ARG, HE_ERR_CUDA. */
 int he_bench_mac(int iters, double *products_per_s);
 

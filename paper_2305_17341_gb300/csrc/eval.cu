@@ -74,7 +74,7 @@ void rot_qp(Ctx *c, const u64 *ct, int B, int level, const u64 *digits, uint32_t
 }
 
 // G hoisted rotations of the same Decompose output, kept in Q_l P; the
-// digits are read once per launch for up to kMultSumMaxKeys keys.
+// digits are read once per launch for the keys of a launch.
 void rot_qp_multi(Ctx *c, const u64 *ct, int B, int level, const u64 *digits, const uint32_t *gs, int G,
                   u64 *const *outs) {
     if (G <= 0) return;

@@ -116,24 +116,6 @@ __device__ __forceinline__ void mac128_q(U128 &acc, u64 a, u64 b, u64 q) {
     if (acc.hi >= q) acc.hi -= q;
 }
 
-// 96-bit accumulation (w2 w1 w0) of products of residues below 2^42: each
-// product is below 2^84, so a sum of up to 2^12 of them stays below 2^96.
-// (w2 w1 w0) += a b from the four 32 x 32 partial products with the carry
-// chain of the 32-bit multiply-add (a1 b1 < 2^20 has no high word).
-__device__ __forceinline__ void mac96(u32 &w0, u32 &w1, u32 &w2, u64 a, u64 b) {
-    const u32 a0 = (u32)a, a1 = (u32)(a >> 32), b0 = (u32)b, b1 = (u32)(b >> 32);
-    asm("mad.lo.cc.u32 %0, %3, %5, %0;\n\t"
-        "madc.hi.cc.u32 %1, %3, %5, %1;\n\t"
-        "addc.u32 %2, %2, 0;\n\t"
-        "mad.lo.cc.u32 %1, %3, %6, %1;\n\t"
-        "madc.hi.u32 %2, %3, %6, %2;\n\t"
-        "mad.lo.cc.u32 %1, %4, %5, %1;\n\t"
-        "madc.hi.u32 %2, %4, %5, %2;\n\t"
-        "mad.lo.u32 %2, %4, %6, %2;"
-        : "+r"(w0), "+r"(w1), "+r"(w2)
-        : "r"(a0), "r"(a1), "r"(b0), "r"(b1));
-}
-
 // -------------------------------------------------- float-quotient product
 // y w mod q for the 40-bit limbs, with the quotient taken as two FP32 digits
 // instead of one 64-bit high product: the high products are what bounds the

@@ -98,18 +98,15 @@ __global__ void __launch_bounds__(256, NS * GK <= 2 ? 3 : 2) k_msum(const __grid
     const u64 *src0 = s_src[w < tot ? w : 0] + 2 * lane, *src1 = s_src[w + 8 < tot ? w + 8 : 0] + 2 * lane;
     const long str0 = s_str[w < tot ? w : 0], str1 = s_str[w + 8 < tot ? w + 8 : 0];
     const u32 ring = bc_smem(ms_ring + w * 64 + 2 * lane), stage = (u32)tot * 512;
-    auto copy = [](u32 dst, const u64 *src) {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-    };
     auto issue = [&](int d) {   // called for d = 0, 1, 2, ... in order
         if (d < g.ndig) {
             const u32 st = ring + (u32)(d & (kMsStages - 1)) * stage;
-            if (w < tot) copy(st, src0);
-            if (w + 8 < tot) copy(st + 8 * 512, src1);
+            if (w < tot) bc_copy16(st, src0);
+            if (w + 8 < tot) bc_copy16(st + 8 * 512, src1);
             src0 += str0, src1 += str1;
-            for (int e = w + 16; e < tot; e += 8) copy(st + (e - w) * 512, s_src[e] + d * s_str[e] + 2 * lane);
+            for (int e = w + 16; e < tot; e += 8) bc_copy16(st + (e - w) * 512, s_src[e] + d * s_str[e] + 2 * lane);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        bc_commit();
     };
 #pragma unroll
     for (int d = 0; d < kMsStages - 1; d++) issue(d);
@@ -140,7 +137,7 @@ __global__ void __launch_bounds__(256, NS * GK <= 2 ? 3 : 2) k_msum(const __grid
             }
             const int d1 = min(g.ndig, d0 + c.lim);
             for (int d = d0; d < d1; d++) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(kMsStages - 2) : "memory");
+                bc_wait_groups<kMsStages - 2>();
                 __syncthreads();   // stage d has landed; stage d - 1's readers are done
                 issue(d + kMsStages - 1);
                 const int so = (d & (kMsStages - 1)) * tot * 64;
@@ -199,7 +196,7 @@ __global__ void __launch_bounds__(256, NS * GK <= 2 ? 3 : 2) k_msum(const __grid
 #pragma unroll
             for (int k = 0; k < 2 * GK; k++) acc[j][k][0] = acc[j][k][1] = WideMac{0, 0, 0, 0};
         for (int d = 0; d < g.ndig; d++) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(kMsStages - 2) : "memory");
+            bc_wait_groups<kMsStages - 2>();
             __syncthreads();
             issue(d + kMsStages - 1);
             const long so = (long)(d & (kMsStages - 1)) * tot * 64;

@@ -302,9 +302,6 @@ struct PassTw {
     }
 };
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(bc_smem(dst)), "l"(src) : "memory");
-}
 
 // The 8 stages of one pass: 4 in registers in layout A, a shared-memory
 // transpose, 4 (3 for M = 128) in layout B, leaving the words in x.
@@ -449,10 +446,10 @@ __device__ __forceinline__ void stage_twiddles(ulonglong2 *dst, const ulonglong2
     typedef PassGeom<LM, ROWS> G_;
     const int n = ROWS ? G_::W / items * G_::M : G_::M;
     const ulonglong2 *src = ROWS ? tab + 256 + (long)blockIdx.x * n : tab;
-    for (int i = threadIdx.x; i < n; i += 256) cp_async16(dst + i, src + i);
-    asm volatile("cp.async.commit_group;" ::: "memory");
+    for (int i = threadIdx.x; i < n; i += 256) bc_copy16(bc_smem(dst + i), src + i);
+    bc_commit();
 }
-__device__ __forceinline__ void staged_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void staged_wait() { bc_wait_groups<0>(); }
 
 template <int LM, int LS, bool ROWS, bool STG, int MINB, bool SUBSC>
 __global__ void __launch_bounds__(256, MINB) k_ntt_fwd_fast(u64 *data, RowMap rm, long nr, int items,
