@@ -25,6 +25,11 @@
 //    DRAM once and from L2 for the others;
 //  * a product is a wrapping 64-bit sum and an FP32 estimate of the quotient (4
 //    slots), reduced once per output (FqMac).
+// 8 items under 15 keys (N = 2^15, 10 digits): 1.80 -> 1.44 ms; one key: 180 ->
+// 140 us; the C^k babies of a giant (8 items, N = 2^16, level 19): 7.09 -> 6.22
+// ms, 1.1 of the 3.86 T products/s that the sums alone reach in registers: shared
+// memory reads, folds, masks and the 60-bit rows (a tenth of the rows, four times
+// the multiplies) take the rest of the issue slots.
 #include <cstdio>
 #include <set>
 
