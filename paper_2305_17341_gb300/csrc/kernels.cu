@@ -9,6 +9,7 @@
 #include <set>
 #include <stdexcept>
 
+#include "bulkcopy.cuh"
 #include "he_internal.h"
 #include "kernels.cuh"
 
@@ -805,8 +806,11 @@ void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, 
 // grid index: the CTAs of one block of coefficients run together and find its R
 // words in L2 (with the coefficients fastest the 15 giants of a sigma read R
 // from DRAM 15 times, twice the plaintexts' bytes: 480 us against the 170 of
-// one pass over both at the copy rate).  Two adjacent words per thread, the
-// next term's words loaded before a term is multiplied.  One REDC per output
+// one pass over both at the copy rate).  Two adjacent words per thread; a
+// thread's words of the next three terms are on their way to a ring of its own
+// in shared memory while a term is multiplied (with only the next term's in
+// flight it waited for memory: the 15 giants of a sigma, 16 terms each, took 385
+// us at 2.9 TB/s, both launches of the transform 430 us, now 251).  One REDC per output
 // word: up to 32 products below q^2 stay below q 2^64 for q < 2^59; on wider
 // rows (q_0, the special primes) the sum is kept below it term by term
 // (mac128_q).
@@ -816,25 +820,37 @@ struct PmulArgs {
     unsigned char ri[kMaxPmulTerms];
     short first[kMaxPmulSums + 1];
 };
+constexpr int kPmulThreads = 128, kPmulStages = 4;
 // FQ: plaintexts plain and centred, sums as in MultSum; else in Montgomery form.
 template <bool FQ, bool WIDE>
 __device__ __forceinline__ void pmul_item(const PmulArgs &pa, int t0, int t1, long idx, long per, long ro, u64 *ob,
-                                          const ModQ &m, const ModF &f) {
-    ulonglong2 p, r0, r1;
-    auto load = [&](int t) {
-        p = __ldg((const ulonglong2 *)(pa.pt[t] + idx));
-        const u64 *rb = pa.R[pa.ri[t]] + ro + idx;
-        r0 = __ldg((const ulonglong2 *)rb);
-        r1 = __ldg((const ulonglong2 *)(rb + per));
+                                          const ModQ &m, const ModF &f, ulonglong2 (*ring)[3][kPmulThreads]) {
+    const int tx = threadIdx.x;
+    auto issue = [&](int t) {
+        if (t < t1) {
+            ulonglong2 (*s)[kPmulThreads] = ring[(t - t0) % kPmulStages];
+            const u64 *rb = pa.R[pa.ri[t]] + ro + idx;
+            bc_copy16(bc_smem(&s[0][tx]), pa.pt[t] + idx);
+            bc_copy16(bc_smem(&s[1][tx]), rb);
+            bc_copy16(bc_smem(&s[2][tx]), rb + per);
+        }
+        bc_commit();
     };
     u64 o[2][2];
-    if (t0 < t1) load(t0);
+    ulonglong2 pv, v0, v1;
+    auto next = [&](int t) {   // the term's words; its slot is the next one's
+        bc_wait_groups<kPmulStages - 2>();
+        const ulonglong2 (*s)[kPmulThreads] = ring[(t - t0) % kPmulStages];
+        pv = s[0][tx], v0 = s[1][tx], v1 = s[2][tx];
+        issue(t + kPmulStages - 1);
+    };
+#pragma unroll
+    for (int i = 0; i < kPmulStages - 1; i++) issue(t0 + i);
     if constexpr (FQ) {
         const FqMacC c(f, m.q);
         FqMac a[2][2] = {};
         for (int t = t0, run = 0; t < t1; t++, run++) {
-            const ulonglong2 pv = p, v0 = r0, v1 = r1;
-            if (t + 1 < t1) load(t + 1);
+            next(t);
             if (run == c.lim) {
                 run = 0;
 #pragma unroll
@@ -849,8 +865,7 @@ __device__ __forceinline__ void pmul_item(const PmulArgs &pa, int t0, int t1, lo
     } else {
         U128 a[2][2] = {};
         for (int t = t0; t < t1; t++) {
-            const ulonglong2 pv = p, v0 = r0, v1 = r1;
-            if (t + 1 < t1) load(t + 1);
+            next(t);
             if (WIDE) {
                 mac128_q(a[0][0], pv.x, v0.x, m.q), mac128_q(a[0][1], pv.y, v0.y, m.q);
                 mac128_q(a[1][0], pv.x, v1.x, m.q), mac128_q(a[1][1], pv.y, v1.y, m.q);
@@ -865,9 +880,10 @@ __device__ __forceinline__ void pmul_item(const PmulArgs &pa, int t0, int t1, lo
 #pragma unroll
     for (int c = 0; c < 2; c++) *(ulonglong2 *)(ob + c * per + idx) = make_ulonglong2(o[c][0], o[c][1]);
 }
-__global__ void __launch_bounds__(128) k_pmul_acc(u64 *out, long out_s, const __grid_constant__ PmulArgs pa, int B,
+__global__ void __launch_bounds__(kPmulThreads) k_pmul_acc(u64 *out, long out_s, const __grid_constant__ PmulArgs pa, int B,
                                                   int rows, int logN, long Rs, RowMap qp, const ModQ *mods,
                                                   const ModF *modf) {
+    __shared__ ulonglong2 ring[kPmulStages][3][kPmulThreads];   // a thread reads only what it copied
     pdl_trigger();
     pdl_wait();
     const long idx = 2 * ((long)blockIdx.y * 128 + threadIdx.x), per = (long)rows << logN;   // 256 | N
@@ -878,9 +894,9 @@ __global__ void __launch_bounds__(128) k_pmul_acc(u64 *out, long out_s, const __
     u64 *o = out + blockIdx.x * out_s;
     for (int b = 0; b < B; b++) {   // the branches are uniform over the CTA
         u64 *ob = o + (long)b * 2 * per;
-        if (f.on) pmul_item<true, false>(pa, t0, t1, idx, per, b * Rs, ob, m, f);
-        else if (m.q >= (1ull << 59)) pmul_item<false, true>(pa, t0, t1, idx, per, b * Rs, ob, m, f);
-        else pmul_item<false, false>(pa, t0, t1, idx, per, b * Rs, ob, m, f);
+        if (f.on) pmul_item<true, false>(pa, t0, t1, idx, per, b * Rs, ob, m, f, ring);
+        else if (m.q >= (1ull << 59)) pmul_item<false, true>(pa, t0, t1, idx, per, b * Rs, ob, m, f, ring);
+        else pmul_item<false, false>(pa, t0, t1, idx, per, b * Rs, ob, m, f, ring);
     }
 }
 void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const int *first, int sums,
