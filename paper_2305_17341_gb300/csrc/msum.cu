@@ -285,13 +285,20 @@ struct MsumCfg {
 static std::vector<MsumCfg> msum_cfgs(int B, int G, bool ck) {
     std::vector<MsumCfg> v;
     const int ns = ck || B >= 2 ? 2 : 1, per = ck ? 1 : ns;
-    const int gk = G < 2 ? 1 : ns == 2 || G < 4 ? 2 : 4;
-    const int ni = (B + per - 1) / per, nk = (G + gk - 1) / gk;
-    for (int wi = 1; wi <= 8 && wi < 2 * ni; wi *= 2)
-        for (int kw = 1; kw * wi <= 8 && kw < 2 * nk; kw *= 2) {
-            const MsumCfg c{ns, gk, wi, kw, 8 / (wi * kw)};
-            if (c.rows() <= kMsRows) v.push_back(c);
-        }
+    const int ni = (B + per - 1) / per;
+    auto splits = [&](int gk) {
+        const int nk = (G + gk - 1) / gk;
+        for (int wi = 1; wi <= 8 && wi < 2 * ni; wi *= 2)
+            for (int kw = 1; kw * wi <= 8 && kw < 2 * nk; kw *= 2) {
+                const MsumCfg c{ns, gk, wi, kw, 8 / (wi * kw)};
+                if (c.rows() <= kMsRows) v.push_back(c);
+            }
+    };
+    // one item leaves registers for four keys a thread, but their rows take the
+    // shared memory of a whole SM: two keys a thread are timed as well (the 15
+    // babies of a sigma at N = 2^16: 187 us with four, 147 with two)
+    splits(G < 2 ? 1 : 2);
+    if (ns == 1 && G >= 4) splits(4);
     // fewest rows first: the most products per word brought in
     std::stable_sort(v.begin(), v.end(), [](const MsumCfg &a, const MsumCfg &b) { return a.rows() < b.rows(); });
     return v;
