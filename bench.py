@@ -35,13 +35,13 @@ N_MAT = 128
 # DRAM bytes per algorithmic byte, from ncu captures of the same kernels
 # (dram__bytes_read.sum + dram__bytes_write.sum of the launch over the bytes
 # the traced class counts): the forward NTT's two passes each read and write
-# the rows once, plus the row pass's twiddle misses (512-row captures of the
-# two passes: 475.80 + 533.30 MB against 536.87 MB); MultSum reads the keys, the digits and c0 once and
-# writes its outputs once (8 items x 4 hoisted rotations at level 20, the
-# step's R^k / Z / T baby launches, compiled for 4 CTAs per SM: 2968.30 MB
-# against 2982.15 MB).  Traffic grows with the rows / items of a launch, so
-# per launch it is this ratio times the launch's algorithmic bytes.
-TRAFFIC_RATIO = {"ntt_fwd": (475.80 + 533.30) / 536.87, "multsum": 2968.30 / 2982.15}
+# the rows once, plus the row pass's twiddles (2024-row captures of the two
+# passes: 2072.59 + 2280.30 MB against 2122.32 MB); MultSum brings the keys, the
+# digits and c0 from DRAM once and writes its outputs once (8 items x 15 hoisted
+# rotations, N = 2^15, level 19: 3579.82 MB against 3617.59 MB).  Traffic grows
+# with the rows / items of a launch, so per launch it is this ratio times the
+# launch's algorithmic bytes.
+TRAFFIC_RATIO = {"ntt_fwd": (2072.59 + 2280.30) / 2122.32, "multsum": 3579.82 / 3617.59}
 # baby-step count n1 used for each matrix dimension
 N1_FOR = {16: 4, 32: 8, 64: 8, 128: 16}
 LEVEL = 20
@@ -471,7 +471,7 @@ def run_ours(args, rank, world, dist):
         ach = bfly / avg_s / 1e9
         peak = bfly_peak / 1e9
         return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "Gbutterfly/s", "frac": ach / peak,
-                "peak_source": "measured lazy-Shoup butterfly microbenchmark on this GPU",
+                "peak_source": "measured butterfly microbenchmark on this GPU",
                 "traffic": ratio * t["bytes"] / t["count"] if ratio else None,
                 "launches": t["count"], "avg_us": avg_s * 1e6,
                 "hbm_gbs": t["bytes"] / t["count"] / avg_s / 1e9}
@@ -1284,7 +1284,7 @@ def run_ntt(args):
                      "hbm_frac_of_measured": t["bytes"] / args.steps / avg / 1e9 / hbm}
     print(json.dumps({"metric": "NTT butterflies/s (N=2^16, %d rows)" % R, "value": out["forward"]["gbfly_s"],
                       "unit": "Gbutterfly/s", "higher_is_better": True, "n_gpus": 1, "steps": args.steps,
-                      "peak_gbfly_s": peak, "peak_source": "measured lazy-Shoup butterfly microbenchmark",
+                      "peak_gbfly_s": peak, "peak_source": "measured butterfly microbenchmark",
                       "forward": out["forward"], "inverse": out["inverse"],
                       "config": {"workload": "%d rows x 2^16 words, primes of q 60+20x40 and p 2x60 cycled"
                                              % R, "ntt_variant": args.ntt_variant, "ntt_chunk": args.ntt_chunk},

@@ -116,7 +116,7 @@ int he_ctx_set_stream(he_ctx *ctx, void *stream);
  * (level, batch size, number of hoisted rotations) times the splits of a CTA's
  * warps over items, keys and coefficients on those very launches and keeps the
  * fastest for the context; the first NTT of the context times the NTT passes
- * compiled for 2 and for 3 CTAs per SM on scratch rows.  Plans compute
+ * compiled for 2, 3 and 4 CTAs per SM on scratch rows.  Plans compute
  * identical words; only speed differs.  on = 0 uses the fixed defaults (the
  * split that stages the fewest rows per CTA; 2 NTT CTAs per SM). */
 int he_ctx_set_autotune(he_ctx *ctx, int on);
@@ -450,7 +450,7 @@ int he_counters(he_ctx *ctx, long long *ms, long long *dp, long long *md, long l
 int he_trace_enable(he_ctx *ctx, int on);
 
 /* Integer roofline of the NTT: measured rate (butterflies per second) of the
- * lazy Shoup butterfly with register operands on the current device, `iters`
+ * float-quotient butterfly with register operands on the current device, `iters`
  * rounds of 16 butterflies per thread over 8 CTAs of 256 threads per SM. */
 int he_bench_butterfly(int iters, double *bfly_per_s);
 int he_trace_read(he_ctx *ctx, int cls, long long *count, double *total_ms, double *bytes, int reset);
