@@ -469,6 +469,8 @@ void launch_multsum_ck(Ctx *c, u64 *const *outs, const u64 *dig1, const u64 *dig
 // positions inside aligned 32-word blocks.  digits: [G][B][ndig][rows][N]; c0:
 // [G][B] ciphertexts at stride c0s; in (may be null, or equal out), out: [B][2]
 // [rows][N].
+// Only the keys are loaded through the read-only path: the digits are written by
+// the kernel before, which may still run when this grid starts.
 struct GiantArgs {
     const u64 *key[kMaxGiants];
     u32 g[kMaxGiants];
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(256, 4) k_multsum_giants(const __grid_constant
             giant(g, dp, kp);
 #pragma unroll 4
             for (int d = 0; d < ndig; d++) {
-                const u64 v = __ldg(dp + d * ds), k0 = __ldg(kp + d * kd), k1 = __ldg(kp + d * kd + kk);
+                const u64 v = dp[d * ds], k0 = __ldg(kp + d * kd), k1 = __ldg(kp + d * kd + kk);
                 if (run == c.lim) run = 0, a0.fold(c, f), a1.fold(c, f);
                 run++;
                 const float vf = FqMac::part(v);
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(256, 4) k_multsum_giants(const __grid_constant
             WideMac a0 = {0, 0, 0, 0}, a1 = {0, 0, 0, 0};
 #pragma unroll 4
             for (int d = 0; d < ndig; d++) {
-                const u64 v = __ldg(dp + d * ds);
+                const u64 v = dp[d * ds];
                 a0.add(v, __ldg(kp + d * kd));
                 a1.add(v, __ldg(kp + d * kd + kk));
             }
@@ -561,7 +563,8 @@ void launch_multsum_giants(Ctx *c, u64 *out, const u64 *in, const u64 *digits, c
 
 // The relinearisation's inner product on the P rows of a run's terms: u [items][2]
 // [A][N] = sum_d digP[item][d][j] key[d][poly][L + 1 + j], A = alpha; two adjacent
-// words per thread, 8 items per CTA sharing the key words.
+// words per thread, 8 items per CTA sharing the key words (the only ones loaded
+// through the read-only path, as in k_multsum_giants).
 __global__ void __launch_bounds__(256, 4) k_relin_ms(u64 *u, const u64 *digP, const u64 *key, int items, int A, int ndig,
                                                      int logN, int Lp1, int nprimes, const ModQ *mods, const ModF *modf) {
     pdl_trigger();
@@ -580,7 +583,7 @@ __global__ void __launch_bounds__(256, 4) k_relin_ms(u64 *u, const u64 *digP, co
         const FqMacC c(f, m.q);
         FqMac a[2][2] = {};
         for (int d = 0, run = 0; d < ndig; d++, run++) {
-            const ulonglong2 v = __ldg((const ulonglong2 *)(dp + (long)d * A * N));
+            const ulonglong2 v = *(const ulonglong2 *)(dp + (long)d * A * N);
             if (run == c.lim) {
                 run = 0;
 #pragma unroll
@@ -598,7 +601,7 @@ __global__ void __launch_bounds__(256, 4) k_relin_ms(u64 *u, const u64 *digP, co
     } else {
         WideMac a[2][2] = {};
         for (int d = 0; d < ndig; d++) {
-            const ulonglong2 v = __ldg((const ulonglong2 *)(dp + (long)d * A * N));
+            const ulonglong2 v = *(const ulonglong2 *)(dp + (long)d * A * N);
 #pragma unroll
             for (int p = 0; p < 2; p++) {
                 const ulonglong2 k = __ldg((const ulonglong2 *)(kp + d * kd + p * kk));
