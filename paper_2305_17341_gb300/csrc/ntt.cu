@@ -463,8 +463,14 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_fwd_fast(u64 *data, RowMap rm
     const int N = 1 << logN;
     pdl_trigger();
     const PassMap<LM, ROWS> pm(rm, nr, items, skip);
-    // uniform over the CTA: a column CTA's row, or the first row of all items
-    if (ROWS ? pm.row >= nr : !pm.on) return;
+    // uniform over the CTA: a column CTA's row, or the first row of all items.
+    // A CTA without work waits all the same: a launch of which every row is
+    // skipped (a sum's digits at a level of one digit) would otherwise end
+    // before the kernels ahead of it, and later kernels wait for this one only.
+    if (ROWS ? pm.row >= nr : !pm.on) {
+        pdl_wait();
+        return;
+    }
     const int t = pm.t, w = pm.w, pidx = pm.pidx;
     const u64 q = mods[pidx].q;
     const ModF f = modf[pidx];
@@ -591,7 +597,10 @@ __global__ void __launch_bounds__(256, MINB) k_ntt_inv_fast(u64 *data, RowMap rm
     const int N = 1 << logN;
     pdl_trigger();
     const PassMap<LM, ROWS> pm(rm, nr, items, RowSkip());
-    if (ROWS && pm.row >= nr) return;   // uniform over the CTA: the first row of all items
+    if (ROWS && pm.row >= nr) {   // uniform over the CTA: the first row of all items
+        pdl_wait();
+        return;
+    }
     const int t = pm.t, w = pm.w, pidx = pm.pidx;
     const u64 q = mods[pidx].q;
     const ModF f = modf[pidx];
