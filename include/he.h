@@ -217,8 +217,9 @@ int he_rot_steps_for_transpose(int n, int n1, int slots, int32_t *out, int *coun
  * group), so the transform needs n1_sub + 2 n/n1 - 2 (Z) or n1_sub + n/n1 - 2
  * (T) matrix rotation keys instead of n1 + 2 n/n1 - 2 or n1 + n/n1 - 2, at
  * the same MultSum count.  n1 is a power of two dividing n, 2 <= n1_sub <=
- * n1 (n1_sub = n1 is the plain transform).  The input is replicated to
- * period n^2 first when it is not; the output is one level lower.
+ * n1 (n1_sub = n1 is the plain transform); the transform takes n1 <= 32, as
+ * every schedule does.  The input is replicated to period n^2 first when it is
+ * not; the output is one level lower.
  * he_rot_steps_for_ksub lists the slot rotation steps (the transform's and
  * the replication's): on entry *count is the capacity of out, on return the
  * number of steps; out may be NULL to ask for the number only.

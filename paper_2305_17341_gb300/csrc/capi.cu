@@ -947,6 +947,7 @@ int he_linear_transform_ksub(he_ctx *ctx, const he_ct *ct, int kind, int n, int 
     Ctx &c = ctx->c;
     if (int rc = check_ct(c, ct)) return rc;
     if (int rc = check_ksub(n, kind, n1, n1_sub, c.S)) return rc;
+    if (n1 > kMaxPmulRots) return fail(HE_ERR_ARG, "baby-step counts are at most 32");
     if (ct->level < 1) return fail(HE_ERR_LEVEL, "not enough levels for the transform");
     GUARD_BEGIN
     he_ct *tmp = clone_ct(c, ct);

@@ -425,12 +425,12 @@ void launch_relin_ms(Ctx *c, u64 *u, const u64 *digP, int items, int ndig, cudaS
 void launch_key_form(Ctx *c, u64 *key, long rows, const RowMap &rm, cudaStream_t st);
 void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, cudaStream_t st);
 // out[y] ([B][2][rows][N] at stride out_s) = sum of the terms first[y] .. first[y+1]
-// of pt (.) R[r], y < sums; at most 32 terms a sum, nR <= 32.
+// of pt (.) R[r], y < sums; throws for more than 32 terms a sum or 32 rotations R.
 struct PmulTerm {
     const u64 *pt;
     int r;
 };
-constexpr int kMaxPmulTerms = 256, kMaxPmulSums = 64;
+constexpr int kMaxPmulTerms = 256, kMaxPmulSums = 64, kMaxPmulRots = 32;
 void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const int *first, int sums,
                       const u64 *const *R, int nR, int B, int level, long Rs, cudaStream_t st);
 constexpr int kMaxGiants = 64;

@@ -816,7 +816,7 @@ void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, 
 // (mac128_q).
 struct PmulArgs {
     const u64 *pt[kMaxPmulTerms];
-    const u64 *R[32];
+    const u64 *R[kMaxPmulRots];
     unsigned char ri[kMaxPmulTerms];
     short first[kMaxPmulSums + 1];
 };
@@ -902,6 +902,10 @@ __global__ void __launch_bounds__(kPmulThreads) k_pmul_acc(u64 *out, long out_s,
 void launch_pmul_sums(Ctx *c, u64 *out, long out_s, const PmulTerm *terms, const int *first, int sums,
                       const u64 *const *R, int nR, int B, int level, long Rs, cudaStream_t st) {
     const int rows = level + 1 + c->alpha;
+    // what PmulArgs holds, and what one reduction per output word takes
+    if (nR > kMaxPmulRots) throw HeError(HE_ERR_ARG, "a plaintext sum takes at most 32 rotations");
+    for (int y = 0; y < sums; y++)
+        if (first[y + 1] - first[y] > kMaxPmulRots) throw HeError(HE_ERR_ARG, "a plaintext sum takes at most 32 terms");
     for (int y0 = 0, y1; y0 < sums; y0 = y1) {
         PmulArgs a;
         for (int j = 0; j < nR; j++) a.R[j] = R[j];
