@@ -513,7 +513,9 @@ int he_mm_plan_destroy(he_mm_plan *plan);
  * Admission: every job is charged an estimate of the device bytes it holds
  * from admission until its results are taken (its batched temporaries, the
  * intermediates of its circuit and its outputs; resident keys are not
- * charged).  A job whose charge alone exceeds hbm_budget_bytes is rejected
+ * charged, nor are groups and runs of many items, which only make a pass
+ * faster: where their scratch does not fit the device, the pass takes one item
+ * at a time).  A job whose charge alone exceeds hbm_budget_bytes is rejected
  * with HE_ERR_ADMISSION.  A job that fits the budget but not what is left of
  * it waits (HE_JOB_WAITING) and is admitted, in submission order, as earlier
  * jobs give their charges back (completion without outputs, or

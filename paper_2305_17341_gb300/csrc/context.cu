@@ -210,11 +210,7 @@ void *DevicePool::get(size_t bytes) {
     void *p = nullptr;
     if (cudaMalloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
-        // give cached blocks back and retry once
-        cudaDeviceSynchronize();
-        for (auto &kv : free_) cudaFree(kv.second), sizes_.erase(kv.second);
-        free_.clear();
-        cached_ = 0;
+        trim_locked();   // and retry once
         if (cudaMalloc(&p, bytes) != cudaSuccess) {
             cudaGetLastError();
             throw std::bad_alloc();
@@ -224,6 +220,29 @@ void *DevicePool::get(size_t bytes) {
     in_use_ += bytes;
     if (in_use_ > peak_) peak_ = in_use_;
     return p;
+}
+
+void DevicePool::trim_locked() {
+    if (free_.empty()) return;
+    cudaDeviceSynchronize();
+    for (auto &kv : free_) cudaFree(kv.second), sizes_.erase(kv.second);
+    free_.clear();
+    cached_ = 0;
+}
+
+void DevicePool::trim() {
+    std::lock_guard<std::mutex> lk(mu_);
+    trim_locked();
+}
+
+void *device_alloc(Ctx *c, size_t bytes) {
+    void *p = nullptr;
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    c->pool.trim();
+    if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
 }
 
 void DevicePool::put(void *p) {
@@ -639,9 +658,9 @@ void create_keys(Ctx *c) {
 static u64 *gen_swk(Ctx *c, const u64 *sprime, uint32_t obj) {
     int N = c->N, np = c->nprimes;
     RowMap all = map_all(c);
-    u64 *key = nullptr;
-    if (cudaMalloc(&key, c->key_words() * 8) != cudaSuccess) throw std::bad_alloc();
     Buf small(&c->pool, N), e(&c->pool, (size_t)np * N), t(&c->pool, N);
+    u64 *key = (u64 *)device_alloc(c, c->key_words() * 8);
+    if (!key) throw std::bad_alloc();
     i64 *sm = (i64 *)small.p;
     std::vector<ShoupPair> hp(c->L + 1);
     for (int d = 0; d < c->dnum; d++) {

@@ -199,12 +199,9 @@ const u64 *get_pt(Ctx *c, int kind, int n, long t, long rot, double value, int k
     auto it = c->ptcache.find(key);
     if (it != c->ptcache.end()) return it->second;
     const int N = c->N, rows = c->qp_rows(level);
-    u64 *pt = nullptr;
-    if (cudaMalloc(&pt, (size_t)rows * N * 8) != cudaSuccess) {
-        cudaGetLastError();
-        throw HeError(HE_ERR_OOM, "plaintext cache allocation failed");
-    }
     Buf zr(&c->pool, c->S), zi(&c->pool, c->S), m(&c->pool, N);
+    u64 *pt = (u64 *)device_alloc(c, (size_t)rows * N * 8);
+    if (!pt) throw HeError(HE_ERR_OOM, "plaintext cache allocation failed");
     if (fac)
         launch_dcd_fill(c, (double *)zr.p, fac->dev, n, t, rot, value, c->stream);
     else
@@ -253,8 +250,8 @@ static long mod_pos(long x, long m) { return ((x % m) + m) % m; }
 // rotates the input by a s; every later group takes the last baby of the
 // previous one, ModDown'd to a ciphertext c and Decomposed, and rotates c by
 // a s, so that baby j = b + s is rho(c; a s) with c = rho(m; a b).
-void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, int n1, int gi0, int gi1,
-              double value, u64 *out, const DcdFactor *fac, int n1_sub) {
+static void lintrans_once(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, int n1, int gi0, int gi1,
+                          double value, u64 *out, const DcdFactor *fac, int n1_sub) {
     const int N = c->N, nq = level + 1, rows = c->qp_rows(level);
     const long n2 = (long)n * n;
     const size_t qpct = (size_t)2 * rows * N;   // one item over Q_l P
@@ -290,13 +287,14 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
     for (int i = gi0; i < gi1; i++)
         if (i) add_giant(i);
     const int ng = (int)giants.size(), nrot = ng - (i0 == 0 ? 1 : 0);
-    const int Gmax = std::min(nrot, (int)std::max<long>(1, std::min<long>(kMaxGiants, (16L << 16) / ((long)B * N))));
+    const bool one = c->scratch == Ctx::kSingle;
+    const int Gmax = std::min(nrot, one ? 1 : (int)std::max<long>(1, std::min<long>(kMaxGiants, (16L << 16) / ((long)B * N))));
     const size_t dgw = (size_t)B * c->ndig(level) * rows * N;
     Buf acc(&c->pool, B * qpct), ctmp(&c->pool, std::max(1, Gmax) * (size_t)B * 2 * nq * N),
         dg2(&c->pool, std::max(1, Gmax) * dgw);
     // the plaintext sums of up to 64 items of N = 2^16 at a time: more sums a launch
     // share more of its reads of R
-    const int Smax = std::max(1, std::min(nrot, (int)std::max<long>(Gmax, (64L << 16) / ((long)B * N))));
+    const int Smax = std::max(1, one ? 1 : std::min(nrot, (int)std::max<long>(Gmax, (64L << 16) / ((long)B * N))));
     Buf S(&c->pool, (size_t)Smax * B * qpct);
     const int head = n1_sub > 1 && n1_sub < n1 ? n1_sub : n1;
     for (int j0 = 1, base = 0; j0 < n1; j0 += head - 1) {
@@ -344,6 +342,11 @@ void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, 
     }
     moddown_rescale(c, acc.p, B, level, out);
     c->n_md += B;
+}
+
+void lintrans(Ctx *c, const u64 *in, int B, int level, int kind, int n, long a, int n1, int gi0, int gi1,
+              double value, u64 *out, const DcdFactor *fac, int n1_sub) {
+    with_scratch(c, [&] { lintrans_once(c, in, B, level, kind, n, a, n1, gi0, gi1, value, out, fac, n1_sub); });
 }
 
 // The ModDown's last store adds into ct in place.
@@ -417,8 +420,8 @@ void zt_stage_public(Ctx *c, const u64 *in, int B, int level, bool is_t, int n, 
 // C^k Z X_j^T and R^k T X_i computed once for every product that uses
 // them; the batch of products is the row segment).  Only the current k's
 // A^(k), B^(k) are held, so the memory grows with nA + nB + P, not with n.
-void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const int *ia, const int *ib, int P,
-                   int level, int n, int n1z, int n1t, u64 *out, bool relin_once, int dcd_z, int dcd_t) {
+static void hmatmul_once(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const int *ia, const int *ib, int P,
+                         int level, int n, int n1z, int n1t, u64 *out, bool relin_once, int dcd_z, int dcd_t) {
     const int depth = hmatmul_depth(n, dcd_z, dcd_t);
     if (level < depth) throw HeError(HE_ERR_LEVEL, "matrix product needs more levels");
     if ((dcd_z && (dcd_z >= n || dcd_z % n1z)) || (dcd_t && (dcd_t >= n || dcd_t % n1t)))
@@ -454,7 +457,10 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
     // kn P items; the bound keeps its temporaries in proportion to the batch's
     // (64 items of N = 2^16 fill the GPU many times over).
     const int nbA = n1z - 1, nbB = n1t - 1;
-    const int kmax = (int)std::max<long>(1, std::min<long>(n, (64L << 16) / ((long)std::max(P, std::max(nA, nB)) * N)));
+    const int kmax =
+        c->scratch == Ctx::kSingle
+            ? 1
+            : (int)std::max<long>(1, std::min<long>(n, (64L << 16) / ((long)std::max(P, std::max(nA, nB)) * N)));
     const bool summed = c->logN >= 14 && c->logN <= 16;   // the register-blocked NTT's row layouts
     Buf SA(&c->pool, (size_t)n1z * nA * qp1), BB(&c->pool, (size_t)n1t * nB * ct1);
     Buf Ak(&c->pool, (size_t)std::min(kmax, n1z) * nA * ct2);
@@ -547,6 +553,13 @@ void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const in
     if (relin_once) relin_into(c, D2.p, P, l2, acc.p);
     else if (summed) relin_sum_finish(c, *sum, D2.p, acc.p);
     rescale(c, acc.p, P, l2, out);
+}
+
+void hmatmul_pairs(Ctx *c, const u64 *A, int nA, const u64 *Bm, int nB, const int *ia, const int *ib, int P,
+                   int level, int n, int n1z, int n1t, u64 *out, bool relin_once, int dcd_z, int dcd_t) {
+    with_scratch(c, [&] {
+        hmatmul_once(c, A, nA, Bm, nB, ia, ib, P, level, n, n1z, n1t, out, relin_once, dcd_z, dcd_t);
+    });
 }
 
 void hmatmul(Ctx *c, const u64 *A, const u64 *Bm, int Bn, int level, int n, int n1z, int n1t, u64 *out,

@@ -6,6 +6,32 @@
 
 namespace he {
 
+// Runs f, a routine whose groups and runs of many items only make it faster
+// (its words do not depend on their size), and where their scratch does not fit
+// the device runs it again with groups and runs of one, which take no more than
+// a loop over the items.  f reads its inputs and writes its output last, so it
+// may be run again; the operation counters are those of one run.
+struct ScratchMode {
+    Ctx *c;
+    const Ctx::Scratch keep;
+    ScratchMode(Ctx *cc, Ctx::Scratch m) : c(cc), keep(cc->scratch) { c->scratch = m; }
+    ~ScratchMode() { c->scratch = keep; }
+};
+template <class F>
+void with_scratch(Ctx *c, F f) {
+    if (c->scratch != Ctx::kAdapt) return f();
+    const long long ms = c->n_ms, dp = c->n_dp, md = c->n_md;
+    try {
+        return f();
+    } catch (const std::bad_alloc &) {
+    } catch (const HeError &e) {
+        if (e.code != HE_ERR_OOM) throw;
+    }
+    c->n_ms = ms, c->n_dp = dp, c->n_md = md;
+    ScratchMode single(c, Ctx::kSingle);
+    f();
+}
+
 uint32_t galois_of_step(const Ctx *c, long step);
 void create_keys(Ctx *c);
 u64 *gen_rotation_key(Ctx *c, uint32_t g);

@@ -162,7 +162,8 @@ int he_mm_plan_create(const he_mm_job *jobs, int n_jobs, he_mm_plan **out) {
         if (std::find(P->ctxs.begin(), P->ctxs.end(), c) == P->ctxs.end()) P->ctxs.push_back(c);
     }
     std::vector<bool> trace;
-    for (Ctx *c : P->ctxs) trace.push_back(c->trace), c->trace = false;
+    std::vector<Ctx::Scratch> scratch;
+    for (Ctx *c : P->ctxs) trace.push_back(c->trace), c->trace = false, scratch.push_back(c->scratch);
     int rc = HE_OK;
     try {
         if (cudaStreamCreateWithFlags(&P->st, cudaStreamNonBlocking) != cudaSuccess ||
@@ -178,11 +179,34 @@ int he_mm_plan_create(const he_mm_job *jobs, int n_jobs, he_mm_plan **out) {
         }
         // 1. recording run, group after group on each context's own stream:
         //    fills every branch pool and the contexts' caches (plaintext
-        //    diagonals, launch tuning)
-        for (Group &g : P->groups) on_branch(g, nullptr, [&] { record_group(P, g); });
-        for (Ctx *c : P->ctxs)
-            if (cudaStreamSynchronize(c->stream) != cudaSuccess || cudaGetLastError() != cudaSuccess)
-                throw HeError(HE_ERR_CUDA, "recording run failed");
+        //    diagonals, launch tuning).  The capture must find the same blocks:
+        //    all groups record with runs of many items or, where their scratch
+        //    does not fit the device, all with runs of one, and so they are captured
+        auto sync = [&] {
+            for (Ctx *c : P->ctxs)
+                if (cudaStreamSynchronize(c->stream) != cudaSuccess || cudaGetLastError() != cudaSuccess)
+                    throw HeError(HE_ERR_CUDA, "recording run failed");
+        };
+        auto record = [&](Ctx::Scratch mode) {
+            for (Ctx *c : P->ctxs) c->scratch = mode;
+            for (Group &g : P->groups) on_branch(g, nullptr, [&] { record_group(P, g); });
+        };
+        bool fits = true;
+        try {
+            record(Ctx::kGroups);
+        } catch (const std::bad_alloc &) {
+            fits = false;
+        } catch (const HeError &e) {
+            if (e.code != HE_ERR_OOM) throw;
+            fits = false;
+        }
+        sync();
+        if (!fits) {
+            for (Group &g : P->groups) g.pool->release_all();
+            for (Ctx *c : P->ctxs) c->pool.trim();
+            record(Ctx::kSingle);
+            sync();
+        }
         for (size_t i = 0; i < P->ctxs.size(); i++) {
             cudaEvent_t e = nullptr;
             if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess)
@@ -229,7 +253,7 @@ int he_mm_plan_create(const he_mm_job *jobs, int n_jobs, he_mm_plan **out) {
         set_error(e.what());
         rc = HE_ERR_ARG;
     }
-    for (size_t i = 0; i < P->ctxs.size(); i++) P->ctxs[i]->trace = trace[i];
+    for (size_t i = 0; i < P->ctxs.size(); i++) P->ctxs[i]->trace = trace[i], P->ctxs[i]->scratch = scratch[i];
     cudaGetLastError();
     if (rc != HE_OK) {
         delete P;

@@ -69,6 +69,7 @@ public:
     void *get(size_t bytes);
     void put(void *p);
     void release_all();
+    void trim();   // gives the cached blocks back to the device
     size_t bytes_in_use() const { return in_use_; }
     size_t bytes_cached() const { return cached_; }
     size_t bytes_peak() const { return peak_; }
@@ -79,6 +80,7 @@ public:
     ~DevicePool() { release_all(); }
 
 private:
+    void trim_locked();
     DevicePool *redirect_ = nullptr;
     // get/put may be called from a serving worker and the caller's thread
     std::mutex mu_;
@@ -212,6 +214,10 @@ struct Ctx {
 
     DevicePool pool;
     std::mutex mu;
+    // Groups and runs of many items in a transform or a product (with_scratch,
+    // eval.h): where their scratch does not fit the device, one item at a time
+    // (kAdapt), or the one or the other from the start.
+    enum Scratch { kAdapt, kGroups, kSingle } scratch = kAdapt;
 
     // Flag that kernels with bounded waits set when a wait runs out: host
     // memory mapped into the device, read by the host after a synchronise.
@@ -290,6 +296,10 @@ struct Ct {
     double scale = 1.0;
     int period = 0;
 };
+
+// cudaMalloc that gives the pool's cached blocks back and tries again before it
+// fails (nullptr)
+void *device_alloc(Ctx *c, size_t bytes);
 
 // error handling
 void set_error(const std::string &msg);

@@ -151,7 +151,11 @@ public:
                 out.push_back(make(lv - 1, (x->scale * y->scale) / (double)c->primes[lv], std::min(x->period, y->period)));
                 o[j - i] = out.back()->d;
             }
-            mult_rescale_many(c, a, al, b, bl, (int)(j - i), lv, o);
+            with_scratch(c, [&] {
+                const int step = c->scratch == Ctx::kSingle ? 1 : (int)(j - i);
+                for (int t = 0; t < (int)(j - i); t += step)
+                    mult_rescale_many(c, a + t, al + t, b + t, bl + t, step, lv, o + t);
+            });
         }
         return out;
     }
@@ -271,15 +275,30 @@ public:
     // of several ciphertexts: those of one level and period (with the level that
     // axis 1's mask takes) as one batch
     std::vector<HC> aggregate_all(const std::vector<const he_ct *> &in, int axis, int n) {
-        const long n2 = (long)n * n;
         const int lv = in[0]->level, per = in[0]->period, B = (int)in.size();
+        if (B == 1) return aggregate_batch(in, axis, n);
         bool same = true;
         for (auto *x : in) same = same && x->level == lv && x->period == per;
-        if (B > 1 && (!same || (axis == 1 && lv < 1))) {
-            std::vector<HC> out;
+        std::vector<HC> out;
+        auto singly = [&] {
             for (auto *x : in) out.push_back(aggregate(x, axis, n));
+        };
+        if (!same || (axis == 1 && lv < 1)) {
+            singly();
             return out;
         }
+        with_scratch(c, [&] {   // nothing in here refreshes
+            out.clear();
+            if (c->scratch == Ctx::kSingle) singly();
+            else out = aggregate_batch(in, axis, n);
+        });
+        return out;
+    }
+
+    // one ciphertext, or several of one level and period
+    std::vector<HC> aggregate_batch(const std::vector<const he_ct *> &in, int axis, int n) {
+        const long n2 = (long)n * n;
+        const int lv = in[0]->level, per = in[0]->period, B = (int)in.size();
         const size_t w = ct_words(c, lv);
         std::vector<HC> out;
         Buf buf;
@@ -640,12 +659,19 @@ public:
             }
             return out;
         }
-        std::vector<HC> pr = mult_all(ps), sums;
-        for (int i = 0; i < k; i++) {
-            HC acc = std::move(pr[i * k]);
-            for (int j = 1; j < k; j++) acc = add_aligned(std::move(acc), std::move(pr[i * k + j]));
-            sums.push_back(std::move(acc));
-        }
+        std::vector<HC> sums;
+        with_scratch(c, [&] {
+            sums.clear();
+            const bool one = c->scratch == Ctx::kSingle;   // a product at a time is held
+            std::vector<HC> pr;
+            if (!one) pr = mult_all(ps);
+            auto product = [&](int t) { return one ? std::move(mult_all({ps[t]})[0]) : std::move(pr[t]); };
+            for (int i = 0; i < k; i++) {
+                HC acc = product(i * k);
+                for (int j = 1; j < k; j++) acc = add_aligned(std::move(acc), product(i * k + j));
+                sums.push_back(std::move(acc));
+            }
+        });
         return aggregate_list(sums, (axis + 1) % 2, n);
     }
 
