@@ -322,7 +322,9 @@ struct HeError : std::runtime_error {
 };
 
 // Launches a kernel that calls pdl_wait so that it may start while the kernel
-// before it in the stream finishes (modarith.cuh).
+// before it in the stream finishes (modarith.cuh).  A launch that fails throws
+// once the stream's earlier work is done: the call ends here, and buffers that
+// belong to its caller must be idle when it does.
 template <class... P, class... A>
 inline void launch_pdl(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};
@@ -332,7 +334,12 @@ inline void launch_pdl(void (*kern)(P...), dim3 grid, unsigned block, size_t sme
     cfg.gridDim = grid, cfg.blockDim = dim3(block), cfg.dynamicSmemBytes = smem, cfg.stream = st;
     cfg.attrs = at, cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
-    if (e != cudaSuccess) throw HeError(HE_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+            cudaStreamSynchronize(st);
+        throw HeError(HE_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
+    }
 }
 
 // host number theory
