@@ -19,8 +19,8 @@ typedef unsigned int u32;
 // was launched for it (the NTT passes are): its CTAs take free SMs, form their
 // indexes and stage their tables, and pdl_wait holds them until every earlier
 // kernel has finished and its writes are visible.  Nothing that an earlier
-// kernel writes is touched before pdl_wait, and every CTA calls it before it
-// ends, one without work too: the kernel after it waits for this grid alone.
+// kernel writes is touched before pdl_wait, and in every launch some CTA calls
+// it, with work or without: the kernel after it waits for this grid alone.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
