@@ -167,17 +167,12 @@ static void relin_into(Ctx *c, const u64 *d2, int B, int level, u64 *out) {
     c->n_md += B;
 }
 
-// Mult (App. A): tensor (d0, d1, d2), then (d0, d1) + KeySwitch(d2, rlk);
-// with accumulate, the product is added to what out holds (the tensor adds
-// (d0, d1), the ModDown's last store adds the key switch).
-void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out, bool accumulate, int b_level) {
+// Mult (App. A): tensor (d0, d1, d2), then (d0, d1) + KeySwitch(d2, rlk).
+void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out) {
     if (!c->rlk) throw HeError(HE_ERR_KEY_MISSING, "relinearisation key missing");
     const int N = c->N, nq = level + 1;
-    const long cs = 2L * nq * N;
-    if (b_level < level) b_level = level;
     Buf d2(&c->pool, (size_t)B * nq * N);
-    launch_tensor_acc(c, out, d2.p, a, b, B, nq, cs, 2L * (b_level + 1) * N, c->map_q(level), c->stream, accumulate,
-                      false, (long)(b_level + 1) * N);
+    launch_tensor(c, out, d2.p, a, b, B, nq, c->map_q(level), c->stream);
     relin_into(c, d2.p, B, level, out);
 }
 
@@ -186,7 +181,7 @@ void add(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out) {
 }
 
 // --------------------------------------------------- plaintext diagonals
-// Cached encodings (NTT, Montgomery) over Q_l P of a diagonal slot vector at
+// Cached encodings (NTT, in the form their kernels take) over Q_l P of a diagonal slot vector at
 // scale q_l.  kind/n/t/rot/value/k as in k_diag_fill.
 const u64 *get_pt(Ctx *c, int kind, int n, long t, long rot, double value, int k, int level,
                   const DcdFactor *fac) {

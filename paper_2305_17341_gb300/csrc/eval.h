@@ -60,9 +60,7 @@ void mult_rescale_many(Ctx *c, const u64 *const *a, const int *a_level, const u6
 // ct [B][2][l+1][N] += Rot(ct; g)
 void rotate_add(Ctx *c, u64 *ct, int B, int level, uint32_t g);
 void drop(Ctx *c, const u64 *in, int B, int level, int to, u64 *out);
-// b may sit at a higher level b_level (its first level + 1 limbs are used in place)
-void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out, bool accumulate = false,
-                int b_level = -1);
+void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out);
 // Sum of relinearised terms (relin.cu): the integers of the runs so far.
 struct RelinSum {
     int P, level, terms = 0;

@@ -204,10 +204,13 @@ struct Ctx {
     // keys (NTT domain): secret key in normal and Montgomery form over all primes
     u64 *d_sk = nullptr, *d_skM = nullptr;  // [nprimes][N]
     u64 *d_pkM = nullptr;                   // [2][L+1][N] Montgomery
-    std::map<uint32_t, u64 *> rtk;          // galois -> [dnum][2][nprimes][N] Montgomery
+    // galois -> [dnum][2][nprimes][N], permuted (msum.cu), in the form of
+    // launch_key_form: plain and centred on limbs with ModF constants, else Montgomery
+    std::map<uint32_t, u64 *> rtk;
     u64 *rlk = nullptr;
 
-    // cached plaintext diagonals (NTT, Montgomery, over Q_l P), keyed by a string id
+    // cached plaintexts (NTT, over Q_l P), keyed by a string id: those that enter
+    // sums in the form of launch_key_form, the PowerMethod's masks in Montgomery form
     std::map<std::string, u64 *> ptcache;
     std::map<std::string, DcdChain> dcd;     // decompositions by (transform, n, n')
     size_t ptcache_bytes = 0;
@@ -218,10 +221,6 @@ struct Ctx {
     // eval.h): where their scratch does not fit the device, one item at a time
     // (kAdapt), or the one or the other from the start.
     enum Scratch { kAdapt, kGroups, kSingle } scratch = kAdapt;
-
-    // Flag that kernels with bounded waits set when a wait runs out: host
-    // memory mapped into the device, read by the host after a synchronise.
-    int *h_err = nullptr, *d_err = nullptr;
 
     // instrumentation
     std::atomic<long long> n_ms{0}, n_dp{0}, n_md{0}, n_launch{0};
@@ -303,9 +302,6 @@ void *device_alloc(Ctx *c, size_t bytes);
 
 // error handling
 void set_error(const std::string &msg);
-// HE_OK, or HE_ERR_TIMEOUT if a kernel's bounded wait ran out since the last
-// check (the flag is cleared).  Call after synchronising the context's stream.
-int device_status(const Ctx *c);
 #define HE_CUDA_CHECK(expr)                                                          \
     do {                                                                             \
         cudaError_t e__ = (expr);                                                    \
@@ -404,12 +400,10 @@ void launch_mulconst_rows(Ctx *c, u64 *out, const u64 *a, const ShoupPair *w, lo
                           const RowMap &rm, cudaStream_t st);
 void launch_automorph(Ctx *c, u64 *out, const u64 *in, long rows, const RowMap &rm, uint32_t g,
                       cudaStream_t st);
-// (d0, d1) -> d01 [B][2][limbs][N], d2 -> [B][limbs][N]; accumulate adds
-// the tensor to what d01 and d2 already hold (acc01 / acc2 select the two
-// outputs separately when given).  b_poly_stride: words from b's first
-// polynomial to its second (0: limbs * N).
-void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, long as, long bs,
-                       const RowMap &rm, cudaStream_t st, bool acc01, bool acc2, long b_poly_stride = 0);
+// (d0, d1) -> d01 [B][2][limbs][N], d2 -> [B][limbs][N] of B pairs of
+// ciphertexts a, b [B][2][limbs][N]
+void launch_tensor(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, const RowMap &rm,
+                   cudaStream_t st);
 // u [B][2][rows][N] over Q_l P += P d on the rows of Q, d [B][2][l+1][N]
 void launch_add_lifted(Ctx *c, u64 *u, const u64 *d, int B, int level, cudaStream_t st);
 // key switching pieces

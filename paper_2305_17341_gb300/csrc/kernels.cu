@@ -330,12 +330,9 @@ void launch_automorph(Ctx *c, u64 *out, const u64 *in, long rows, const RowMap &
 }
 
 // tensor product in the NTT domain: d0 = a0 b0, d1 = a0 b1 + a1 b0, d2 = a1 b1.
-// d01: [B][2][limbs][N] (d0, d1 of each item); d2: [B][limbs][N].  The
-// operands' first `limbs` limbs are used: item strides as, bs; b's second
-// polynomial starts bps words after its first (a higher-level b is read in
-// place, without a level-dropping copy).
-__global__ void k_tensor(u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, int N,
-                         long as, long bs, long bps, RowMap rm, const ModQ *mods, int accumulate) {
+// a, b, d01: [B][2][limbs][N] (d01: d0, d1 of each item); d2: [B][limbs][N].
+__global__ void k_tensor(u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, int N, RowMap rm,
+                         const ModQ *mods) {
     pdl_trigger();
     pdl_wait();
     long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -345,30 +342,23 @@ __global__ void k_tensor(u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, i
     long off = idx - (long)it * per;
     int limb = (int)(off / N);
     const ModQ &m = mods[rm.at(limb)];
-    const u64 *pa = a + it * as, *pb = b + it * bs;
-    u64 a0 = pa[off], a1 = pa[per + off], b0 = pb[off], b1 = pb[bps + off];
+    const u64 *pa = a + it * 2 * per, *pb = b + it * 2 * per;
+    u64 a0 = pa[off], a1 = pa[per + off], b0 = pb[off], b1 = pb[per + off];
     U128 acc = {0, 0};
     mac128(acc, a0, b1);
     mac128(acc, a1, b0);
     u64 t1 = redc(acc.lo, acc.hi, m);
     u64 v0 = mulmod(a0, b0, m), v1 = redc(t1 * m.r2, mulhi64(t1, m.r2), m), v2 = mulmod(a1, b1, m);
     u64 *o = d01 + (long)it * 2 * per + off;
-    u64 *o2 = d2 + (long)it * per + off;
-    if (accumulate & 1) {
-        v0 = addmod(v0, o[0], m.q);
-        v1 = addmod(v1, o[per], m.q);
-    }
-    if (accumulate & 2) v2 = addmod(v2, o2[0], m.q);
     o[0] = v0;
     o[per] = v1;
-    o2[0] = v2;
+    d2[(long)it * per + off] = v2;
 }
-void launch_tensor_acc(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, long as, long bs,
-                       const RowMap &rm, cudaStream_t st, bool acc01, bool acc2, long bps) {
+void launch_tensor(Ctx *c, u64 *d01, u64 *d2, const u64 *a, const u64 *b, int B, int limbs, const RowMap &rm,
+                   cudaStream_t st) {
     long n = (long)B * limbs * c->N;
     c->n_launch++;
-    launch_pdl(k_tensor, dim3(nblk(n, 256)), 256, 0, st, d01, d2, a, b, B, limbs, c->N, as, bs, bps ? bps : (long)limbs * c->N,
-                                           rm, c->d_mod, (acc01 ? 1 : 0) | (acc2 ? 2 : 0));
+    launch_pdl(k_tensor, dim3(nblk(n, 256)), 256, 0, st, d01, d2, a, b, B, limbs, c->N, rm, c->d_mod);
 }
 
 // ------------------------------------------------------------- ModUp

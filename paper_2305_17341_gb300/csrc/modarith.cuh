@@ -74,8 +74,6 @@ __device__ __forceinline__ u64 shoup(u64 a, u64 w, u64 wp, u64 q) {
     return r >= q ? r - q : r;
 }
 
-__device__ __forceinline__ u64 reduce2q(u64 a, u64 q) { return a >= q ? a - q : a; }
-
 // a mod q for any 64-bit a: Shoup's product by 1 lands in [0, 2q), then one
 // conditional subtraction.
 __device__ __forceinline__ u64 reduce_any(u64 a, u64 q, u64 wone) {
