@@ -61,7 +61,9 @@ void mult_rescale_many(Ctx *c, const u64 *const *a, const int *a_level, const u6
 void rotate_add(Ctx *c, u64 *ct, int B, int level, uint32_t g);
 void drop(Ctx *c, const u64 *in, int B, int level, int to, u64 *out);
 void mult_relin(Ctx *c, const u64 *a, const u64 *b, int B, int level, u64 *out);
-// Sum of relinearised terms (relin.cu): the integers of the runs so far.
+// Sum of at most kRelinTerms relinearised terms (relin.cu): the integers of the
+// runs so far.
+constexpr int kRelinTerms = 256;
 struct RelinSum {
     int P, level, terms = 0;
     Buf SY, YP;

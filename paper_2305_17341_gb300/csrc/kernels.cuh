@@ -49,7 +49,7 @@ __device__ __forceinline__ int md_overflow(const u64 (&y)[A], const MdExact &k) 
 // units of 2^22 q is off by less than 1.65 (1.2): half a unit, half a unit of
 // 2^-24 for each conversion, and the same for each addition of a partial sum of
 // up to as many times q / 2^23; then |sum - ha 2^22 q| < 2^62.9 fits a signed
-// word.  Longer sums are folded to |.| < 1.3 q in between.
+// word.  Longer sums are folded to |.| < 1.5 q in between.
 struct FqMacC {
     float c;     // 2^6 / q
     int lim;     // products between folds
@@ -72,7 +72,8 @@ struct FqMac {
             : "+r"(a0), "+r"(a1)
             : "r"((u32)v), "r"((u32)(v >> 32)), "r"((u32)k), "r"((u32)(k >> 32)));
     }
-    // |result| < 1.3 q
+    // |result| < 1.5 q: the second digit is off by half a unit, a quarter each for
+    // the rounding of h and of the product, 0.41 for that of 1/q
     __device__ __forceinline__ void fold(const FqMacC &c, const ModF &m) {
         const int ha = __float2int_rn(s * c.c);
         u64 r = fq_madws(ha, c.Ql, ((u64)a1 << 32) | a0);

@@ -121,18 +121,18 @@ __device__ __forceinline__ void mac128_q(U128 &acc, u64 a, u64 b, u64 q) {
 // butterfly (IMAD.HI and IMAD.WIDE issue at half the rate of IMAD), while
 // the FP32 multiply-adds run on the FMA lanes that integer code leaves idle.
 //
-// w is centred, |w| <= q/2, with wq = w / (q 2^8); y is signed, |y| <= 17.2 q.
+// w is centred, |w| <= q/2, with wq = w / (q 2^8); y is signed, |y| <= 17.5 q.
 //   ha = round((y >> 14) wq)              ~ y w / (q 2^22)
 //   P  = y w - ha (q 2^22)                exact mod 2^64
 //   hb = round((P >> 32) 2^32 / q)
 //   t  = P - hb q
-// For q < 1.5 2^40: |y w / q| <= 8.6 q, so |ha| < 2^21.7 and its error is
-// below 0.5 + 2^21.7 2^-23 = 0.91 (y and wq each carry a half unit of 2^-24),
-// |P| <= 0.91 2^22 q < 2^62.5 fits a signed word; |hb| <= 2^21.9, its error
+// For q < 1.5 2^40: |y w / q| <= 8.75 q, so |ha| < 2^21.72 and its error is
+// below 0.5 + 2^21.72 2^-23 < 0.92 (y and wq each carry a half unit of 2^-24),
+// |P| <= 0.92 2^22 q < 2^62.5 fits a signed word; |hb| <= 2^21.9, its error
 // is below 0.5 + 2^21.9 2^-23 + 2^32/q <= 0.97 (q >= 2^40), and for smaller
 // q, where the first two terms shrink with q and 2^32/q <= 2^-4 (q >= 2^36),
 // below 0.97 too: |t| < q, t signed.  16 butterfly stages from |x| <= q stay
-// below 17 q.  18 instructions per butterfly against 21.6 with the truncated
+// below 16.6 q, a difference u - x of the fused epilogues below 17.5 q.  18 instructions per butterfly against 21.6 with the truncated
 // Shoup quotient, 1406 against 1000 G butterflies/s with register operands.
 // The products are written as a wide product and an add in one statement:
 // the compiler then emits one multiply-add without the moves that a wide
@@ -177,7 +177,9 @@ struct FqPair {
 // Sum of products y_i w_i + e modulo a prime with ModF constants, with one
 // quotient for the sum (its two digits, as in fq_mul): 3 or 4 wide or low
 // multiply-adds per word of y against 14 multiply slots for a Shoup product.
-// At most 4 narrow sources, or 5 wide ones, and e < q.
+// Bound: sum |y_i w_i| + e below 2^42 q (get), in at most ten words.  Four narrow
+// sources (y < 2^41, |w| <= q/2) or five wide ones and e < q stay below it; so do
+// the sums of lin_row (relin.cu), which derives its own case.
 struct FqDot {
     u64 a;
     float s;
@@ -198,8 +200,10 @@ struct FqDot {
         a = fq_madw(y0, w0, a);
         a = ((u64)fq_madl(y0, w1, fq_madl(y1, w0, (u32)(a >> 32))) << 32) | (u32)a;
     }
-    // the residue in [0, q): the sum is below 2^42 q (narrow; wide 2^35 q), so
-    // |ha| <= 2^20 is exact to 0.75, |P| <= 0.75 2^22 q + q and |t| < q
+    // the residue in [0, q): for a sum below 2^42 q, |ha| <= 2^20 is off by less
+    // than 0.78 with 4 words and, below 2^41.2 q, 0.92 with 10: half a unit, 2^-5
+    // for each addition to the estimate, 2^-23 |ha| for the rounding of the words
+    // and factors, 2^-9 a word for the 14 bits cut off.  |P| < 2^62.5, |t| < q
     __device__ __forceinline__ u64 get(u64 q, const ModF &m) const;
 };
 
@@ -210,7 +214,7 @@ __device__ __forceinline__ u64 FqDot::get(u64 q, const ModF &m) const {
     const u64 r = fq_madw(ha, (u32)m.nQ, a);
     return fq_pos(fq_low((u32)r, fq_madl(ha, (u32)(m.nQ >> 32), (u32)(r >> 32)), m), q);
 }
-// any signed |v| <= 17.2 q to |result| <= 0.57 q
+// any signed |v| <= 17.5 q to |result| <= 0.57 q
 __device__ __forceinline__ u64 fq_red(u64 v, const ModF &m) { return fq_low((u32)v, (u32)(v >> 32), m); }
 
 // Montgomery REDC with the prime and -q^-1 mod 2^64 given directly.

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256, NS * GK <= 2 ? 3 : 2) k_msum(const __grid
             for (int k = 0; k < 2 * GK; k++)
 #pragma unroll
                 for (int e = 0; e < 2; e++) {
-                    if constexpr (CK) {   // signed, |.| < 1.3 q: the masks' products reduce
+                    if constexpr (CK) {   // signed, |.| < 1.5 q: the masks' products reduce
                         acc[j][k][e].fold(c, f);
                         o[j][k][e] = ((u64)acc[j][k][e].a1 << 32) | acc[j][k][e].a0;
                     } else {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256, NS * GK <= 2 ? 3 : 2) k_msum(const __grid
                 u64 o0 = o[j][2 * k][e], o1 = o[j][2 * k + 1][e];
                 if constexpr (CK) {
                     const u64 w1 = __ldg(ma.m1[ki] + (long)r * N + x), w2 = __ldg(ma.m2[ki] + (long)r * N + x);
-                    if (f.on) {   // |sums| < 1.3 q, masks plain and centred
+                    if (f.on) {   // |sums| < 1.5 q, masks plain and centred
                         const float c = FqMacC(f, m.q).c;
                         const ulonglong2 v1 = fq_svar(w1, c), v2 = fq_svar(w2, c);
                         o0 = fq_pos(fq_red(fq_mul(o[0][2 * k][e], v1, f) + fq_mul(o0, v2, f), f), m.q);

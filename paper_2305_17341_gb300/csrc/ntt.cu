@@ -275,7 +275,7 @@ __device__ __forceinline__ int ntt_arith(u64 q, const ModF &f) { return f.on ? A
 template <int AR>
 __device__ __forceinline__ u64 subscale_value(const SubScale &ep, int r, u64 u, u64 s, u64 q, u64 wone, const ModF &f) {
     if constexpr (AR == AR_FQ) {
-        return fq_pos(fq_mul(u - s, ep.wf[r], f), q);   // |u - s| <= 17.2 q
+        return fq_pos(fq_mul(u - s, ep.wf[r], f), q);   // |u - s| <= 17.5 q
     } else {
         const ShoupPair wr = ep.w[r];
         return shoup(submod(u, fwd_residue<AR>(s, q, wone, f), q), wr.w, wr.wp, q);

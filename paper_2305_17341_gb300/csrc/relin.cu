@@ -17,7 +17,7 @@
 // place of ndig (l + 1 + alpha) - (l + 1) + 2 (l + 1) rows of forward NTT and the
 // inner product on every row: 20 instead of 229 rows at level 18 with alpha = 2.
 // The integer sums are kept as two words (sums of low and of high 32 bits,
-// below 2^40 for up to 256 terms).
+// below 2^40 for up to kRelinTerms terms; n <= 181 at the ring degrees of this path).
 #include "eval.h"
 #include "kernels.cuh"
 
@@ -280,7 +280,10 @@ __global__ void __launch_bounds__(256) k_relin_down(const u64 *uP, u64 *YP, int 
 // A linear map of `words` integers y_w (each below 2^40) onto the rows of Q:
 // sum_w y_w W[w][r] mod q_r, plus Kc W[words][r] (0: none).  Used for the Q rows of
 // the summed digits (the low and high words of a digit's y; own rows copied)
-// and for the summed ModDown.
+// and for the summed ModDown.  Of kRelinTerms = 256 terms with A <= 4 sources the
+// low words' sums are below 2^40, the high words' below 2^36 (y < 2^60), the
+// counts below 2^10: against |W| <= q/2 all of them stay below 2^41.2 q, within
+// FqDot's bound although there are up to ten.
 struct LinRows {
     int words;
     const ulonglong2 *Wf;   // [words (+1)][nt]: factors of fq_mul
@@ -425,6 +428,7 @@ RelinSum::RelinSum(Ctx *c, int P_, int level_)
 
 // Terms d2 [K][P][level + 1][N] (NTT domain; overwritten).
 void relin_sum_run(Ctx *c, RelinSum &S, u64 *d2, int K) {
+    if (S.terms + K > kRelinTerms) throw HeError(HE_ERR_ARG, "too many terms in a summed relinearisation");
     switch (c->alpha) {
     case 1: run_a<1>(c, S, d2, K); break;
     case 2: run_a<2>(c, S, d2, K); break;
