@@ -38,10 +38,11 @@ N_MAT = 128
 # the rows once, plus the row pass's twiddles (2024-row captures of the two
 # passes: 2072.59 + 2280.30 MB against 2122.32 MB); MultSum brings the keys, the
 # digits and c0 from DRAM once and writes its outputs once (8 items x 15 hoisted
-# rotations, N = 2^15, level 19: 3579.82 MB against 3617.59 MB).  Traffic grows
+# rotations, level 19: 4.47 + 2.73 GB against 7.235 GB at N = 2^16, 2.23 + 1.35 GB
+# against 3.618 GB at N = 2^15).  Traffic grows
 # with the rows / items of a launch, so per launch it is this ratio times the
 # launch's algorithmic bytes.
-TRAFFIC_RATIO = {"ntt_fwd": (2072.59 + 2280.30) / 2122.32, "multsum": 3579.82 / 3617.59}
+TRAFFIC_RATIO = {"ntt_fwd": (2072.59 + 2280.30) / 2122.32, "multsum": (4.47 + 2.73) / 7.235}
 # baby-step count n1 used for each matrix dimension
 N1_FOR = {16: 4, 32: 8, 64: 8, 128: 16}
 LEVEL = 20

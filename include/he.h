@@ -136,7 +136,8 @@ int he_ctx_set_multsum_variant(he_ctx *ctx, int variant);
  * 2, 3, 5: one 8-stage tile per CTA, compiled for 2, 3 or 4 CTAs per SM
  * (forward and inverse); 4 and 6 are accepted and run as 3 (a persistent
  * form fed by bulk copies and a one-pass form on 8-CTA clusters were slower
- * at every size: 0.965 and 0.983 ms for 1024 rows of N = 2^16 against 0.619).
+ * where they were measured, 1024 rows of N = 2^16: 0.965 and 0.983 ms against
+ * 0.619).
  * Errors: HE_ERR_ARG for other values. */
 int he_ctx_set_ntt_variant(he_ctx *ctx, int variant);
 
@@ -437,8 +438,11 @@ int he_decompose(he_ctx *ctx, const uint64_t *poly_dev, long long n_items, int l
  * and returns when it is done.  Errors: as he_decompose. */
 int he_moddown(he_ctx *ctx, const uint64_t *in_dev, long long n_items, int level, uint64_t *out_dev);
 
-/* Counters of the key-switch phases since the last reset: MultSum, Decompose,
- * ModDown (Table 1 caption), and kernel launches.  Any pointer may be NULL. */
+/* Operations of the paper's schedule since the last reset (Table 1 caption:
+ * MultSum, Decompose, ModDown), and kernel launches.  The three count what the
+ * schedule performs, not the work done for it: where the linear parts of several
+ * relinearisations run once on their sum, each of them still counts.  Any
+ * pointer may be NULL. */
 int he_counters(he_ctx *ctx, long long *ms, long long *dp, long long *md, long long *launches, int reset);
 
 /* Kernel tracing.  While enabled, the library records a CUDA event pair on the

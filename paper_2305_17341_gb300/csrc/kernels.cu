@@ -800,8 +800,8 @@ void launch_permute_key(Ctx *c, u64 *out, const u64 *in, long rows, uint32_t g, 
 // thread's words of the next three terms are on their way to a ring of its own
 // in shared memory while a term is multiplied (with only the next term's in
 // flight it waited for memory: the 15 giants of a sigma, 16 terms each, took 385
-// us at 2.9 TB/s, both launches of the transform 430 us, now 251).  One REDC per output
-// word: up to 32 products below q^2 stay below q 2^64 for q < 2^59; on wider
+// us at 2.9 TB/s, both launches of the transform 430 us, now 251: N = 2^15, level
+// 11, one ciphertext).  One REDC per output word: up to 32 products below q^2 stay below q 2^64 for q < 2^59; on wider
 // rows (q_0, the special primes) the sum is kept below it term by term
 // (mac128_q).
 struct PmulArgs {

@@ -296,7 +296,8 @@ static std::vector<MsumCfg> msum_cfgs(int B, int G, bool ck) {
     };
     // one item leaves registers for four keys a thread, but their rows take the
     // shared memory of a whole SM: two keys a thread are timed as well (the 15
-    // babies of a sigma at N = 2^16: 187 us with four, 147 with two)
+    // babies of a sigma, the best split of each: 188 us with four, 145 with two at
+    // N = 2^15, level 11; 834 and 684 at N = 2^16, level 20)
     splits(G < 2 ? 1 : 2);
     if (ns == 1 && G >= 4) splits(4);
     // fewest rows first: the most products per word brought in

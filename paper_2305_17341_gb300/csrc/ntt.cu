@@ -14,8 +14,8 @@
 // butterfly gives about two thirds (721 -> 619), the twiddles in their order
 // of use and the columns' single crossing of shared memory 619 -> 584, the
 // compile-time column stride and the staged row twiddles the rest.  What bounds
-// it: the FMA-heavy pipe (70 % busy in the column pass) at 23 and 27
-// instructions per butterfly, 18 of them arithmetic.
+// it: the FMA-heavy pipe (70 % busy in the column pass, 63 % in the row pass, 2024
+// rows) at 23 and 28 instructions per butterfly, 18 of them arithmetic.
 // The register-blocked kernels for logN 14..16 go lazier: on the 40-bit
 // limbs (ModF::on) both directions run the signed float-quotient product of
 // modarith.cuh; on other primes the forward skips the per-stage reduction
